@@ -130,7 +130,8 @@ int adi_wave_reset(adi_wave *h, const float *const *m, const float *const *phi,
 int adi_wave_step(adi_wave *h, const adi_source *src, void *stream);
 
 /* Advance by `steps` time steps (Algorithm 1's loop).  The steps of a
- * single grid are replayed from a captured CUDA graph.
+ * single grid are chained launches, or replayed from a captured CUDA graph
+ * (adi_wave_tuning.use_graph).
  *   src      host array of n_shots sources or NULL.
  *   rec_xy   HOST array [n_rec][2] of receiver nodes (ix, iy) of shot 0, or
  *            NULL with n_rec = 0; receivers need n_shots == 1.
@@ -207,6 +208,7 @@ const char *adi_wave_last_error(const adi_wave *h);
  *                   warp-shuffle parallel cyclic reduction (2, 4, 8, 16 or
  *                   32; the CR-to-PCR switch level);
  * use_graph:        1 = replay steps from a captured CUDA graph, -1 = never;
+ *                   0 = graphs where the step is made of separate sweeps;
  * solver:           ADI_SOLVER_TREE (cyclic reduction of the interface
  *                   system across warp lanes by register shuffles, PCR of the
  *                   warp summaries) or ADI_SOLVER_CR_SMEM (cyclic reduction
@@ -253,7 +255,12 @@ const char *adi_wave_last_error(const adi_wave *h);
  *                   split over a cluster of that many CTAs (K = 32, one row
  *                   per cluster; 4: CTAs of 32..128 threads, four per SM);
  *                   ADI_STAGE_BAND: 2, 4 or 8 CTAs per row.
- * Zero fields mean "choose automatically". */
+ * Zero fields mean "choose automatically".  With every field but use_graph
+ * zero, a step whose systems are dominant enough (couplings below 2^-30
+ * across 12 or 16 unknowns: tau up to about h / max c) is one launch that
+ * solves both directions locally instead of the two sweeps; the fields
+ * adi_wave_get_tuning reports then are those the sweeps would have, and
+ * setting any of them selects the sweeps. */
 enum { ADI_STAGE_AUTO = 0, ADI_STAGE_SMEM = 1, ADI_STAGE_L2 = 2, ADI_STAGE_DIRECT = 2,
        ADI_STAGE_TMA = 3, ADI_STAGE_COOP = 4 /* y_stage only */,
        ADI_STAGE_BAND = 5 /* x_stage only */ };
@@ -283,7 +290,7 @@ int adi_wave_set_tuning(adi_wave *h, const adi_wave_tuning *t);
  * sums the recorded durations per kind into ms[kind] and launch counts
  * into launches[kind] for kind < n_kinds, and clears the records.  Kinds:
  * 0 = x sweep (RHS + x solve), 1 = y sweep (+ update), 2 = other (the
- * batched persistent step). */
+ * one-launch step, the batched persistent step). */
 enum { ADI_KERNEL_X = 0, ADI_KERNEL_Y = 1, ADI_KERNEL_OTHER = 2, ADI_KERNEL_KINDS = 3 };
 int adi_wave_profile(adi_wave *h, int32_t enable);
 int adi_wave_profile_read(adi_wave *h, double *ms, int64_t *launches,

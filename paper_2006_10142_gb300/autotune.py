@@ -141,7 +141,10 @@ def tune(nx: int, ny: int, fp64: str = "auto", steps: int = 3, warmup: int = 1,
         sim.run(steps)
         ms, cnt = sim.profile_read()
         sim.profile(False)
-        r = (ms[0] / max(cnt[0], 1), ms[1] / max(cnt[1], 1))
+        if cnt[0] == 0 and cnt[2] > 0:  # one launch does both sweeps: half of it each
+            r = (0.5 * ms[2] / cnt[2], 0.5 * ms[2] / cnt[2])
+        else:
+            r = (ms[0] / max(cnt[0], 1), ms[1] / max(cnt[1], 1))
         if verbose:
             print(json.dumps({"cfg": cfg, "x_ms": r[0], "y_ms": r[1]}))
         return r

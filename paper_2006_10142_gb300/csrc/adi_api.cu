@@ -282,6 +282,29 @@ y_done:
   P.cta_threads_y = cty;
   if (t.persist < -1 || t.persist > 1) { why = "persist must be -1, 0 or 1"; return ADI_EINVAL; }
   P.persist = t.persist > 0 ? 1 : 0;
+  // One pass per step (adi_tile.cu, adi_patch.cu) unless a knob of the
+  // separate sweeps is set: wherever the couplings of both directions decay
+  // below 2^-30 within its halo, the elimination is FP32 and a row fills a
+  // TMA box (32 columns).  us per step, sweeps and one pass: 128^2 7.3 and
+  // 6.1, 1024^2 15.5 and 7.5, 2048^2 36.1 and 25.9, 4096^2 137 and 58,
+  // 16384^2 2063 and 768.  Its steps are launched one by one: consecutive
+  // launches overlap, which those on either side of a graph's end do not
+  // (1024^2: 7.5 against 9.3 from graphs of two steps).
+  P.tile = 0;
+  P.tile_rows = 0;
+  const bool sweeps_set = t.chunk_x || t.chunk_y || t.rows_per_cta || t.cols_per_cta || t.pcr_size || t.solver ||
+                          t.cta_threads || t.cta_threads_y || t.y_stage || t.persist || t.x_stage || t.x_cluster;
+  if (!sweeps_set && !P.fp64x && !P.fp64y && G.nx >= 32) {
+    P.tile = tile_halo(std::max(sxm, sym));
+    if (P.tile) {
+      int dev = 0, nsm = 0;
+      if (cudaGetDevice(&dev) != cudaSuccess ||
+          cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        nsm = 152;
+      P.tile_rows = tile_band_rows(G.nx, G.ny, P.tile, nsm);
+      if (t.use_graph == 0) P.graph = 0;
+    }
+  }
   G.plan = P;
   return ADI_OK;
 }

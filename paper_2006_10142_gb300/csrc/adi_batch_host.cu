@@ -115,7 +115,7 @@ int adi_wave::enqueue_batch_step(cudaStream_t st) {
   if (batch_mode == 2) return enqueue_batch_steps_parallel(1, st);
   if (batch_mode == 1) {
     for (Grid& G : g) {
-      int rc = launch_fwd(G, G.buf[G.cur], G.buf[1 - G.cur], G.w, nullptr, G.gd, st);
+      int rc = launch_fwd(G, G.buf[G.cur], G.buf[1 - G.cur], G.w, nullptr, G.gd, G.cur, false, st);
       if (rc != ADI_OK) return rc;
     }
   } else {
@@ -188,7 +188,7 @@ int adi_wave::enqueue_batch_steps_parallel(int nsteps, cudaStream_t st) {
     cudaStream_t bs = branch[shot_branch[s]];
     int cur = G.cur;
     for (int t = 0; t < nsteps; ++t) {
-      rc = launch_fwd(G, G.buf[cur], G.buf[1 - cur], G.w, nullptr, G.gd, bs);
+      rc = launch_fwd(G, G.buf[cur], G.buf[1 - cur], G.w, nullptr, G.gd, cur, false, bs);
       if (rc != ADI_OK) return rc;
       cur = 1 - cur;
     }

@@ -1231,24 +1231,30 @@ int y_pipe_box_rows(int tcol, int K) {
   return R < 256 ? R : 256;
 }
 
-// Tensor map of a pitched [ny][ld] FP32 field as 2D {ld, ny}, boxes of
-// {box_cols, box_rows} (box_cols = 4, 8, 16 or 32), no swizzle, zero fill outside.
-cudaError_t encode_strip_map(CUtensorMap* out, const float* base, int ld, int ny, int box_cols,
-                             int box_rows) {
+// Tensor map of a pitched [ny][ld] FP32 field as 2D {nx, ny}, boxes of
+// {box_cols, box_rows} (box_cols a multiple of 4), zero fill outside.
+cudaError_t encode_box_map(CUtensorMap* out, const float* base, int nx, int ld, int ny, int box_cols,
+                           int box_rows, bool swizzle) {
   EncodeTiledFn fn = nullptr;
   cudaError_t e = get_encode_fn(&fn);
   if (e != cudaSuccess) return e;
   if (ld % 32 != 0 || box_rows < 1 || box_rows > 256 || ((uintptr_t)base & 15) != 0 ||
-      (box_cols != 4 && box_cols != 8 && box_cols != 16 && box_cols != 32))
+      box_cols < 4 || box_cols > 256 || box_cols % 4 != 0 || (swizzle && box_cols != 32))
     return cudaErrorInvalidValue;
-  const cuuint64_t dims[2] = {(cuuint64_t)ld, (cuuint64_t)ny};
+  const cuuint64_t dims[2] = {(cuuint64_t)nx, (cuuint64_t)ny};
   const cuuint64_t strides[1] = {(cuuint64_t)ld * 4};
   const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
   const cuuint32_t es[2] = {1, 1};
   const CUresult r = fn(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(base), dims,
-                        strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                        strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                        swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
                         CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+cudaError_t encode_strip_map(CUtensorMap* out, const float* base, int ld, int ny, int box_cols,
+                             int box_rows) {
+  return encode_box_map(out, base, ld, ld, ny, box_cols, box_rows, false);
 }
 
 template <int K, int MAXT, int W, bool ADJ>

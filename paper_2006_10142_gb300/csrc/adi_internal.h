@@ -19,6 +19,10 @@ struct GridDev {
   int n_rec;
   const int* rec;       // [n_rec][2] receiver nodes
   float* traces;        // [steps][n_rec]
+  // The one-pass step (adi_tile.cu) has CTAs that read the level while
+  // others finish, so the level alternates between two words: a step reads
+  // kf[par] and leaves its successor in kf[1 - par].
+  long long kf[2];
 };
 
 // Device error word bits.
@@ -114,6 +118,49 @@ cudaError_t launch_y_coop(const YArgs& a, int K, const YCoop& yc, const YMaps& m
 cudaError_t launch_y_coop_adj(const YArgs& a, int K, const YCoop& yc, const CUtensorMap& lam,
                               const CUtensorMap& m, cudaStream_t st);
 cudaError_t configure_y_coop_kernels();
+
+// One whole step in one pass, for systems whose couplings decay fast enough
+// (adi_tile.cu, adi_patch.cu): x and y solves are local, with halos of H
+// unknowns.
+struct TileArgs {
+  int nx, ny, ld;
+  int strips;          // set by the launcher
+  int band_rows;       // rows of a band, a multiple of 16
+  int par;             // which of gd->kf holds the level
+  float cx, cy;        // tau^2 / h1^2, tau^2 / h2^2
+  float scx, scy;      // tau^2 / (2 h1^2), tau^2 / (2 h2^2)
+  float src_scale;     // tau^2 / (h1 h2)
+  float* u_prev;       // in: u^{k-1}; out: u^{k+1}
+  float* w_out;        // copies of w and z for the adjoint, or null (both)
+  float* z_out;
+  int gather;          // sample the receivers of gd
+  GridDev* gd;
+  int* err;
+};
+struct TileMaps {
+  CUtensorMap u, m;  // u^k, m (panel boxes)
+  CUtensorMap p, o;  // u^{k-1}: strip boxes to read, panel boxes to write
+};
+// Halo the local solves need for off-diagonals up to s_max (12 or 16), 0 =
+// the couplings decay too slowly.
+int tile_halo(double s_max);
+int tile_strips(int nx);
+// rows of a band, a multiple of 16, or 0 = by patches
+int tile_band_rows(int nx, int ny, int H, int nsm);
+cudaError_t encode_tile_map(CUtensorMap* out, const float* base, int nx, int ld, int ny, bool strip);
+cudaError_t launch_tile(const TileArgs& a, int H, const TileMaps& mp, cudaStream_t st);
+cudaError_t configure_tile_kernels();
+// The same step patch by patch (adi_patch.cu).
+int patch_rows(int H);
+int patch_strips(int nx);
+cudaError_t encode_patch_map(CUtensorMap* out, const float* base, int nx, int ld, int ny, bool u);
+cudaError_t launch_patch(const TileArgs& a, int H, const CUtensorMap& u, const CUtensorMap& m, cudaStream_t st);
+cudaError_t configure_patch_kernels();
+// 2D tensor map {nx, ny} of a field of row pitch ld with boxes of {box_cols,
+// box_rows}, zero fill outside, optionally in the 128-byte swizzle
+// (box_cols = 32).
+cudaError_t encode_box_map(CUtensorMap* out, const float* base, int nx, int ld, int ny, int box_cols,
+                           int box_rows, bool swizzle);
 
 // The wider problem class and the literal half-level schemes (adi_models.cu).
 // mode 0: Eq. CN1 with m^k = g_k m and a source field; 1: Eqs. fr1 / fr2 over

@@ -1,0 +1,162 @@
+// adi_local.cuh -- building blocks of the local line solves (adi_tile.cu,
+// adi_patch.cu): packed FP32 arithmetic and the division-free elimination.
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "adi_device.cuh"
+#include "adi_internal.h"
+
+namespace adi {
+
+__device__ __forceinline__ float lds(uint32_t a) { return *reinterpret_cast<const float*>(__cvta_shared_to_generic(a)); }
+
+// Two FP32 numbers in one 64-bit register pair: one packed instruction does
+// the work of two, which halves the issue slots of the elimination.
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 pk(float lo, float hi) {
+  f2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float lo2(f2 v) { return __uint_as_float((uint32_t)v); }
+__device__ __forceinline__ float hi2(f2 v) { return __uint_as_float((uint32_t)(v >> 32)); }
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+  f2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
+  f2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 add2(f2 a, f2 b) {
+  f2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 dup2(float v) { return pk(v, v); }
+__device__ __forceinline__ f2 lds2(uint32_t a) { return *reinterpret_cast<const f2*>(__cvta_shared_to_generic(a)); }
+__device__ __forceinline__ ulonglong2 lds4(uint32_t a) {
+  return *reinterpret_cast<const ulonglong2*>(__cvta_shared_to_generic(a));
+}
+
+// Elimination of -s x_{k-1} + (1 + 2s) x_k - s x_{k+1} = d without a
+// reciprocal in its chain.  With gamma_k = a_k / p_k and delta_k = N_k / p_k,
+//     a_k = s_k p_{k-1},  p_k = p_{k-1} + s_k (2 p_{k-1} - a_{k-1}),
+//     N_k = s_k N_{k-1} + d_k p_{k-1}
+// (every term of p is positive, so nothing cancels): two dependent FMAs per
+// unknown, and the reciprocals of the p_k are independent of one another.  p
+// grows by at most 1 + 2s per unknown, 2^16 over a block at s = 1/2, the
+// largest s the halo of 16 allows; every block starts again from p = 1.
+//
+// The packed instructions take no negated operands, so signs are carried by
+// the data instead, in a fixed pattern of period 4: s enters as (-1)^k s_k,
+// d as sigma_k d_k with sigma = + - - +, and with them a as (-1)^k a_k, N as
+// sigma_k N_k; solve() takes the reciprocal of -p, and then
+//     X_k = -sigma_k x_k  obeys  X_k = G_k X_{k+1} + D_k.
+__device__ __forceinline__ constexpr float sgn_d(int k) { return ((k & 3) == 1 || (k & 3) == 2) ? -1.f : 1.f; }
+struct Elim2 {
+  f2 p, a, N;
+  __device__ __forceinline__ void begin(f2 a0, f2 n0) {
+    p = dup2(1.f);
+    a = a0;
+    N = n0;
+  }
+  template <int KP>  // parity of k
+  __device__ __forceinline__ void add(f2 s, f2 d) {
+    const f2 t = fma2(dup2(KP ? -2.f : 2.f), p, a);  // +-(2 p - a)
+    a = mul2(s, p);
+    N = fma2(s, N, mul2(d, p));
+    p = fma2(s, t, p);
+  }
+  // the last H of a chunk's unknowns
+  template <int H>
+  __device__ __forceinline__ void tail(const f2 (&S)[16], const f2 (&D)[16]) {
+#pragma unroll
+    for (int k = 16 - H; k < 16; ++k) {
+      if (k & 1) add<1>(S[k], D[k]);
+      else add<0>(S[k], D[k]);
+    }
+  }
+  // the chunk: S, D become G, D of the back substitution
+  __device__ __forceinline__ void chunk(f2 (&S)[16], f2 (&D)[16]) {
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      if (k & 1) add<1>(S[k], D[k]);
+      else add<0>(S[k], D[k]);
+      solve(S[k], D[k]);
+    }
+  }
+  __device__ __forceinline__ void solve(f2& G, f2& D) const {
+    const f2 r = pk(rcp_t(-lo2(p)), rcp_t(-hi2(p)));
+    G = mul2(a, r);
+    D = mul2(N, r);
+  }
+};
+
+// u^{k+1} = q + z from X (z = -sigma X)
+__device__ __forceinline__ f2 updated(int i, f2 q, f2 X) {
+  return sgn_d(i) > 0.f ? fma2(dup2(-1.f), X, q) : fma2(dup2(-1.f), q, X);
+}
+
+
+// Programmatic dependent launch: a kernel launched with launch_chained() may
+// start while the kernel before it is finishing; it touches nothing that
+// kernel writes before chain_wait(), which returns once that kernel (and
+// with it everything before it) has completed.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Receiver sampling inside the step: traces[s][r] = u^{k+1}(rec r), s = k -
+// k0, of the receivers in columns [x0, x1), rows [y0, y1).  find() looks up
+// the thread's first receiver early, so that only the sample itself is left
+// for take(), which all threads of the CTA call after a barrier behind the
+// stores of u^{k+1}.
+struct Sampler {
+  int at;  // the node of receiver threadIdx.x, -1 = none of this CTA's
+  static __device__ __forceinline__ int node(const GridDev* gd, int r, int x0, int x1, int y0, int y1) {
+    const int2 p = reinterpret_cast<const int2*>(gd->rec)[r];
+    return p.x >= x0 && p.x < x1 && p.y >= y0 && p.y < y1 ? (p.y - y0) * (x1 - x0) + (p.x - x0) : -1;
+  }
+  __device__ __forceinline__ void find(const GridDev* gd, long long lev, int x0, int x1, int y0, int y1) {
+    const long long s = lev - gd->k0;
+    const bool on = gd->traces != nullptr && s >= 0 && s < gd->steps && (int)threadIdx.x < gd->n_rec;
+    at = on ? node(gd, threadIdx.x, x0, x1, y0, y1) : -1;
+  }
+  __device__ __forceinline__ void take(const GridDev* gd, long long lev, const float* u_new, int ld, int x0, int x1,
+                                       int y0, int y1) const {
+    const int n = gd->n_rec, w = x1 - x0;
+    const long long s = lev - gd->k0;
+    auto put = [&](int r, int v) {
+      gd->traces[s * n + r] = __ldcg(u_new + (size_t)(y0 + v / w) * ld + x0 + v % w);
+    };
+    if (at >= 0) put(threadIdx.x, at);
+    if (n <= (int)blockDim.x || gd->traces == nullptr || s < 0 || s >= gd->steps) return;
+    for (int r = threadIdx.x + blockDim.x; r < n; r += blockDim.x) {
+      const int v = node(gd, r, x0, x1, y0, y1);
+      if (v >= 0) put(r, v);
+    }
+  }
+};
+
+// Launch that may overlap the end of the kernel before it in the stream (see
+// chain_wait()).
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*kern)(P...), int blocks, int threads, size_t smem, cudaStream_t st, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks, 1, 1);
+  cfg.blockDim = dim3(threads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+}  // namespace adi

@@ -133,6 +133,8 @@ extern "C" int adi_wave_step_noalloc(const adi_wave_desc* desc, int32_t ld, doub
   GridDev hg = {};
   hg.k = k;
   hg.k0 = k;
+  hg.kf[0] = k;
+  hg.kf[1] = k;
   hg.steps = 1;
   hg.wavelet = on ? src->wavelet : nullptr;
   hg.n_wavelet = on ? src->n_wavelet : 0;
@@ -141,6 +143,27 @@ extern "C" int adi_wave_step_noalloc(const adi_wave_desc* desc, int32_t ld, doub
   set_record_kernel<<<1, 1, 0, st>>>(hg, slot->gd);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail_msg(ADI_ECUDA, std::string("grid record: ") + cudaGetErrorString(e));
+
+  if (P.tile) {  // the whole step in one launch; w stays on chip
+    const bool patch = P.tile_rows == 0;
+    TileMaps mp;
+    if (patch) {
+      e = encode_patch_map(&mp.u, u_cur, d.nx, ld, d.ny, true);
+      if (e == cudaSuccess) e = encode_patch_map(&mp.m, m, d.nx, ld, d.ny, false);
+    } else {
+      e = encode_tile_map(&mp.u, u_cur, d.nx, ld, d.ny, false);
+      if (e == cudaSuccess) e = encode_tile_map(&mp.m, m, d.nx, ld, d.ny, false);
+      if (e == cudaSuccess) e = encode_tile_map(&mp.o, u_prev, d.nx, ld, d.ny, false);
+      if (e == cudaSuccess) e = encode_tile_map(&mp.p, u_prev, d.nx, ld, d.ny, true);
+    }
+    if (e != cudaSuccess) return fail_msg(ADI_ECUDA, std::string("tensor maps: ") + cudaGetErrorString(e));
+    TileArgs ta = tile_args(G);
+    ta.u_prev = u_prev;
+    ta.gd = slot->gd;
+    e = patch ? launch_patch(ta, P.tile, mp.u, mp.m, st) : launch_tile(ta, P.tile, mp, st);
+    if (e != cudaSuccess) return fail_msg(ADI_ECUDA, std::string("step launch: ") + cudaGetErrorString(e));
+    return ADI_OK;
+  }
 
   XArgs xa;
   xa.nx = d.nx;

@@ -46,8 +46,25 @@ cudaError_t adi::configure_current_device() {
   if (e == cudaSuccess) e = configure_adjoint_kernels();
   if (e == cudaSuccess) e = configure_y_coop_kernels();
   if (e == cudaSuccess) e = configure_model_kernels();
+  if (e == cudaSuccess) e = configure_tile_kernels();
+  if (e == cudaSuccess) e = configure_patch_kernels();
   if (e == cudaSuccess) g_configured[dev] = true;
   return e;
+}
+
+// The grid's and plan's part of the one-pass step's arguments.
+TileArgs adi::tile_args(const Grid& G) {
+  TileArgs a = {};
+  a.nx = G.nx;
+  a.ny = G.ny;
+  a.ld = G.ld;
+  a.band_rows = G.plan.tile_rows;
+  a.cx = (float)(G.dt * G.dt / (G.hx * G.hx));
+  a.cy = (float)(G.dt * G.dt / (G.hy * G.hy));
+  a.scx = (float)(G.dt * G.dt / (2.0 * G.hx * G.hx));
+  a.scy = (float)(G.dt * G.dt / (2.0 * G.hy * G.hy));
+  a.src_scale = (float)(G.dt * G.dt / (G.hx * G.hy));
+  return a;
 }
 
 // Scratch of the y sweep without clusters (y_stage 4): segment summaries for
@@ -85,6 +102,8 @@ int adi_wave::ensure_ycoop(Grid& G) {
 // The grid record goes to the device as a kernel argument: no copy engine
 // and no host buffer that must outlive the call.
 int adi_wave::upload_gd(Grid& G, cudaStream_t st) {
+  G.hgd.kf[0] = G.hgd.k;
+  G.hgd.kf[1] = G.hgd.k;
   CK(launch_put_gd(G.gd, G.hgd, st), "upload grid state");
   launches += 1;
   return ADI_OK;
@@ -308,23 +327,67 @@ int adi_wave::prof_end(cudaStream_t st, cudaEvent_t a, int kind) {
 int adi_wave::enqueue_step(Grid& G, cudaStream_t st, bool gather) {
   float* u_cur = G.buf[G.cur];
   float* u_prev = G.buf[1 - G.cur];
-  int rc = launch_fwd(G, u_cur, u_prev, G.w, nullptr, G.gd, st);
+  int rc = launch_fwd(G, u_cur, u_prev, G.w, nullptr, G.gd, G.cur, gather, st);
   if (rc != ADI_OK) return rc;
-  if (gather) {
-    CK(launch_gather(G.gd, u_prev, G.ld, G.hgd.n_rec, st), "gather launch");
-    launches += 1;
-  }
   G.cur = 1 - G.cur;
   G.k += 1;
   G.from_init = false;
   return ADI_OK;
 }
 
+// The same step as one launch (adi_tile.cu, adi_patch.cu); w and z are
+// written only when z_out is given.
+int adi_wave::launch_fwd_tile(Grid& G, const float* u_cur, float* u_prev, float* w, float* z_out,
+                              GridDev* gd, int par, bool gather, cudaStream_t st) {
+  const bool patch = G.plan.tile_rows == 0;
+  auto encode = [&](CUtensorMap* out, const float* p, bool u) {
+    return patch ? encode_patch_map(out, p, G.nx, G.ld, G.ny, u) : encode_tile_map(out, p, G.nx, G.ld, G.ny, false);
+  };
+  if (G.tt_form != (patch ? 2 : 1)) {
+    for (int q = 0; q < 2; ++q) {
+      CK(encode(&G.tt_buf[q], G.buf[q], true), "step map u");
+      if (!patch) CK(encode_tile_map(&G.tt_strip[q], G.buf[q], G.nx, G.ld, G.ny, true), "step map u");
+    }
+    CK(encode(&G.tt_m, G.m, false), "step map m");
+    G.tt_form = patch ? 2 : 1;
+  }
+  TileMaps mp;
+  mp.m = G.tt_m;
+  if (u_cur == G.buf[0] || u_cur == G.buf[1]) mp.u = G.tt_buf[u_cur == G.buf[1]];
+  else CK(encode(&mp.u, u_cur, true), "step map");
+  if (patch) {
+    // u^{k-1} is read and written without a map
+  } else if (u_prev == G.buf[0] || u_prev == G.buf[1]) {
+    mp.o = G.tt_buf[u_prev == G.buf[1]];
+    mp.p = G.tt_strip[u_prev == G.buf[1]];
+  } else {
+    CK(encode_tile_map(&mp.o, u_prev, G.nx, G.ld, G.ny, false), "step map");
+    CK(encode_tile_map(&mp.p, u_prev, G.nx, G.ld, G.ny, true), "step map");
+  }
+  TileArgs a = tile_args(G);
+  a.par = par;
+  a.u_prev = u_prev;
+  a.w_out = z_out != nullptr ? w : nullptr;
+  a.z_out = z_out;
+  a.gather = gather ? 1 : 0;
+  a.gd = gd;
+  a.err = d_err;
+  cudaEvent_t ev = nullptr;
+  if (profile && prof_begin(st, &ev) != ADI_OK) return ADI_ECUDA;
+  CK(patch ? launch_patch(a, G.plan.tile, mp.u, mp.m, st) : launch_tile(a, G.plan.tile, mp, st), "step launch");
+  if (profile && prof_end(st, ev, ADI_KERNEL_OTHER) != ADI_OK) return ADI_ECUDA;
+  launches += 1;
+  return ADI_OK;
+}
+
 // One forward step on explicit buffers: x sweep into w, y sweep + update
-// writing u^{k+1} over u_prev (and z into z_out when given).
+// writing u^{k+1} over u_prev (and z into z_out when given).  par: which
+// level word of gd the one-pass step reads (it leaves the next level in the
+// other one).  gather: sample the receivers of gd.
 int adi_wave::launch_fwd(Grid& G, const float* u_cur, float* u_prev, float* w, float* z_out,
-                         GridDev* gd, cudaStream_t st) {
+                         GridDev* gd, int par, bool gather, cudaStream_t st) {
   const GridPlan& P = G.plan;
+  if (P.tile) return launch_fwd_tile(G, u_cur, u_prev, w, z_out, gd, par, gather, st);
   XArgs xa;
   xa.nx = G.nx;
   xa.ny = G.ny;
@@ -422,6 +485,10 @@ int adi_wave::launch_fwd(Grid& G, const float* u_cur, float* u_prev, float* w, f
   }
   if (profile && prof_end(st, a, ADI_KERNEL_Y) != ADI_OK) return ADI_ECUDA;
   launches += 2;
+  if (gather) {
+    CK(launch_gather(gd, u_prev, G.ld, G.hgd.n_rec, st), "gather launch");
+    launches += 1;
+  }
   return ADI_OK;
 }
 
@@ -461,7 +528,7 @@ int adi_wave::launch_pair_graph(Grid& G, cudaStream_t st, bool gather) {
     }
   }
   CK(cudaGraphLaunch(ex, st), "graph launch");
-  launches += gather ? 6 : 4;
+  launches += G.plan.tile ? 2 : gather ? 6 : 4;
   G.k += 2;
   return ADI_OK;
 }
@@ -773,6 +840,7 @@ int adi_wave::enqueue_model_step(Grid& G, cudaStream_t st, bool gather) {
     G.w = B;
     G.tm_lines = 0;  // cached tensor maps name the buffers by role
     G.ts_rows = 0;
+    G.tt_form = 0;
   }
   G.k += 1;
   G.from_init = false;

@@ -30,13 +30,16 @@ struct GridPlan {
   int persist = 0;   // 1: persistent sweeps with L2 prefetch of the next tile
   int x_stage = 2;   // 1: rows staged through shared memory, 2: direct, 3: TMA pipeline
   int xc = 1;        // TMA pipeline: CTAs per row (1 or 2)
+  int tile = 0;      // halo of the one-pass step (adi_tile.cu), 0 = separate sweeps
+  int tile_rows = 0; // rows per band of the one-pass step, 0 = by patches (adi_patch.cu)
 
   bool operator==(const GridPlan& o) const {
     return kx == o.kx && log2tsys == o.log2tsys && spc == o.spc && pcr == o.pcr &&
            fp64x == o.fp64x && ky == o.ky && log2W == o.log2W && log2tcol == o.log2tcol &&
            C == o.C && fp64y == o.fp64y && graph == o.graph && tree == o.tree &&
            cta_threads == o.cta_threads && cta_threads_y == o.cta_threads_y &&
-           y_stage == o.y_stage && persist == o.persist && x_stage == o.x_stage && xc == o.xc;
+           y_stage == o.y_stage && persist == o.persist && x_stage == o.x_stage && xc == o.xc &&
+           tile == o.tile && tile_rows == o.tile_rows;
   }
 };
 
@@ -58,6 +61,8 @@ struct Grid {
   int tm_lines = 0;                 // box height they were encoded with, 0 = none
   CUtensorMap ts_buf[2], ts_m, ts_w;  // strip maps (pipelined y sweep)
   int ts_rows = 0;                  // 64 * box rows + box columns they were encoded with, 0 = none
+  CUtensorMap tt_buf[2], tt_strip[2], tt_m;  // maps of the one-pass step
+  int tt_form = 0;                  // form they were encoded for: 1 = bands, 2 = patches, 0 = none
   YCoop yc = {0, 0, 0, nullptr, nullptr};  // scratch of the y sweep without clusters (y_stage 4)
 };
 
@@ -178,7 +183,9 @@ struct adi_wave {
   // internals
   int enqueue_step(adi::Grid& G, cudaStream_t st, bool gather);
   int launch_fwd(adi::Grid& G, const float* u_cur, float* u_prev, float* w, float* z_out,
-                 adi::GridDev* gd, cudaStream_t st);
+                 adi::GridDev* gd, int par, bool gather, cudaStream_t st);
+  int launch_fwd_tile(adi::Grid& G, const float* u_cur, float* u_prev, float* w, float* z_out,
+                      adi::GridDev* gd, int par, bool gather, cudaStream_t st);
   int ensure_adj_work(adi::Grid& G, int E, int n_rec);
   void free_adj_work();
   int launch_pair_graph(adi::Grid& G, cudaStream_t st, bool gather);
@@ -196,4 +203,5 @@ int fail(adi_wave* h, int code, const std::string& msg);
 int cuda_fail(adi_wave* h, cudaError_t e, const char* what);
 int plan_grid(Grid& G, const adi_wave_tuning& t, std::string& why);
 void set_thread_error(const std::string& msg);
+TileArgs tile_args(const Grid& G);
 }  // namespace adi

@@ -66,6 +66,9 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
+// The same for every state space.
+__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async;" ::: "memory"); }
+
 // Tiled 3D tensor load into this CTA's shared memory at `dst` (1024-byte
 // aligned for the 128-byte swizzle); completes `box bytes` on `bar`.
 // Coordinates are in elements, innermost first; c0 * 4 bytes must be a
@@ -114,6 +117,14 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap* tm, int c0, int 
       "cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(
           reinterpret_cast<uint64_t>(tm)),
       "r"(c0), "r"(c1), "r"(c2), "r"(src)
+      : "memory");
+}
+// The same for a 2D box.
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* tm, int c0, int c1, uint32_t src) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
+          reinterpret_cast<uint64_t>(tm)),
+      "r"(c0), "r"(c1), "r"(src)
       : "memory");
 }
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
