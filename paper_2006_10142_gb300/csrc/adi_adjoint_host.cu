@@ -162,12 +162,11 @@ int adi_wave::adjoint(const float* resid, double* grad_m, float* grad_wavelet, i
     CKA(cudaMemcpyAsync(aw.B, rr.ckpt[c] + ffl, fbytes, cudaMemcpyDeviceToDevice, st), "restore");
     hg.k = rr.k0 + s0;
     hg.k0 = hg.k;
-    hg.kf[0] = hg.kf[1] = hg.k;
     CKA(cudaMemcpyAsync(aw.gd, &hg, sizeof(GridDev), cudaMemcpyHostToDevice, st), "adjoint state");
     float* cur = aw.B;
     float* prev = aw.A;
     for (int i = 0; i < len; ++i) {
-      rc = launch_fwd(G, cur, prev, aw.wseg + ffl * i, aw.zseg + ffl * i, aw.gd, i & 1, false, st);
+      rc = launch_fwd(G, cur, prev, aw.wseg + ffl * i, aw.zseg + ffl * i, aw.gd, false, st);
       if (rc != ADI_OK) return rc;
       std::swap(cur, prev);
     }

@@ -302,7 +302,6 @@ y_done:
           cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         nsm = 152;
       P.tile_rows = tile_band_rows(G.nx, G.ny, P.tile, nsm);
-      if (t.use_graph == 0) P.graph = 0;
     }
   }
   G.plan = P;
@@ -403,15 +402,19 @@ extern "C" int adi_wave_get_state(const adi_wave* h, int32_t shot, float* u_prev
   if (!h || shot < 0 || shot >= (int)h->g.size()) return ADI_EINVAL;
   const Grid& G = h->g[shot];
   cudaStream_t st = (cudaStream_t)stream;
-  const size_t wb = sizeof(float) * (size_t)G.nx;
-  if (u_prev) {
-    cudaError_t e = cudaMemcpy2DAsync(u_prev, wb, G.buf[1 - G.cur], sizeof(float) * G.ld, wb, G.ny,
-                                      cudaMemcpyDeviceToDevice, st);
-    if (e != cudaSuccess) return cuda_fail(const_cast<adi_wave*>(h), e, "get_state");
-  }
-  if (u_cur) {
-    cudaError_t e = cudaMemcpy2DAsync(u_cur, wb, G.buf[G.cur], sizeof(float) * G.ld, wb, G.ny,
-                                      cudaMemcpyDeviceToDevice, st);
+  if (u_prev || u_cur) {
+    CopyArgs c = {};
+    c.nx = G.nx;
+    c.ny = G.ny;
+    c.spitch = G.ld;
+    c.dpitch = G.nx;
+    c.src0 = u_prev ? G.buf[1 - G.cur] : G.buf[G.cur];
+    c.dst0 = u_prev ? u_prev : u_cur;
+    if (u_prev && u_cur) {
+      c.src1 = G.buf[G.cur];
+      c.dst1 = u_cur;
+    }
+    const cudaError_t e = launch_copy_fields(c, GridDev{}, st);
     if (e != cudaSuccess) return cuda_fail(const_cast<adi_wave*>(h), e, "get_state");
   }
   if (k) *k = G.k;

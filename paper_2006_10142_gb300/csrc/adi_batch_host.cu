@@ -110,12 +110,18 @@ int adi_wave::setup_batch(cudaStream_t st) {
   return ADI_OK;
 }
 
+// One step of one shot by the single-grid kernels, buf[cur] = u^k.
+int adi_wave::launch_batch_fwd(Grid& G, int cur, cudaStream_t st) {
+  return G.plan.tile ? launch_fwd_tile(G, G.buf[cur], G.buf[1 - cur], G.gd, cur, false, st)
+                     : launch_fwd(G, G.buf[cur], G.buf[1 - cur], G.w, nullptr, G.gd, false, st);
+}
+
 int adi_wave::enqueue_batch_step(cudaStream_t st) {
   const int n = (int)g.size();
   if (batch_mode == 2) return enqueue_batch_steps_parallel(1, st);
   if (batch_mode == 1) {
     for (Grid& G : g) {
-      int rc = launch_fwd(G, G.buf[G.cur], G.buf[1 - G.cur], G.w, nullptr, G.gd, G.cur, false, st);
+      int rc = launch_batch_fwd(G, G.cur, st);
       if (rc != ADI_OK) return rc;
     }
   } else {
@@ -162,7 +168,137 @@ int adi_wave::ensure_branches() {
   return ADI_OK;
 }
 
-int adi_wave::enqueue_batch_steps_parallel(int nsteps, cudaStream_t st) {
+// Tables of the one-launch step: built on the first run in batch mode 2 and
+// again when a reset has changed a plan.  All such shots take the same form
+// and the largest halo any of them needs.  Bands and patches by the times of
+// tile_band_rows(): bands of the length that gives the shortest step, the
+// longest CTAs first.
+int adi_wave::ensure_batch_tiles() {
+  std::vector<GridPlan> plans;
+  for (const Grid& G : g) plans.push_back(G.plan);
+  if (plans == bt_plans) return ADI_OK;
+  bt_n = 0;
+  std::vector<int> shots;
+  bt_h = 12;
+  for (size_t s = 0; s < g.size(); ++s)
+    if (g[s].plan.tile) {
+      shots.push_back((int)s);
+      bt_h = std::max(bt_h, g[s].plan.tile);
+    }
+  bt_plans = plans;
+  if (shots.size() < 2) return ADI_OK;
+  int dev = 0, nsm = 0;
+  CKB(cudaGetDevice(&dev), "get device");
+  CKB(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev), "SM count");
+  const double slots = 2.0 * nsm;
+  double patches = 0;
+  int max_blocks = 1;
+  for (int s : shots) {
+    patches += (double)patch_strips(g[s].nx) * ((g[s].ny + patch_rows(bt_h) - 1) / patch_rows(bt_h));
+    max_blocks = std::max(max_blocks, (g[s].ny + 15) / 16);
+  }
+  double best = 1.2 + 6.3 * std::max(1.0, patches / slots);
+  int best_b = 0;
+  for (int b = 4; b <= max_blocks; ++b) {
+    double total = 0;
+    int longest = 0;
+    bool ok = true;
+    for (int s : shots) {
+      const int blocks = (g[s].ny + 15) / 16;
+      const int bands = (blocks + b - 1) / b;
+      const int len = std::min(b, blocks) + (bands == 1 ? 0 : bands == 2 ? 1 : 2);
+      longest = std::max(longest, len);
+      total += (double)tile_strips(g[s].nx) * (blocks + (bands > 1 ? 2.0 * (bands - 1) : 0.0));
+      ok = ok && g[s].nx >= 224;
+    }
+    const double t = 3.5 + 3.05 * std::max((double)longest, total / slots);
+    if (ok && t < best) {
+      best = t;
+      best_b = b;
+    }
+  }
+  bt_patch = best_b == 0;
+  std::vector<BatchTile> tiles;
+  struct Item {
+    int cost;
+    int2 it;
+  };
+  std::vector<Item> items;
+  for (int s : shots) {
+    Grid& G = g[s];
+    BatchTile t = {};
+    for (int q = 0; q < 2; ++q) {
+      if (bt_patch) {
+        CKB(encode_patch_map(&t.u[q], G.buf[q], G.nx, G.ld, G.ny, true), "batch map u");
+      } else {
+        CKB(encode_tile_map(&t.u[q], G.buf[q], G.nx, G.ld, G.ny, false), "batch map u");
+        CKB(encode_tile_map(&t.p[q], G.buf[q], G.nx, G.ld, G.ny, true), "batch map u");
+      }
+      t.buf[q] = G.buf[q];
+    }
+    if (bt_patch) CKB(encode_patch_map(&t.m, G.m, G.nx, G.ld, G.ny, false), "batch map m");
+    else CKB(encode_tile_map(&t.m, G.m, G.nx, G.ld, G.ny, false), "batch map m");
+    t.a = tile_args(G);
+    t.a.gd = G.gd;
+    t.a.err = d_err;
+    t.a.band_rows = bt_patch ? patch_rows(bt_h) : 16 * best_b;
+    t.a.strips = bt_patch ? patch_strips(G.nx) : tile_strips(G.nx);
+    const int bands = (G.ny + t.a.band_rows - 1) / t.a.band_rows;
+    for (int b = 0; b < bands; ++b)
+      for (int c = 0; c < t.a.strips; ++c) {
+        const int rows = std::min(t.a.band_rows, G.ny - b * t.a.band_rows);
+        items.push_back(Item{bt_patch ? 0 : -rows, make_int2((int)tiles.size(), b * t.a.strips + c)});
+      }
+    tiles.push_back(t);
+  }
+  std::stable_sort(items.begin(), items.end(), [](const Item& x, const Item& y) { return x.cost < y.cost; });
+  std::vector<int2> list;
+  for (const Item& i : items) list.push_back(i.it);
+  bt_plans.clear();  // until the tables are in place
+  cudaFree(bt_dev);
+  cudaFree(bt_items);
+  bt_dev = nullptr;
+  bt_items = nullptr;
+  CKB(cudaMalloc(&bt_dev, sizeof(BatchTile) * tiles.size()), "alloc batch tables");
+  CKB(cudaMalloc(&bt_items, sizeof(int2) * list.size()), "alloc batch tables");
+  CKB(cudaMemcpy(bt_dev, tiles.data(), sizeof(BatchTile) * tiles.size(), cudaMemcpyHostToDevice), "batch tables");
+  CKB(cudaMemcpy(bt_items, list.data(), sizeof(int2) * list.size(), cudaMemcpyHostToDevice), "batch tables");
+  bt_n = (int)tiles.size();
+  bt_n_items = (int)list.size();
+  bt_plans = plans;
+  return ADI_OK;
+}
+
+// `steps` steps of every shot: one launch per step for the one-pass shots,
+// then the others' sweeps on parallel branches.
+int adi_wave::run_batch_tiles(int steps, cudaStream_t st) {
+  const int cur0 = g[0].cur;  // the shots advance together: one orientation
+  for (int t = 0; t < steps; ++t) {
+    const int par = cur0 ^ (t & 1);
+    cudaEvent_t ev = nullptr;
+    if (profile && prof_begin(st, &ev) != ADI_OK) return ADI_ECUDA;
+    CKB(bt_patch ? launch_patch_batch(bt_dev, bt_items, bt_n_items, par, bt_h, st)
+                 : launch_tile_batch(bt_dev, bt_items, bt_n_items, par, bt_h, st), "batched step launch");
+    if (profile && prof_end(st, ev, ADI_KERNEL_OTHER) != ADI_OK) return ADI_ECUDA;
+    launches += 1;
+  }
+  if (bt_n < (int)g.size()) {
+    for (int t = 0; t < steps; ++t) {
+      const int rc = enqueue_batch_steps_parallel(1, st, true);
+      if (rc != ADI_OK) return rc;
+    }
+  }
+  for (Grid& G : g) {
+    if (!G.plan.tile) continue;  // advanced above
+    if (steps & 1) G.cur = 1 - G.cur;
+    G.k += steps;
+    G.from_init = false;
+  }
+  return ADI_OK;
+}
+
+// rest: only the shots that the one-launch step leaves.
+int adi_wave::enqueue_batch_steps_parallel(int nsteps, cudaStream_t st, bool rest) {
   int rc = ensure_branches();
   if (rc != ADI_OK) return rc;
   const int n = (int)g.size();
@@ -185,10 +321,11 @@ int adi_wave::enqueue_batch_steps_parallel(int nsteps, cudaStream_t st) {
   for (int b = 0; b < nb; ++b) CKB(cudaStreamWaitEvent(branch[b], fork_ev, 0), "branch wait");
   for (int s : shot_order) {
     Grid& G = g[s];
+    if (rest && G.plan.tile) continue;
     cudaStream_t bs = branch[shot_branch[s]];
     int cur = G.cur;
     for (int t = 0; t < nsteps; ++t) {
-      rc = launch_fwd(G, G.buf[cur], G.buf[1 - cur], G.w, nullptr, G.gd, cur, false, bs);
+      rc = launch_batch_fwd(G, cur, bs);
       if (rc != ADI_OK) return rc;
       cur = 1 - cur;
     }
@@ -198,6 +335,7 @@ int adi_wave::enqueue_batch_steps_parallel(int nsteps, cudaStream_t st) {
     CKB(cudaStreamWaitEvent(st, join_ev[b], 0), "join wait");
   }
   for (Grid& G : g) {
+    if (rest && G.plan.tile) continue;
     if (nsteps & 1) G.cur = 1 - G.cur;
     G.k += nsteps;
     G.from_init = false;

@@ -893,37 +893,6 @@ __global__ void gather_kernel(const GridDev* gd, const float* __restrict__ u_new
   gd->traces[s * gd->n_rec + r] = u_new[(size_t)iy * ld + ix];
 }
 
-// Start-up, Eq. (CN2): u^0 = phi, u^1 = phi + tau psi (+ tau^2/2 (m Lap phi + f^0)).
-__global__ void init_kernel(int nx, int ny, int ld, const float* __restrict__ m,
-                            const float* __restrict__ phi, const float* __restrict__ psi,
-                            float* __restrict__ u0, float* __restrict__ u1, double tau,
-                            double cx_half, double cy_half, int taylor, int sx, int sy,
-                            double src_half, const float* __restrict__ wavelet, int n_wavelet) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y;
-  if (i >= nx || j >= ny) return;
-  const size_t c = (size_t)j * nx + i;
-  const float phf = phi[c];
-  if (!psi && !taylor) {  // u^1 = u^0 = phi: no arithmetic
-    u0[(size_t)j * ld + i] = phf;
-    u1[(size_t)j * ld + i] = phf;
-    return;
-  }
-  const double ph = phf;
-  double v = ph + (psi ? tau * (double)psi[c] : 0.0);
-  if (taylor) {
-    const double l = (i > 0) ? phi[c - 1] : 0.0;
-    const double r = (i + 1 < nx) ? phi[c + 1] : 0.0;
-    const double dn = (j > 0) ? phi[c - nx] : 0.0;
-    const double up = (j + 1 < ny) ? phi[c + nx] : 0.0;
-    const double mm = m[(size_t)j * ld + i];
-    v += mm * (cx_half * (l + r - 2.0 * ph) + cy_half * (dn + up - 2.0 * ph));
-    if (i == sx && j == sy && wavelet != nullptr && n_wavelet > 0) v += src_half * wavelet[0];
-  }
-  u0[(size_t)j * ld + i] = (float)ph;
-  u1[(size_t)j * ld + i] = (float)v;
-}
-
 // min(m), max(m) as float bit patterns (m > 0 compares as unsigned) and a
 // flag for non-finite or non-positive entries.
 __global__ void scan_m_kernel(const float* __restrict__ m, int nx, int ny, int ld,
@@ -1439,17 +1408,6 @@ cudaError_t launch_gather(const GridDev* gd, const float* u_new, int ld, int n_r
   return cudaGetLastError();
 }
 
-cudaError_t launch_init(int nx, int ny, int ld, const float* m_pitched, const float* phi,
-                        const float* psi, float* u0, float* u1, double tau, double cx_half,
-                        double cy_half, int taylor, int sx, int sy, double src_half,
-                        const float* wavelet, int n_wavelet, cudaStream_t st) {
-  dim3 block(256, 1, 1);
-  dim3 grid((nx + 255) / 256, ny, 1);
-  init_kernel<<<grid, block, 0, st>>>(nx, ny, ld, m_pitched, phi, psi, u0, u1, tau, cx_half,
-                                      cy_half, taylor, sx, sy, src_half, wavelet, n_wavelet);
-  return cudaGetLastError();
-}
-
 __global__ void scan_init_kernel(unsigned int* out3) {
   out3[0] = 0x7f7fffffu;
   out3[1] = 0u;
@@ -1471,10 +1429,25 @@ cudaError_t launch_scan_m(const float* m, int nx, int ny, int ld, unsigned int* 
   return cudaGetLastError();
 }
 
-__global__ void put_gd_kernel(GridDev* dst, const GridDev v) { *dst = v; }
+constexpr int kPutMax = 32;
+struct PutArgs {
+  GridDev v[kPutMax];
+  GridDev* dst[kPutMax];
+};
+__global__ void put_gd_kernel(const __grid_constant__ PutArgs a, int n) {
+  if ((int)threadIdx.x < n) *a.dst[threadIdx.x] = a.v[threadIdx.x];
+}
 
-cudaError_t launch_put_gd(GridDev* dst, const GridDev& v, cudaStream_t st) {
-  put_gd_kernel<<<1, 1, 0, st>>>(dst, v);
+cudaError_t launch_put_gd(GridDev* const* dst, const GridDev* v, int n, cudaStream_t st) {
+  for (int i0 = 0; i0 < n; i0 += kPutMax) {
+    const int c = std::min(kPutMax, n - i0);
+    PutArgs a = {};
+    for (int i = 0; i < c; ++i) {
+      a.v[i] = v[i0 + i];
+      a.dst[i] = dst[i0 + i];
+    }
+    put_gd_kernel<<<1, kPutMax, 0, st>>>(a, c);
+  }
   return cudaGetLastError();
 }
 

@@ -72,17 +72,43 @@ struct YArgs {
 cudaError_t launch_x(const XArgs& a, int K, bool fp64, bool tree, cudaStream_t st);
 cudaError_t launch_y(const YArgs& a, int K, bool fp64, bool tree, cudaStream_t st);
 cudaError_t launch_gather(const GridDev* gd, const float* u_new, int ld, int n_rec, cudaStream_t st);
-cudaError_t launch_init(int nx, int ny, int ld, const float* m_pitched, const float* phi,
-                        const float* psi, float* u0, float* u1, double tau, double cx_half,
-                        double cy_half, int taylor, int src_ix, int src_iy, double src_half,
-                        const float* wavelet, int n_wavelet, cudaStream_t st);
+// Fields between the caller's contiguous rows and the handle's pitched ones
+// (adi_copy.cu): dst0 <- src0 and, if src1 is given, dst1 <- src1; without
+// src1 a given dst1 gets src0 too.  Both launches also write the grid record
+// gd to gd_dst if that is given.
+struct CopyArgs {
+  int nx, ny;
+  int spitch, dpitch;  // floats per row
+  const float* src0;
+  const float* src1;
+  float* dst0;
+  float* dst1;
+  GridDev* gd_dst;
+};
+cudaError_t launch_copy_fields(const CopyArgs& a, const GridDev& gd, cudaStream_t st);
+struct InitArgs {
+  int nx, ny, ld;
+  const float* m;    // pitched
+  const float* phi;  // contiguous, psi too (or null)
+  const float* psi;
+  float* u0;
+  float* u1;
+  double tau, cx_half, cy_half;
+  int taylor;
+  int sx, sy;
+  double src_half;
+  const float* wavelet;
+  int n_wavelet;
+  GridDev* gd_dst;
+};
+cudaError_t launch_init(const InitArgs& a, const GridDev& gd, cudaStream_t st);
 // min(m), max(m) bit patterns and a non-finite/non-positive flag into out3
 // (device) and then host3 (mapped pinned host memory, device address): three
 // launches, no copies.
 cudaError_t launch_scan_m(const float* m, int nx, int ny, int ld, unsigned int* out3,
                           unsigned int* host3, cudaStream_t st);
-// *dst = v on the stream (one-thread kernel; v travels as the argument).
-cudaError_t launch_put_gd(GridDev* dst, const GridDev& v, cudaStream_t st);
+// *dst[i] = v[i] on the stream for i < n (the records travel as kernel arguments).
+cudaError_t launch_put_gd(GridDev* const* dst, const GridDev* v, int n, cudaStream_t st);
 size_t x_smem_bytes(int spc, int tsys, bool fp64, bool tree);
 size_t y_smem_bytes(int W, int C, int tcol, bool fp64, bool tree);
 size_t y_stage_bytes(int threads, int K);
@@ -131,8 +157,6 @@ struct TileArgs {
   float scx, scy;      // tau^2 / (2 h1^2), tau^2 / (2 h2^2)
   float src_scale;     // tau^2 / (h1 h2)
   float* u_prev;       // in: u^{k-1}; out: u^{k+1}
-  float* w_out;        // copies of w and z for the adjoint, or null (both)
-  float* z_out;
   int gather;          // sample the receivers of gd
   GridDev* gd;
   int* err;
@@ -156,6 +180,17 @@ int patch_strips(int nx);
 cudaError_t encode_patch_map(CUtensorMap* out, const float* base, int nx, int ld, int ny, bool u);
 cudaError_t launch_patch(const TileArgs& a, int H, const CUtensorMap& u, const CUtensorMap& m, cudaStream_t st);
 cudaError_t configure_patch_kernels();
+// One grid of a batch advanced by one launch per step: arguments (par and
+// u_prev from the launch) and tensor maps, in device memory.
+struct BatchTile {
+  CUtensorMap u[2], p[2], m;  // of buf[0], buf[1] (panel and strip boxes) and m
+  TileArgs a;
+  float* buf[2];
+};
+cudaError_t launch_tile_batch(const BatchTile* tiles, const int2* items, int n_items, int par, int H,
+                              cudaStream_t st);
+cudaError_t launch_patch_batch(const BatchTile* tiles, const int2* items, int n_items, int par, int H,
+                               cudaStream_t st);
 // 2D tensor map {nx, ny} of a field of row pitch ld with boxes of {box_cols,
 // box_rows}, zero fill outside, optionally in the 128-byte swizzle
 // (box_cols = 32).

@@ -91,7 +91,8 @@ struct Elim2 {
     }
   }
   __device__ __forceinline__ void solve(f2& G, f2& D) const {
-    const f2 r = pk(rcp_t(-lo2(p)), rcp_t(-hi2(p)));
+    f2 r = pk(rcp_t(-lo2(p)), rcp_t(-hi2(p)));
+    r = fma2(fma2(p, r, dup2(1.f)), r, r);  // one Newton step on the approximate reciprocal
     G = mul2(a, r);
     D = mul2(N, r);
   }

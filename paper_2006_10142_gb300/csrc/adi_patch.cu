@@ -50,10 +50,10 @@ constexpr int kPatchSmem = kPOffBar + 8 + 1016;  // the base is aligned to 1024
 
 }  // namespace
 
-template <int H, bool KEEP>
-__global__ void __launch_bounds__(kPN, 2)
-    patch_step_kernel(const TileArgs a, const __grid_constant__ CUtensorMap tm_u,
-                      const __grid_constant__ CUtensorMap tm_m) {
+// Patch `blk` of one grid.
+template <int H>
+__device__ __forceinline__ void patch_body(const TileArgs& a, const CUtensorMap* tm_u, const CUtensorMap* tm_m,
+                                           int blk) {
   constexpr int PY = kPR - 2 * H;  // rows of a patch
   extern __shared__ unsigned char smem_raw[];
   const uint32_t sa0 = (uint32_t)__cvta_generic_to_shared(smem_raw);
@@ -66,8 +66,8 @@ __global__ void __launch_bounds__(kPN, 2)
   const uint32_t bar = sa + kPOffBar;
   const int tid = threadIdx.x;
   const int lane = tid & 31;
-  const int strip = blockIdx.x % a.strips;
-  const int band = blockIdx.x / a.strips;
+  const int strip = blk % a.strips;
+  const int band = blk / a.strips;
   const int r0 = band * PY - H;         // first staged row
   const int c0 = strip * kPX - kPH;     // first staged column
 
@@ -87,9 +87,9 @@ __global__ void __launch_bounds__(kPN, 2)
   if (tid < 32) {
     if (lane == 0) mbar_arrive_expect_tx(bar, (uint32_t)((kPCols / 32) * (66 + kPR) * 128));
     __syncwarp();
-    if (lane < 4) tma_load_2d(sa + kPOffM + (uint32_t)(lane * kMPanel), &tm_m, c0 + 32 * lane, r0, bar);
+    if (lane < 4) tma_load_2d(sa + kPOffM + (uint32_t)(lane * kMPanel), tm_m, c0 + 32 * lane, r0, bar);
     chain_wait();
-    if (lane < 4) tma_load_2d(sa + (uint32_t)(lane * kUPanel), &tm_u, c0 + 32 * lane, r0 - 1, bar);
+    if (lane < 4) tma_load_2d(sa + (uint32_t)(lane * kUPanel), tm_u, c0 + 32 * lane, r0 - 1, bar);
   } else {
     chain_wait();
   }
@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(kPN, 2)
     sy = gd->src_iy;
     fsrc = sg * (a.src_scale * gd->wavelet[lev]);
   }
-  if (blockIdx.x == 0 && tid == 0) a.gd->kf[a.par ^ 1] = lev + 1;
+  if (blk == 0 && tid == 0) a.gd->kf[a.par ^ 1] = lev + 1;
   Sampler rec;
   if (a.gather) rec.find(gd, lev, c0 + kPH, c0 + kPH + kPX, r0 + H, r0 + H + PY);
 
@@ -247,11 +247,6 @@ __global__ void __launch_bounds__(kPN, 2)
         const uint32_t key = (uint32_t)((i & 7) << 4);
         S[i] = mul2((i & 1) ? scy_n : scy_p, lds2((ym ^ key) + i * 128));
         D[i] = lds2((yw ^ key) + i * 128);
-        if (KEEP && i >= ylo && i < yhi) {
-          float* o = a.w_out + ((ptrdiff_t)(r0 + 16 * yc + i) * (ptrdiff_t)ld + yi);
-          if (ok0) o[0] = sgn_d(i) * lo2(D[i]);
-          if (ok1) o[1] = sgn_d(i) * hi2(D[i]);
-        }
       }
       e.begin(0ull, 0ull);
       e.tail<H>(S, D);
@@ -287,11 +282,6 @@ __global__ void __launch_bounds__(kPN, 2)
           float* o = orow + i * ld;
           if (ok1) *reinterpret_cast<f2*>(o) = un;
           else if (ok0) o[0] = lo2(un);
-          if (KEEP) {
-            float* z = a.z_out + ((ptrdiff_t)(r0 + 16 * yc + i) * (ptrdiff_t)ld + yi);
-            if (ok0) z[0] = -sgn_d(i) * lo2(X);
-            if (ok1) z[1] = -sgn_d(i) * hi2(X);
-          }
           if (ok0) chk = fma2(un, 0ull, chk);
         }
       }
@@ -306,6 +296,25 @@ __global__ void __launch_bounds__(kPN, 2)
   }
 }
 
+template <int H>
+__global__ void __launch_bounds__(kPN, 2)
+    patch_step_kernel(const TileArgs a, const __grid_constant__ CUtensorMap tm_u,
+                      const __grid_constant__ CUtensorMap tm_m) {
+  patch_body<H>(a, &tm_u, &tm_m, blockIdx.x);
+}
+
+// A step of many grids: items[b] = (grid, patch) of CTA b.
+template <int H>
+__global__ void __launch_bounds__(kPN, 2)
+    patch_batch_kernel(const BatchTile* __restrict__ tiles, const int2* __restrict__ items, int par) {
+  const int2 it = __ldg(items + blockIdx.x);
+  const BatchTile& t = tiles[it.x];
+  TileArgs a = t.a;
+  a.par = par;
+  a.u_prev = t.buf[par ^ 1];
+  patch_body<H>(a, &t.u[par], &t.m, it.y);
+}
+
 // ---------------------------------------------------------------------------
 // host
 // ---------------------------------------------------------------------------
@@ -316,31 +325,29 @@ cudaError_t encode_patch_map(CUtensorMap* out, const float* base, int nx, int ld
   return encode_box_map(out, base, nx, ld, ny, 32, u ? kPR + 2 : kPR, true);
 }
 
-template <int H, bool KEEP>
-static cudaError_t launch_patch_t(const TileArgs& a, const CUtensorMap& u, const CUtensorMap& m, cudaStream_t st) {
-  const int bands = (a.ny + kPR - 2 * H - 1) / (kPR - 2 * H);
-  return launch_chained(patch_step_kernel<H, KEEP>, a.strips * bands, kPN, kPatchSmem, st, a, u, m);
-}
-
 cudaError_t launch_patch(const TileArgs& a_in, int H, const CUtensorMap& u, const CUtensorMap& m, cudaStream_t st) {
   TileArgs a = a_in;
   a.strips = patch_strips(a.nx);
-  const bool keep = a.w_out != nullptr;
-  if (keep && a.z_out == nullptr) return cudaErrorInvalidValue;
-  if (H == 12) return keep ? launch_patch_t<12, true>(a, u, m, st) : launch_patch_t<12, false>(a, u, m, st);
-  if (H == 16) return keep ? launch_patch_t<16, true>(a, u, m, st) : launch_patch_t<16, false>(a, u, m, st);
-  return cudaErrorInvalidValue;
+  if (H != 12 && H != 16) return cudaErrorInvalidValue;
+  const int bands = (a.ny + patch_rows(H) - 1) / patch_rows(H);
+  return launch_chained(H == 12 ? patch_step_kernel<12> : patch_step_kernel<16>, a.strips * bands, kPN, kPatchSmem, st,
+                        a, u, m);
+}
+
+cudaError_t launch_patch_batch(const BatchTile* tiles, const int2* items, int n_items, int par, int H,
+                               cudaStream_t st) {
+  return launch_chained(H == 12 ? patch_batch_kernel<12> : patch_batch_kernel<16>, n_items, kPN, kPatchSmem, st,
+                        tiles, items, par);
 }
 
 cudaError_t configure_patch_kernels() {
   cudaError_t e = cudaSuccess;
-#define ADI_PATCH_CFG(H, K)                                                                   \
-  if (e == cudaSuccess)                                                                       \
-    e = cudaFuncSetAttribute(patch_step_kernel<H, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPatchSmem);
-  ADI_PATCH_CFG(12, false)
-  ADI_PATCH_CFG(12, true)
-  ADI_PATCH_CFG(16, false)
-  ADI_PATCH_CFG(16, true)
+#define ADI_PATCH_CFG(K) \
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, kPatchSmem);
+  ADI_PATCH_CFG(patch_step_kernel<12>)
+  ADI_PATCH_CFG(patch_step_kernel<16>)
+  ADI_PATCH_CFG(patch_batch_kernel<12>)
+  ADI_PATCH_CFG(patch_batch_kernel<16>)
 #undef ADI_PATCH_CFG
   return e;
 }

@@ -104,7 +104,7 @@ int adi_wave::ensure_ycoop(Grid& G) {
 int adi_wave::upload_gd(Grid& G, cudaStream_t st) {
   G.hgd.kf[0] = G.hgd.k;
   G.hgd.kf[1] = G.hgd.k;
-  CK(launch_put_gd(G.gd, G.hgd, st), "upload grid state");
+  CK(launch_put_gd(&G.gd, &G.hgd, 1, st), "upload grid state");
   launches += 1;
   return ADI_OK;
 }
@@ -171,9 +171,26 @@ int adi_wave::run_batch(int steps, const adi_source* src, cudaStream_t st) {
     G.hgd.n_rec = 0;
     G.hgd.rec = nullptr;
     G.hgd.traces = nullptr;
-    if (upload_gd(G, st) != ADI_OK) return ADI_ECUDA;
+    G.hgd.kf[0] = G.hgd.kf[1] = G.k;
+  }
+  {
+    std::vector<GridDev*> dst;
+    std::vector<GridDev> v;
+    for (Grid& G : g) {
+      dst.push_back(G.gd);
+      v.push_back(G.hgd);
+    }
+    CK(launch_put_gd(dst.data(), v.data(), (int)g.size(), st), "upload grid states");
+    launches += ((int)g.size() + 31) / 32;
   }
   rr.valid = false;
+  bool aligned = true;  // a reset that failed half way leaves shots in two orientations
+  for (const Grid& G : g) aligned = aligned && G.cur == g[0].cur;
+  if (batch_mode == 2 && aligned) {
+    const int rc = ensure_batch_tiles();
+    if (rc != ADI_OK) return rc;
+    if (bt_n > 0) return run_batch_tiles(steps, st);
+  }
   const bool use_graph = g[0].plan.graph && !profile;
   int t = 0;
   if (use_graph) {
@@ -243,8 +260,15 @@ int adi_wave::start_grid(int s, const float* m, const float* phi, const float* p
     unsigned int res3[3] = {scan_host[0], scan_host[1], scan_host[2]};
     launches += 3;
     if (res3[2]) return fail(this, ADI_EINVAL, "m must be finite and > 0 everywhere");
-    CK(cudaMemcpy2DAsync(G.m, sizeof(float) * G.ld, m, sizeof(float) * G.nx,
-                         sizeof(float) * G.nx, G.ny, cudaMemcpyDeviceToDevice, st), "copy m");
+    CopyArgs c = {};
+    c.nx = G.nx;
+    c.ny = G.ny;
+    c.spitch = G.nx;
+    c.dpitch = G.ld;
+    c.src0 = m;
+    c.dst0 = G.m;
+    CK(launch_copy_fields(c, GridDev{}, st), "copy m");
+    launches += 1;
     float lo, hi;
     memcpy(&lo, &res3[0], 4);
     memcpy(&hi, &res3[1], 4);
@@ -267,14 +291,28 @@ int adi_wave::start_grid(int s, const float* m, const float* phi, const float* p
   G.hgd.k0 = 1;
   G.hgd.src_ix = -1;
   G.hgd.src_iy = -1;
-  if (upload_gd(G, st) != ADI_OK) return ADI_ECUDA;
+  G.hgd.kf[0] = G.hgd.kf[1] = 1;
   const bool has_src = sr && sr->ix >= 0 && sr->wavelet && sr->n_wavelet > 0;
-  CK(launch_init(G.nx, G.ny, G.ld, G.m, phi, psi, G.buf[0], G.buf[1], G.dt,
-                 G.dt * G.dt / (2.0 * G.hx * G.hx), G.dt * G.dt / (2.0 * G.hy * G.hy),
-                 G.start == ADI_START_TAYLOR2 ? 1 : 0, has_src ? sr->ix : -1,
-                 has_src ? sr->iy : -1, G.dt * G.dt / (2.0 * G.hx * G.hy),
-                 has_src ? sr->wavelet : nullptr, has_src ? sr->n_wavelet : 0, st),
-     "init kernel");
+  InitArgs ia = {};
+  ia.nx = G.nx;
+  ia.ny = G.ny;
+  ia.ld = G.ld;
+  ia.m = G.m;
+  ia.phi = phi;
+  ia.psi = psi;
+  ia.u0 = G.buf[0];
+  ia.u1 = G.buf[1];
+  ia.tau = G.dt;
+  ia.cx_half = G.dt * G.dt / (2.0 * G.hx * G.hx);
+  ia.cy_half = G.dt * G.dt / (2.0 * G.hy * G.hy);
+  ia.taylor = G.start == ADI_START_TAYLOR2 ? 1 : 0;
+  ia.sx = has_src ? sr->ix : -1;
+  ia.sy = has_src ? sr->iy : -1;
+  ia.src_half = G.dt * G.dt / (2.0 * G.hx * G.hy);
+  ia.wavelet = has_src ? sr->wavelet : nullptr;
+  ia.n_wavelet = has_src ? sr->n_wavelet : 0;
+  ia.gd_dst = G.gd;
+  CK(launch_init(ia, G.hgd, st), "init kernel");
   launches += 1;
   G.cur = 1;
   G.k = 1;
@@ -324,10 +362,11 @@ int adi_wave::prof_end(cudaStream_t st, cudaEvent_t a, int kind) {
   return ADI_OK;
 }
 
-int adi_wave::enqueue_step(Grid& G, cudaStream_t st, bool gather) {
+int adi_wave::enqueue_step(Grid& G, cudaStream_t st, bool gather, bool one_pass) {
   float* u_cur = G.buf[G.cur];
   float* u_prev = G.buf[1 - G.cur];
-  int rc = launch_fwd(G, u_cur, u_prev, G.w, nullptr, G.gd, G.cur, gather, st);
+  int rc = one_pass ? launch_fwd_tile(G, u_cur, u_prev, G.gd, G.cur, gather, st)
+                    : launch_fwd(G, u_cur, u_prev, G.w, nullptr, G.gd, gather, st);
   if (rc != ADI_OK) return rc;
   G.cur = 1 - G.cur;
   G.k += 1;
@@ -335,10 +374,10 @@ int adi_wave::enqueue_step(Grid& G, cudaStream_t st, bool gather) {
   return ADI_OK;
 }
 
-// The same step as one launch (adi_tile.cu, adi_patch.cu); w and z are
-// written only when z_out is given.
-int adi_wave::launch_fwd_tile(Grid& G, const float* u_cur, float* u_prev, float* w, float* z_out,
-                              GridDev* gd, int par, bool gather, cudaStream_t st) {
+// The same step as one launch (adi_tile.cu, adi_patch.cu).  par: which level
+// word of gd it reads (it leaves the next level in the other one).
+int adi_wave::launch_fwd_tile(Grid& G, const float* u_cur, float* u_prev, GridDev* gd, int par, bool gather,
+                              cudaStream_t st) {
   const bool patch = G.plan.tile_rows == 0;
   auto encode = [&](CUtensorMap* out, const float* p, bool u) {
     return patch ? encode_patch_map(out, p, G.nx, G.ld, G.ny, u) : encode_tile_map(out, p, G.nx, G.ld, G.ny, false);
@@ -367,8 +406,6 @@ int adi_wave::launch_fwd_tile(Grid& G, const float* u_cur, float* u_prev, float*
   TileArgs a = tile_args(G);
   a.par = par;
   a.u_prev = u_prev;
-  a.w_out = z_out != nullptr ? w : nullptr;
-  a.z_out = z_out;
   a.gather = gather ? 1 : 0;
   a.gd = gd;
   a.err = d_err;
@@ -381,13 +418,11 @@ int adi_wave::launch_fwd_tile(Grid& G, const float* u_cur, float* u_prev, float*
 }
 
 // One forward step on explicit buffers: x sweep into w, y sweep + update
-// writing u^{k+1} over u_prev (and z into z_out when given).  par: which
-// level word of gd the one-pass step reads (it leaves the next level in the
-// other one).  gather: sample the receivers of gd.
+// writing u^{k+1} over u_prev (and z into z_out when given).  gather: sample
+// the receivers of gd.
 int adi_wave::launch_fwd(Grid& G, const float* u_cur, float* u_prev, float* w, float* z_out,
-                         GridDev* gd, int par, bool gather, cudaStream_t st) {
+                         GridDev* gd, bool gather, cudaStream_t st) {
   const GridPlan& P = G.plan;
-  if (P.tile) return launch_fwd_tile(G, u_cur, u_prev, w, z_out, gd, par, gather, st);
   XArgs xa;
   xa.nx = G.nx;
   xa.ny = G.ny;
@@ -494,22 +529,22 @@ int adi_wave::launch_fwd(Grid& G, const float* u_cur, float* u_prev, float* w, f
 
 void adi_wave::drop_graphs() {
   for (int o = 0; o < 2; ++o)
-    for (int q = 0; q < 2; ++q)
+    for (int q = 0; q < 4; ++q)
       if (pair[o][q]) {
         cudaGraphExecDestroy(pair[o][q]);
         pair[o][q] = nullptr;
       }
 }
 
-int adi_wave::launch_pair_graph(Grid& G, cudaStream_t st, bool gather) {
-  cudaGraphExec_t& ex = pair[G.cur][gather ? 1 : 0];
+int adi_wave::launch_pair_graph(Grid& G, cudaStream_t st, bool gather, bool one_pass) {
+  cudaGraphExec_t& ex = pair[G.cur][(gather ? 1 : 0) + (one_pass ? 2 : 0)];
   if (!ex) {
     const int cur0 = G.cur;
     const long long k0 = G.k;
     const int64_t l0 = launches;
     CK(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal), "begin capture");
-    int rc = enqueue_step(G, cap, gather);
-    if (rc == ADI_OK) rc = enqueue_step(G, cap, gather);
+    int rc = enqueue_step(G, cap, gather, one_pass);
+    if (rc == ADI_OK) rc = enqueue_step(G, cap, gather, one_pass);
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamEndCapture(cap, &graph);
     G.cur = cur0;
@@ -528,7 +563,7 @@ int adi_wave::launch_pair_graph(Grid& G, cudaStream_t st, bool gather) {
     }
   }
   CK(cudaGraphLaunch(ex, st), "graph launch");
-  launches += G.plan.tile ? 2 : gather ? 6 : 4;
+  launches += one_pass ? 2 : gather ? 6 : 4;
   G.k += 2;
   return ADI_OK;
 }
@@ -607,7 +642,12 @@ int adi_wave::run(int steps, const adi_source* src, const int32_t* rec_xy, int n
   }
 
   const bool gather = n_rec > 0;
-  const bool use_graph = G.plan.graph && !profile;
+  // A run that keeps checkpoints is one to be differentiated: its steps are
+  // the separate sweeps, whose w and z the reverse sweep recomputes.  The
+  // gradient is made of differences of nearly equal FP32 fields (z - w), so
+  // its last digits follow the rounding of every forward value.
+  const bool one_pass = G.plan.tile != 0 && every == 0;
+  const bool use_graph = (one_pass ? tuning.use_graph > 0 : G.plan.graph) && !profile;
   const size_t fbytes = sizeof(float) * (size_t)G.ld * G.ny;
   int s = 0;
   while (s < steps) {
@@ -631,13 +671,13 @@ int adi_wave::run(int steps, const adi_source* src, const int32_t* rec_xy, int n
     }
     if (use_graph) {
       while (seg - t >= 2) {
-        int rc = launch_pair_graph(G, st, gather);
+        int rc = launch_pair_graph(G, st, gather, one_pass);
         if (rc != ADI_OK) return rc;
         t += 2;
       }
     }
     while (t < seg) {
-      int rc = enqueue_step(G, st, gather);
+      int rc = enqueue_step(G, st, gather, one_pass);
       if (rc != ADI_OK) return rc;
       t += 1;
     }
@@ -650,17 +690,24 @@ int adi_wave::run(int steps, const adi_source* src, const int32_t* rec_xy, int n
 int adi_wave::set_state(int shot, const float* u_prev, const float* u_cur, int64_t k,
                         cudaStream_t st) {
   Grid& G = g[shot];
-  const size_t wb = sizeof(float) * (size_t)G.nx;
-  CK(cudaMemcpy2DAsync(G.buf[1 - G.cur], sizeof(float) * G.ld, u_prev, wb, wb, G.ny,
-                       cudaMemcpyDeviceToDevice, st), "set_state");
-  CK(cudaMemcpy2DAsync(G.buf[G.cur], sizeof(float) * G.ld, u_cur, wb, wb, G.ny,
-                       cudaMemcpyDeviceToDevice, st), "set_state");
   G.k = k;
   G.from_init = false;
   G.hgd.k = k;
   G.hgd.k0 = k;
+  G.hgd.kf[0] = G.hgd.kf[1] = k;
   G.hgd.steps = 0;
-  if (upload_gd(G, st) != ADI_OK) return ADI_ECUDA;
+  CopyArgs c = {};
+  c.nx = G.nx;
+  c.ny = G.ny;
+  c.spitch = G.nx;
+  c.dpitch = G.ld;
+  c.src0 = u_prev;
+  c.src1 = u_cur;
+  c.dst0 = G.buf[1 - G.cur];
+  c.dst1 = G.buf[G.cur];
+  c.gd_dst = G.gd;
+  CK(launch_copy_fields(c, G.hgd, st), "set_state");
+  launches += 1;
   rr.valid = false;
   return ADI_OK;
 }
@@ -744,6 +791,8 @@ adi_wave::~adi_wave() {
   if (d_shots) cudaFree(d_shots);
   if (d_items) cudaFree(d_items);
   if (d_sync) cudaFree(d_sync);
+  if (bt_dev) cudaFree(bt_dev);
+  if (bt_items) cudaFree(bt_items);
   for (int b = 0; b < kBranches; ++b) {
     if (branch[b]) cudaStreamDestroy(branch[b]);
     if (join_ev[b]) cudaEventDestroy(join_ev[b]);

@@ -128,7 +128,7 @@ struct adi_wave {
   unsigned int* scan_host_dev = nullptr;
   int rec_cap = 0;
   cudaStream_t cap = nullptr;  // private stream used only for graph capture
-  cudaGraphExec_t pair[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};  // [orientation][gather]
+  cudaGraphExec_t pair[2][4] = {};  // [orientation][gather + 2 one_pass]
   adi_wave_tuning tuning = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
   int ckpt_every = 0;
   adi::RunRecord rr;
@@ -151,7 +151,7 @@ struct adi_wave {
   std::vector<int> shot_order;  // batch mode 2: shots by decreasing size
   std::vector<int> shot_branch; // batch mode 2: branch of each shot
   int ensure_branches();
-  int enqueue_batch_steps_parallel(int nsteps, cudaStream_t st);
+  int enqueue_batch_steps_parallel(int nsteps, cudaStream_t st, bool rest = false);
   adi::BatchShot* d_shots = nullptr;
   int2* d_items = nullptr;
   int n_items = 0;
@@ -163,6 +163,15 @@ struct adi_wave {
   int64_t pair_launches = 0;
   int setup_batch(cudaStream_t st);
   int enqueue_batch_step(cudaStream_t st);
+  // batch mode 2, one launch per step for the shots whose plan is one-pass
+  adi::BatchTile* bt_dev = nullptr;      // one per such shot
+  int2* bt_items = nullptr;              // (index into bt_dev, CTA of that grid) per CTA
+  int bt_n = 0, bt_n_items = 0, bt_h = 0;
+  bool bt_patch = false;
+  std::vector<adi::GridPlan> bt_plans;   // plans the tables were made for
+  int ensure_batch_tiles();
+  int run_batch_tiles(int steps, cudaStream_t st);
+  int launch_batch_fwd(adi::Grid& G, int cur, cudaStream_t st);
   int run_batch(int steps, const adi_source* src, cudaStream_t st);
 
   int create(const adi_wave_desc* desc, int n, const float* const* m, const float* const* phi,
@@ -181,14 +190,14 @@ struct adi_wave {
   ~adi_wave();
 
   // internals
-  int enqueue_step(adi::Grid& G, cudaStream_t st, bool gather);
+  int enqueue_step(adi::Grid& G, cudaStream_t st, bool gather, bool one_pass);
   int launch_fwd(adi::Grid& G, const float* u_cur, float* u_prev, float* w, float* z_out,
-                 adi::GridDev* gd, int par, bool gather, cudaStream_t st);
-  int launch_fwd_tile(adi::Grid& G, const float* u_cur, float* u_prev, float* w, float* z_out,
-                      adi::GridDev* gd, int par, bool gather, cudaStream_t st);
+                 adi::GridDev* gd, bool gather, cudaStream_t st);
+  int launch_fwd_tile(adi::Grid& G, const float* u_cur, float* u_prev, adi::GridDev* gd, int par, bool gather,
+                      cudaStream_t st);
   int ensure_adj_work(adi::Grid& G, int E, int n_rec);
   void free_adj_work();
-  int launch_pair_graph(adi::Grid& G, cudaStream_t st, bool gather);
+  int launch_pair_graph(adi::Grid& G, cudaStream_t st, bool gather, bool one_pass);
   void drop_graphs();
   int prof_begin(cudaStream_t st, cudaEvent_t* a);
   int prof_end(cudaStream_t st, cudaEvent_t a, int kind);

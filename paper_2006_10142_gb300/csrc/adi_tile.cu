@@ -81,11 +81,10 @@ struct Col {
 
 }  // namespace
 
-template <int H, bool KEEP>
-__global__ void __launch_bounds__(kTN, 2)
-    tile_step_kernel(const TileArgs a, const __grid_constant__ CUtensorMap tm_u,
-                     const __grid_constant__ CUtensorMap tm_m, const __grid_constant__ CUtensorMap tm_p,
-                     const __grid_constant__ CUtensorMap tm_o) {
+// CTA `blk` of one grid.
+template <int H>
+__device__ __forceinline__ void tile_body(const TileArgs& a, const CUtensorMap* tm_u, const CUtensorMap* tm_m,
+                                          const CUtensorMap* tm_p, const CUtensorMap* tm_o, int blk) {
   extern __shared__ unsigned char smem_raw[];
   const uint32_t sa0 = (uint32_t)__cvta_generic_to_shared(smem_raw);
   const uint32_t sa = (sa0 + 1023u) & ~1023u;
@@ -95,8 +94,8 @@ __global__ void __launch_bounds__(kTN, 2)
   const uint32_t bar = sa + kOffBar;
   const int tid = threadIdx.x;
   const int lane = tid & 31;
-  const int strip = blockIdx.x % a.strips;
-  const int band = blockIdx.x / a.strips;
+  const int strip = blk % a.strips;
+  const int band = blk / a.strips;
   const int y0 = band * a.band_rows;
   const int y1 = min(a.ny, y0 + a.band_rows);
   const int rs = max(0, y0 - kTB);                 // first row processed
@@ -125,19 +124,21 @@ __global__ void __launch_bounds__(kTN, 2)
     const int p = lane & 7, f = lane >> 3;
     const int col = c0 + 32 * p, row = rs + kTB * b;
     if (f == 0) {
-      tma_load_2d(sa + (uint32_t)((b % 3) * kSlot + p * kPanel), &tm_u, col, row + 1, mb);
-      if (b == 0) tma_load_2d(sa + (uint32_t)(2 * kSlot + p * kPanel), &tm_u, col, row + 1 - kTB, mb);
+      tma_load_2d(sa + (uint32_t)((b % 3) * kSlot + p * kPanel), tm_u, col, row + 1, mb);
+      if (b == 0) tma_load_2d(sa + (uint32_t)(2 * kSlot + p * kPanel), tm_u, col, row + 1 - kTB, mb);
     } else if (f == 1) {
-      tma_load_2d(sa + (uint32_t)(kOffM + (b & 1) * kSlot + p * kPanel), &tm_m, col, row, mb);
+      tma_load_2d(sa + (uint32_t)(kOffM + (b & 1) * kSlot + p * kPanel), tm_m, col, row, mb);
     } else if (lane == 16) {
-      tma_prefetch_2d(&tm_p, strip * kTX, row);
+      tma_prefetch_2d(tm_p, strip * kTX, row);
     }
   };
   // one thread: block b of u^{k-1}, the strip's own columns
   auto issue_prev = [&](int b) {
     mbar_arrive_expect_tx(bar + 16u, (uint32_t)kOut);
-    tma_load_2d(sa + (uint32_t)kOffP, &tm_p, strip * kTX, rs + kTB * b, bar + 16u);
+    tma_load_2d(sa + (uint32_t)kOffP, tm_p, strip * kTX, rs + kTB * b, bar + 16u);
   };
+  chain_wait();
+  chain_release();
   if (tid < 32) {
     issue(0);
     if (lane == 0) issue_prev(0);
@@ -174,7 +175,7 @@ __global__ void __launch_bounds__(kTN, 2)
       sy = gd->src_iy;
       fsrc = sg * (a.src_scale * gd->wavelet[lev]);
     }
-    if (blockIdx.x == 0 && tid == 0) a.gd->kf[a.par ^ 1] = lev + 1;
+    if (blk == 0 && tid == 0) a.gd->kf[a.par ^ 1] = lev + 1;
   }
 
   // y phase: columns 2 tid, 2 tid + 1 of the strip, 16 columns into the stage
@@ -198,11 +199,6 @@ __global__ void __launch_bounds__(kTN, 2)
     float* o = a.u_prev + (size_t)j * ld + yi;
     if (ok0) o[0] = lo2(un);
     if (ok1) o[1] = hi2(un);
-    if (KEEP) {
-      float* z = a.z_out + (size_t)j * ld + yi;
-      if (ok0) z[0] = -sgn_d(i) * lo2(X);
-      if (ok1) z[1] = -sgn_d(i) * hi2(X);
-    }
     if (ok0) chk = fma2(un, 0ull, chk);
   };
 
@@ -322,14 +318,6 @@ __global__ void __launch_bounds__(kTN, 2)
         const uint32_t key = (uint32_t)((i & 7) << 4);
         const f2 s = mul2((i & 1) ? scy_n : scy_p, lds2((pm ^ key) + i * 128));
         const f2 w = lds2((yw ^ key) + i * 128);
-        if (KEEP) {
-          const int j = row0 + i;
-          if (j >= y0 && j < y1) {
-            float* o = a.w_out + (size_t)j * ld + yi;
-            if (ok0) o[0] = sgn_d(i) * lo2(w);
-            if (ok1) o[1] = sgn_d(i) * hi2(w);
-          }
-        }
         if (i & 1) e.add<1>(s, w);
         else e.add<0>(s, w);
         e.solve(C.g[i], C.d[i]);
@@ -354,11 +342,6 @@ __global__ void __launch_bounds__(kTN, 2)
           X = fma2(cur ? C.g[i] : P.g[i], X, cur ? C.d[i] : P.d[i]);
           const f2 un = updated(i, cur ? C.q[i] : P.q[i], X);
           *reinterpret_cast<f2*>(__cvta_shared_to_generic((yw ^ (uint32_t)((e2 & 7) << 4)) + e2 * 128)) = un;
-          if (KEEP) {
-            float* z = a.z_out + (size_t)(r0 + e2) * ld + yi;
-            if (ok0) z[0] = -sgn_d(i) * lo2(X);
-            if (ok1) z[1] = -sgn_d(i) * hi2(X);
-          }
           chk = fma2(un, 0ull, chk);
         }
       } else {
@@ -376,7 +359,7 @@ __global__ void __launch_bounds__(kTN, 2)
     if (tid < 32) {
       if (full) {
         const int col = strip * kTX + 32 * lane;
-        if (lane < kTX / 32 && col < a.nx) tma_store_2d(&tm_o, col, r0, sa + kOffW + (uint32_t)(lane * kPanel));
+        if (lane < kTX / 32 && col < a.nx) tma_store_2d(tm_o, col, r0, sa + kOffW + (uint32_t)(lane * kPanel));
         bulk_commit();
       }
       fence_proxy_async_smem();
@@ -426,6 +409,26 @@ __global__ void __launch_bounds__(kTN, 2)
   const bool bad = lo2(chk) != 0.f || hi2(chk) != 0.f;
   if (__any_sync(0xffffffffu, bad) && lane == 0 && a.err) atomicOr(a.err, ERR_NUMERIC);
   if (timed_out && lane == 0 && a.err) atomicOr(a.err, ERR_TIMEOUT);
+}
+
+template <int H>
+__global__ void __launch_bounds__(kTN, 2)
+    tile_step_kernel(const TileArgs a, const __grid_constant__ CUtensorMap tm_u,
+                     const __grid_constant__ CUtensorMap tm_m, const __grid_constant__ CUtensorMap tm_p,
+                     const __grid_constant__ CUtensorMap tm_o) {
+  tile_body<H>(a, &tm_u, &tm_m, &tm_p, &tm_o, blockIdx.x);
+}
+
+// A step of many grids: items[b] = (grid, CTA of that grid) of CTA b.
+template <int H>
+__global__ void __launch_bounds__(kTN, 2)
+    tile_batch_kernel(const BatchTile* __restrict__ tiles, const int2* __restrict__ items, int par) {
+  const int2 it = __ldg(items + blockIdx.x);
+  const BatchTile& t = tiles[it.x];
+  TileArgs a = t.a;
+  a.par = par;
+  a.u_prev = t.buf[par ^ 1];
+  tile_body<H>(a, &t.u[par], &t.m, &t.p[par ^ 1], &t.u[par ^ 1], it.y);
 }
 
 // ---------------------------------------------------------------------------
@@ -478,32 +481,29 @@ cudaError_t encode_tile_map(CUtensorMap* out, const float* base, int nx, int ld,
   return encode_box_map(out, base, nx, ld, ny, strip ? kTX : 32, kTB, !strip);
 }
 
-template <int H, bool KEEP>
-static cudaError_t launch_tile_t(const TileArgs& a, const TileMaps& mp, cudaStream_t st) {
-  const int bands = (a.ny + a.band_rows - 1) / a.band_rows;
-  tile_step_kernel<H, KEEP><<<a.strips * bands, kTN, kTileSmem, st>>>(a, mp.u, mp.m, mp.p, mp.o);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_tile(const TileArgs& a_in, int H, const TileMaps& mp, cudaStream_t st) {
   TileArgs a = a_in;
   a.strips = tile_strips(a.nx);
-  const bool keep = a.w_out != nullptr;
-  if (a.band_rows < kTB || a.band_rows % kTB != 0 || (keep && a.z_out == nullptr)) return cudaErrorInvalidValue;
-  if (H == 12) return keep ? launch_tile_t<12, true>(a, mp, st) : launch_tile_t<12, false>(a, mp, st);
-  if (H == 16) return keep ? launch_tile_t<16, true>(a, mp, st) : launch_tile_t<16, false>(a, mp, st);
-  return cudaErrorInvalidValue;
+  if (a.band_rows < kTB || a.band_rows % kTB != 0 || (H != 12 && H != 16)) return cudaErrorInvalidValue;
+  const int bands = (a.ny + a.band_rows - 1) / a.band_rows;
+  return launch_chained(H == 12 ? tile_step_kernel<12> : tile_step_kernel<16>, a.strips * bands, kTN, kTileSmem, st,
+                        a, mp.u, mp.m, mp.p, mp.o);
+}
+
+cudaError_t launch_tile_batch(const BatchTile* tiles, const int2* items, int n_items, int par, int H,
+                              cudaStream_t st) {
+  return launch_chained(H == 12 ? tile_batch_kernel<12> : tile_batch_kernel<16>, n_items, kTN, kTileSmem, st, tiles,
+                        items, par);
 }
 
 cudaError_t configure_tile_kernels() {
   cudaError_t e = cudaSuccess;
-#define ADI_TILE_CFG(H, K)                                                                   \
-  if (e == cudaSuccess)                                                                      \
-    e = cudaFuncSetAttribute(tile_step_kernel<H, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmem);
-  ADI_TILE_CFG(12, false)
-  ADI_TILE_CFG(12, true)
-  ADI_TILE_CFG(16, false)
-  ADI_TILE_CFG(16, true)
+#define ADI_TILE_CFG(K) \
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmem);
+  ADI_TILE_CFG(tile_step_kernel<12>)
+  ADI_TILE_CFG(tile_step_kernel<16>)
+  ADI_TILE_CFG(tile_batch_kernel<12>)
+  ADI_TILE_CFG(tile_batch_kernel<16>)
 #undef ADI_TILE_CFG
   return e;
 }
