@@ -61,6 +61,8 @@ __device__ __noinline__ void add_wavelet_grad(float* gw, long long level, double
 // (m is read again for the division rather than kept in registers).
 template <int K, typename T, int MAXT>
 __global__ void __launch_bounds__(MAXT, adj_min_ctas(MAXT)) y_adj_kernel(const YAdjArgs a) {
+  chain_wait();
+  chain_release();
   extern __shared__ __align__(16) unsigned char smem[];
   const int W = 1 << a.log2W;
   const int tcol = 1 << a.log2tcol;
@@ -84,7 +86,7 @@ __global__ void __launch_bounds__(MAXT, adj_min_ctas(MAXT)) y_adj_kernel(const Y
 #pragma unroll
     for (int k = 0; k < K; ++k) {
       const T mk = (T)__ldg(a.m + base + k * ld);
-      d[k] = mk * (T)__ldg(a.lam + base + k * ld);
+      d[k] = mk * (T)__ldca(a.lam + base + k * ld);
       s[k] = sc * mk;
     }
   } else {
@@ -92,7 +94,7 @@ __global__ void __launch_bounds__(MAXT, adj_min_ctas(MAXT)) y_adj_kernel(const Y
     for (int k = 0; k < K; ++k) {
       const bool ok = colok && j0 + k < a.ny;
       const T mk = ok ? (T)__ldg(a.m + base + k * ld) : T(1);
-      d[k] = ok ? mk * (T)__ldg(a.lam + base + k * ld) : T(0);
+      d[k] = ok ? mk * (T)__ldca(a.lam + base + k * ld) : T(0);
       s[k] = ok ? sc * mk : T(0);
     }
   }
@@ -109,6 +111,8 @@ __global__ void __launch_bounds__(MAXT, adj_min_ctas(MAXT)) y_adj_kernel(const Y
 // the solve, to keep registers for the solver).
 template <int K, typename T, int MAXT>
 __global__ void __launch_bounds__(MAXT, adj_min_ctas(MAXT)) x_adj_kernel(const XAdjArgs a) {
+  chain_wait();
+  chain_release();
   extern __shared__ __align__(16) unsigned char smem[];
   const int tsys = 1 << a.log2tsys;
   const int tid = threadIdx.x;
@@ -186,6 +190,8 @@ __global__ void __launch_bounds__(MAXT, adj_min_ctas(MAXT)) x_adj_kernel(const X
 // [s: same] at a.stage_off.
 template <int K, int MAXT>
 __global__ void __launch_bounds__(MAXT, adj_min_ctas(MAXT)) x_adj_staged_kernel(const XAdjArgs a) {
+  chain_wait();
+  chain_release();
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int NQ = K / 4;  // float4 groups per thread
   const int threads = blockDim.x;
@@ -208,7 +214,7 @@ __global__ void __launch_bounds__(MAXT, adj_min_ctas(MAXT)) x_adj_staged_kernel(
     if (j < a.ny && col < a.nx) {
       const size_t row = (size_t)j * a.ld;
       m4 = __ldg(reinterpret_cast<const float4*>(a.m + row + col));
-      b4 = __ldg(reinterpret_cast<const float4*>(a.wbar + row + col));
+      b4 = __ldca(reinterpret_cast<const float4*>(a.wbar + row + col));
     }
     const float mv[4] = {m4.x, m4.y, m4.z, m4.w};
     const float wb[4] = {b4.x, b4.y, b4.z, b4.w};
@@ -250,7 +256,7 @@ __global__ void __launch_bounds__(MAXT, adj_min_ctas(MAXT)) x_adj_staged_kernel(
     const size_t row = (size_t)j * a.ld;
     const float4 x4 = sd[swz4(f)];
     const float4 m4 = __ldg(reinterpret_cast<const float4*>(a.m + row + col));
-    const float4 b4 = __ldg(reinterpret_cast<const float4*>(a.wbar + row + col));
+    const float4 b4 = __ldca(reinterpret_cast<const float4*>(a.wbar + row + col));
     const float4 w4 = __ldcs(reinterpret_cast<const float4*>(a.w + row + col));
     const float4 zz = __ldcs(reinterpret_cast<const float4*>(a.z + row + col));
     const float xv[4] = {x4.x, x4.y, x4.z, x4.w};
@@ -295,6 +301,8 @@ __device__ __forceinline__ void st4(float* p, const float (&v)[4]) {
 }
 
 __global__ void __launch_bounds__(256) lam_update_kernel(LamArgs a) {
+  chain_wait();
+  chain_release();
   const int i0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
   const int j = blockIdx.y;
   if (i0 >= a.nx || j >= a.ny) return;
@@ -304,7 +312,7 @@ __global__ void __launch_bounds__(256) lam_update_kernel(LamArgs a) {
   const int q1 = a.resid != nullptr ? __ldg(a.rrow + j + 1) : 0;
   auto prod = [&](size_t at) {
     const float4 m4 = __ldg(reinterpret_cast<const float4*>(a.m + at));
-    const float4 r4 = __ldg(reinterpret_cast<const float4*>(a.rbar + at));
+    const float4 r4 = __ldca(reinterpret_cast<const float4*>(a.rbar + at));
     return make_float4(m4.x * r4.x, m4.y * r4.y, m4.z * r4.z, m4.w * r4.w);
   };
   const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -317,8 +325,8 @@ __global__ void __launch_bounds__(256) lam_update_kernel(LamArgs a) {
 #pragma unroll
   for (int k = 0; k < 4; ++k)
     if (i0 + k >= a.nx) mr[k] = 0.f;
-  const float mL = i0 > 0 ? __ldg(a.m + c - 1) * __ldg(a.rbar + c - 1) : 0.f;
-  const float mR = i0 + 4 < a.nx ? __ldg(a.m + c + 4) * __ldg(a.rbar + c + 4) : 0.f;
+  const float mL = i0 > 0 ? __ldg(a.m + c - 1) * __ldca(a.rbar + c - 1) : 0.f;
+  const float mR = i0 + 4 < a.nx ? __ldg(a.m + c + 4) * __ldca(a.rbar + c + 4) : 0.f;
   const float4 z0 = ld4(a.L0 + c), l1 = ld4(a.L1 + c), l2 = ld4(a.L2 + c);
   const float zb[4] = {z0.x, z0.y, z0.z, z0.w};
   float v1[4] = {l1.x, l1.y, l1.z, l1.w};
@@ -385,12 +393,10 @@ static cudaError_t launch_xa_t(const XAdjArgs& a_in, cudaStream_t st) {
     const size_t sm = align64(tree) + x_stage_bytes(threads, K);
     if (((size_t)K << a.log2tsys) >= (size_t)a.nx && sm <= kAdjSmem) {
       a.stage_off = (int)align64(tree);
-      x_adj_staged_kernel<K, MAXT><<<blocks, threads, sm, st>>>(a);
-      return cudaGetLastError();
+      return launch_chained(x_adj_staged_kernel<K, MAXT>, blocks, threads, sm, st, a);
     }
   }
-  x_adj_kernel<K, T, MAXT><<<blocks, threads, tree, st>>>(a);
-  return cudaGetLastError();
+  return launch_chained(x_adj_kernel<K, T, MAXT>, blocks, threads, tree, st, a);
 }
 
 template <int K, typename T, int MAXT>
@@ -404,13 +410,14 @@ static cudaError_t launch_ya_t(const YAdjArgs& a, cudaStream_t st) {
   cfg.blockDim = dim3(threads, 1, 1);
   cfg.dynamicSmemBytes = y_smem_bytes(W, a.C, 1 << a.log2tcol, sizeof(T) == 8, true);
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
+  attr[1] = chain_attribute();
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = a.C;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, y_adj_kernel<K, T, MAXT>, a);
 }
 
@@ -468,8 +475,7 @@ cudaError_t launch_y_adj(const YAdjArgs& a, int K, bool fp64, cudaStream_t st) {
 
 cudaError_t launch_lam_update(const LamArgs& a, cudaStream_t st) {
   dim3 block(256, 1, 1), grid((a.nx + 1023) / 1024, a.ny, 1);
-  lam_update_kernel<<<grid, block, 0, st>>>(a);
-  return cudaGetLastError();
+  return launch_chained(lam_update_kernel, grid, block, 0, st, a);
 }
 
 cudaError_t launch_seed(float* lam, int ld, const int* rec, int n_rec, const float* resid,

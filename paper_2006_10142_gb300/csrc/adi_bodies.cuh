@@ -52,8 +52,8 @@ __device__ __forceinline__ void x_rows_body(const XArgs& a, int blk, unsigned ch
     }
     load_vec<K>(uc, a.u + row + i0);
     load_vec<K>(v, a.m + row + i0);
-    const float uL = (i0 > 0) ? __ldg(a.u + row + i0 - 1) : 0.f;
-    const float uR = (i0 + K < a.nx) ? __ldg(a.u + row + i0 + K) : 0.f;
+    const float uL = (i0 > 0) ? __ldca(a.u + row + i0 - 1) : 0.f;
+    const float uR = (i0 + K < a.nx) ? __ldca(a.u + row + i0 + K) : 0.f;
     // padding columns (i >= nx) hold zero u and zero m, so r = s = 0 there
 #pragma unroll
     for (int k = 0; k < K; ++k) {
@@ -126,17 +126,17 @@ __device__ __forceinline__ void x_rows_body_staged(const XArgs& a, int blk, unsi
     const size_t row = (size_t)j * a.ld;
     float4 c4 = z4, m4 = z4, v4 = z4, w4 = z4;
     if (ok) {
-      c4 = __ldg(reinterpret_cast<const float4*>(a.u + row + col));
+      c4 = __ldca(reinterpret_cast<const float4*>(a.u + row + col));
       m4 = __ldg(reinterpret_cast<const float4*>(a.m + row + col));
-      if (j > 0) v4 = __ldg(reinterpret_cast<const float4*>(a.u + row - a.ld + col));
-      if (j + 1 < a.ny) w4 = __ldg(reinterpret_cast<const float4*>(a.u + row + a.ld + col));
+      if (j > 0) v4 = __ldca(reinterpret_cast<const float4*>(a.u + row - a.ld + col));
+      if (j + 1 < a.ny) w4 = __ldca(reinterpret_cast<const float4*>(a.u + row + a.ld + col));
     }
     // u at col - 1 and col + 4: the neighbouring lanes' groups (same row
     // whenever the node exists), loaded at the warp's two ends
     float uL = __shfl_up_sync(0xffffffffu, c4.w, 1);
     float uR = __shfl_down_sync(0xffffffffu, c4.x, 1);
-    if (lane == 0) uL = (ok && col > 0) ? __ldg(a.u + row + col - 1) : 0.f;
-    if (lane == 31) uR = (ok && col + 4 < a.nx) ? __ldg(a.u + row + col + 4) : 0.f;
+    if (lane == 0) uL = (ok && col > 0) ? __ldca(a.u + row + col - 1) : 0.f;
+    if (lane == 31) uR = (ok && col + 4 < a.nx) ? __ldca(a.u + row + col + 4) : 0.f;
     if (col == 0) uL = 0.f;
     if (col + 4 >= a.nx) uR = 0.f;
     const float uc[4] = {c4.x, c4.y, c4.z, c4.w};

@@ -1,0 +1,39 @@
+// adi_chain.cuh -- consecutive kernels of a time loop that overlap their
+// launches (programmatic dependent launch).
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace adi {
+
+// Programmatic dependent launch: a kernel launched with launch_chained() may
+// start while the kernel before it is finishing; it touches nothing that
+// kernel writes before chain_wait(), which returns once that kernel (and
+// with it everything before it) has completed.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Launch attribute of a kernel that may overlap the end of the one before it
+// in the stream.  Every such kernel begins with chain_wait().
+inline cudaLaunchAttribute chain_attribute() {
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  return at;
+}
+
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*kern)(P...), dim3 blocks, dim3 threads, size_t smem, cudaStream_t st,
+                           const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = blocks;
+  cfg.blockDim = threads;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1] = {chain_attribute()};
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+}  // namespace adi

@@ -35,6 +35,8 @@ constexpr int min_ctas(int maxt) { return maxt <= 64 ? 8 : maxt <= 128 ? 4 : max
 
 template <int K, typename T, int MAXT, bool TREE>
 __global__ void __launch_bounds__(MAXT, min_ctas(MAXT)) x_sweep_kernel(const XArgs a) {
+  chain_wait();
+  chain_release();
   extern __shared__ __align__(16) unsigned char smem[];
   if constexpr (sizeof(T) == 4) {
     if (a.stage_off >= 0) {
@@ -97,6 +99,8 @@ template <int K, int MAXT, int XC>
 __global__ void __launch_bounds__(MAXT, min_ctas(MAXT))
     x_pipe_kernel(const XArgs a, const __grid_constant__ CUtensorMap tm_u,
                   const __grid_constant__ CUtensorMap tm_m, const __grid_constant__ CUtensorMap tm_w) {
+  chain_wait();
+  chain_release();
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int NQ = K / 4;
   const int tid = threadIdx.x;
@@ -174,9 +178,9 @@ __global__ void __launch_bounds__(MAXT, min_ctas(MAXT))
       const int jr = blk * a.spc + (e >> log2row);
       float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
       if (jr < a.ny && col < a.nx) {
-        if (jr > 0) v = __ldg(reinterpret_cast<const float4*>(a.u + (size_t)(jr - 1) * a.ld + col));
+        if (jr > 0) v = __ldca(reinterpret_cast<const float4*>(a.u + (size_t)(jr - 1) * a.ld + col));
         if (jr + 1 < a.ny) {
-          const float4 t = __ldg(reinterpret_cast<const float4*>(a.u + (size_t)(jr + 1) * a.ld + col));
+          const float4 t = __ldca(reinterpret_cast<const float4*>(a.u + (size_t)(jr + 1) * a.ld + col));
           v.x += t.x; v.y += t.y; v.z += t.z; v.w += t.w;
         }
       }
@@ -223,8 +227,8 @@ __global__ void __launch_bounds__(MAXT, min_ctas(MAXT))
       stage_vec<K>(v, mr, li0);
       // neighbours across the split between the two CTAs of a pair come from L2
       const size_t rowg = (size_t)j * a.ld;
-      const float uL = (i0 > 0) ? (li0 > 0 ? stage_at(ur, li0 - 1) : __ldg(a.u + rowg + i0 - 1)) : 0.f;
-      const float uR = (i0 + K < a.nx) ? (li0 + K < rowf ? stage_at(ur, li0 + K) : __ldg(a.u + rowg + i0 + K)) : 0.f;
+      const float uL = (i0 > 0) ? (li0 > 0 ? stage_at(ur, li0 - 1) : __ldca(a.u + rowg + i0 - 1)) : 0.f;
+      const float uR = (i0 + K < a.nx) ? (li0 + K < rowf ? stage_at(ur, li0 + K) : __ldca(a.u + rowg + i0 + K)) : 0.f;
 #pragma unroll
       for (int k = 0; k < K; ++k) {
         const float c = uc[k];
@@ -503,6 +507,8 @@ template <int K, int MAXT, int XC>
 __global__ void __launch_bounds__(MAXT, min_ctas(MAXT))
     x_band_kernel(const XArgs a, const __grid_constant__ CUtensorMap tm_u,
                   const __grid_constant__ CUtensorMap tm_m, const __grid_constant__ CUtensorMap tm_w) {
+  chain_wait();
+  chain_release();
   static_assert((K == 16 || K == 32) && XC > 1, "band form: K = 16 or 32, rows over a cluster");
   extern __shared__ __align__(16) unsigned char smem[];
   const int tid = threadIdx.x;
@@ -664,6 +670,8 @@ __global__ void __launch_bounds__(MAXT, min_ctas(MAXT))
 // ---------------------------------------------------------------------------
 template <int K, typename T, int MAXT, bool TREE>
 __global__ void __launch_bounds__(MAXT, min_ctas(MAXT)) y_sweep_kernel(const YArgs a) {
+  chain_wait();
+  chain_release();
   extern __shared__ __align__(16) unsigned char smem[];
   const int rank = cluster_rank(a.C);
   if (!a.persist) {
@@ -709,6 +717,8 @@ __global__ void __launch_bounds__(MAXT, min_ctas(MAXT))
     y_pipe_kernel(const YArgs a, const __grid_constant__ CUtensorMap tm_w,
                   const __grid_constant__ CUtensorMap tm_m, const __grid_constant__ CUtensorMap tm_uc,
                   const __grid_constant__ CUtensorMap tm_up) {
+  chain_wait();
+  chain_release();
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int QG = 32 / W;  // row groups (q) per warp
   const int C = a.C;
@@ -884,7 +894,9 @@ __global__ void __launch_bounds__(MAXT, min_ctas(MAXT))
 // ---------------------------------------------------------------------------
 
 // Receiver sampling after a step: traces[s][r] = u^{k}(rec r), s = k - k0 - 1.
-__global__ void gather_kernel(const GridDev* gd, const float* __restrict__ u_new, int ld) {
+__global__ void gather_kernel(const GridDev* gd, const float* u_new, int ld) {
+  chain_wait();
+  chain_release();
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= gd->n_rec) return;
   const long long s = gd->k - gd->k0 - 1;
@@ -1026,8 +1038,7 @@ static cudaError_t launch_x_t(const XArgs& a_in, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     blocks = std::max(1, std::min(blocks, nsm * std::max(per_sm, 1)));
   }
-  x_sweep_kernel<K, T, MAXT, TREE><<<blocks, threads, sm, st>>>(a);
-  return cudaGetLastError();
+  return launch_chained(x_sweep_kernel<K, T, MAXT, TREE>, blocks, threads, sm, st, a);
 }
 
 template <int K, typename T, int MAXT, bool TREE>
@@ -1044,13 +1055,14 @@ static cudaError_t launch_y_t(const YArgs& a_in, cudaStream_t st) {
   cfg.blockDim = dim3(threads, 1, 1);
   cfg.dynamicSmemBytes = ysm + (a.stage_off >= 0 ? y_stage_bytes(threads, K) : 0);
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
+  attr[1] = chain_attribute();
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = a.C;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   if (a.persist) {  // one wave of resident clusters
     int nc = 0;
     cudaError_t e = cudaOccupancyMaxActiveClusters(&nc, y_sweep_kernel<K, T, MAXT, TREE>, &cfg);
@@ -1087,21 +1099,21 @@ static cudaError_t launch_x_pipe_t(const XArgs& a_in, const CUtensorMap& tu, con
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, x_pipe_kernel<K, MAXT, XC>, threads, sm);
     if (e != cudaSuccess) return e;
     const int blocks = std::max(1, std::min(nblk, nsm * std::max(per_sm, 1)));
-    x_pipe_kernel<K, MAXT, XC><<<blocks, threads, sm, st>>>(a, tu, tm, tw);
-    return cudaGetLastError();
+    return launch_chained(x_pipe_kernel<K, MAXT, XC>, blocks, threads, sm, st, a, tu, tm, tw);
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(nblk * XC, 1, 1);
   cfg.blockDim = dim3(threads, 1, 1);
   cfg.dynamicSmemBytes = sm;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
+  attr[1] = chain_attribute();
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = XC;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   int nc = 0;
   cudaError_t e = cudaOccupancyMaxActiveClusters(&nc, x_pipe_kernel<K, MAXT, XC>, &cfg);
   if (e != cudaSuccess) return e;
@@ -1132,13 +1144,14 @@ static cudaError_t launch_x_band_t(const XArgs& a_in, const CUtensorMap& tu, con
   cfg.blockDim = dim3(tsys, 1, 1);
   cfg.dynamicSmemBytes = sm;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
+  attr[1] = chain_attribute();
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = XC;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   int nc = 0;
   cudaError_t e = cudaOccupancyMaxActiveClusters(&nc, x_band_kernel<K, MAXT, XC>, &cfg);
   if (e != cudaSuccess) return e;
@@ -1241,13 +1254,14 @@ static cudaError_t launch_y_pipe_t(const YArgs& a_in, const YMaps& mp, cudaStrea
   cfg.blockDim = dim3(threads, 1, 1);
   cfg.dynamicSmemBytes = sm;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
+  attr[1] = chain_attribute();
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = a.C;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   const bool xa = y_pipe_async_ok(a.C, tcol);
   auto kern = xa ? y_pipe_kernel<K, MAXT, W, ADJ, true> : y_pipe_kernel<K, MAXT, W, ADJ, false>;
   int nc = 0;
@@ -1404,8 +1418,7 @@ cudaError_t launch_gather(const GridDev* gd, const float* u_new, int ld, int n_r
                           cudaStream_t st) {
   if (n_rec <= 0) return cudaSuccess;
   const int threads = 128;
-  gather_kernel<<<(n_rec + threads - 1) / threads, threads, 0, st>>>(gd, u_new, ld);
-  return cudaGetLastError();
+  return launch_chained(gather_kernel, (n_rec + threads - 1) / threads, threads, 0, st, gd, u_new, ld);
 }
 
 __global__ void scan_init_kernel(unsigned int* out3) {

@@ -228,12 +228,11 @@ struct ModelYArgs {
   const float* g;
   int n_g;
   long long level;
-  const GridDev* gd;
+  GridDev* gd;
   int* err;
 };
 cudaError_t launch_x_model(const ModelXArgs& a, int K, cudaStream_t st);
 cudaError_t launch_y_model(const ModelYArgs& a, int K, cudaStream_t st);
-cudaError_t launch_advance_level(GridDev* gd, cudaStream_t st);
 cudaError_t configure_model_kernels();
 // Row tensor map for the pipelined x sweep (see adi_tma.cuh).
 cudaError_t encode_row_map(CUtensorMap* out, const float* base, int ld, int ny, int box_lines);

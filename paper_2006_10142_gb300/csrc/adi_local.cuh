@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "adi_chain.cuh"
 #include "adi_device.cuh"
 #include "adi_internal.h"
 
@@ -104,13 +105,6 @@ __device__ __forceinline__ f2 updated(int i, f2 q, f2 X) {
 }
 
 
-// Programmatic dependent launch: a kernel launched with launch_chained() may
-// start while the kernel before it is finishing; it touches nothing that
-// kernel writes before chain_wait(), which returns once that kernel (and
-// with it everything before it) has completed.
-__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // Receiver sampling inside the step: traces[s][r] = u^{k+1}(rec r), s = k -
 // k0, of the receivers in columns [x0, x1), rows [y0, y1).  find() looks up
 // the thread's first receiver early, so that only the sample itself is left
@@ -142,22 +136,5 @@ struct Sampler {
     }
   }
 };
-
-// Launch that may overlap the end of the kernel before it in the stream (see
-// chain_wait()).
-template <typename... P, typename... A>
-cudaError_t launch_chained(void (*kern)(P...), int blocks, int threads, size_t smem, cudaStream_t st, const A&... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(blocks, 1, 1);
-  cfg.blockDim = dim3(threads, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, args...);
-}
 
 }  // namespace adi

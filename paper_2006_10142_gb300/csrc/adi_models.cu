@@ -19,8 +19,8 @@
 //   samples at k and k + 1.
 // The kernels load their operands directly (no TMA pipeline) and solve with
 // the tree solver of adi_sweeps.cuh: rows in one CTA, columns over a
-// thread-block cluster.  The level k is a kernel argument; the host advances
-// the grid record's level after the step (advance_level_kernel).
+// thread-block cluster.  The level k is a kernel argument; the y pass advances
+// the grid record's level for the receiver sampling.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -44,6 +44,8 @@ __device__ __forceinline__ float wavelet_at(const GridDev* gd, long long k) {
 
 template <int K, int MAXT>
 __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 2 : 1) x_model_kernel(const ModelXArgs a) {
+  chain_wait();
+  chain_release();
   extern __shared__ __align__(16) unsigned char smem[];
   const int tsys = 1 << a.log2tsys;
   const int tid = threadIdx.x;
@@ -60,13 +62,13 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 2 : 1) x_model_kernel(cons
     float A[K], B[K], M[K];
     load_vec<K>(A, a.a + row + i0);
     load_vec<K>(M, a.m + row + i0);
-    const float aL = i0 > 0 ? __ldg(a.a + row + i0 - 1) : 0.f;
-    const float aR = i0 + K < a.nx ? __ldg(a.a + row + i0 + K) : 0.f;
+    const float aL = i0 > 0 ? __ldca(a.a + row + i0 - 1) : 0.f;
+    const float aR = i0 + K < a.nx ? __ldca(a.a + row + i0 + K) : 0.f;
     if (a.mode == 0) {
       // Lap u^k (B) and Lap u^{k-1} (A), both five-point
       load_vec<K>(B, a.b + row + i0);
-      const float bL = i0 > 0 ? __ldg(a.b + row + i0 - 1) : 0.f;
-      const float bR = i0 + K < a.nx ? __ldg(a.b + row + i0 + K) : 0.f;
+      const float bL = i0 > 0 ? __ldca(a.b + row + i0 - 1) : 0.f;
+      const float bR = i0 + K < a.nx ? __ldca(a.b + row + i0 + K) : 0.f;
       float vb[K], va[K];
 #pragma unroll
       for (int k = 0; k < K; ++k) { vb[k] = 0.f; va[k] = 0.f; }
@@ -133,6 +135,8 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 2 : 1) x_model_kernel(cons
 
 template <int K, int MAXT>
 __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 2 : 1) y_model_kernel(const ModelYArgs a) {
+  chain_wait();
+  chain_release();
   extern __shared__ __align__(16) unsigned char smem[];
   const int C = a.C;
   cluster_arrive_early(C);
@@ -156,20 +160,20 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 2 : 1) y_model_kernel(cons
 #pragma unroll
     for (int k = 0; k < K; ++k) {
       const bool ok = colok && j0 + k < a.ny;
-      d[k] = ok ? __ldg(a.w + base + k * ld) : 0.f;
+      d[k] = ok ? __ldca(a.w + base + k * ld) : 0.f;
       s[k] = ok ? sc * gn * __ldg(a.m + base + k * ld) : 0.f;
     }
   } else {
     const float alpha = a.mode == 1 ? 1.f : 0.f;
     const float beta = a.mode == 1 ? 1.f : 2.f;
-    float bprev = (colok && j0 > 0 && j0 - 1 < a.ny) ? __ldg(a.b + base - ld) : 0.f;
-    float bcur = (colok && j0 < a.ny) ? __ldg(a.b + base) : 0.f;
+    float bprev = (colok && j0 > 0 && j0 - 1 < a.ny) ? __ldca(a.b + base - ld) : 0.f;
+    float bcur = (colok && j0 < a.ny) ? __ldca(a.b + base) : 0.f;
 #pragma unroll
     for (int k = 0; k < K; ++k) {
       const bool ok = colok && j0 + k < a.ny;
-      const float bnext = (colok && j0 + k + 1 < a.ny) ? __ldg(a.b + base + (k + 1) * ld) : 0.f;
+      const float bnext = (colok && j0 + k + 1 < a.ny) ? __ldca(a.b + base + (k + 1) * ld) : 0.f;
       const float mk = ok ? __ldg(a.m + base + k * ld) : 0.f;
-      d[k] = ok ? 2.f * __ldg(a.w + base + k * ld) - bcur + alpha * sc * mk * (bprev + bnext - 2.f * bcur) : 0.f;
+      d[k] = ok ? 2.f * __ldca(a.w + base + k * ld) - bcur + alpha * sc * mk * (bprev + bnext - 2.f * bcur) : 0.f;
       s[k] = ok ? beta * sc * mk : 0.f;
       bprev = bcur;
       bcur = bnext;
@@ -184,13 +188,14 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 2 : 1) y_model_kernel(cons
     }
   }
   y_solve_cols<K, float, true>(smem, a.log2W, a.log2tcol, C, rank, 32, col, gq, d, s);
+  if (blockIdx.x == 0 && tid == 0) a.gd->k += 1;  // both passes take the level as an argument
   if (!colok) return;
   float chk = 0.f;
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     if (j0 + k < a.ny) {
       const size_t idx = base + k * ld;
-      const float un = a.mode == 0 ? 2.f * __ldg(a.b + idx) - a.io[idx] + d[k] : d[k];
+      const float un = a.mode == 0 ? 2.f * __ldca(a.b + idx) - a.io[idx] + d[k] : d[k];
       a.io[idx] = un;
       chk += un - un;
     }
@@ -198,15 +203,12 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 2 : 1) y_model_kernel(cons
   if (__any_sync(__activemask(), chk != 0.f) && a.err) atomicOr(a.err, ERR_NUMERIC);
 }
 
-__global__ void advance_level_kernel(GridDev* gd) { gd->k += 1; }
-
 template <int K, int MAXT>
 static cudaError_t launch_xm_t(const ModelXArgs& a, cudaStream_t st) {
   const int threads = a.spc << a.log2tsys;
   if (threads % 32 != 0 || threads > MAXT) return cudaErrorInvalidValue;
   const size_t sm = x_smem_bytes(a.spc, 1 << a.log2tsys, false, true);
-  x_model_kernel<K, MAXT><<<(a.ny + a.spc - 1) / a.spc, threads, sm, st>>>(a);
-  return cudaGetLastError();
+  return launch_chained(x_model_kernel<K, MAXT>, (a.ny + a.spc - 1) / a.spc, threads, sm, st, a);
 }
 
 template <int K, int MAXT>
@@ -219,13 +221,14 @@ static cudaError_t launch_ym_t(const ModelYArgs& a, cudaStream_t st) {
   cfg.blockDim = dim3(threads, 1, 1);
   cfg.dynamicSmemBytes = y_smem_bytes(W, a.C, 1 << a.log2tcol, false, true);
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
+  attr[1] = chain_attribute();
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = a.C;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, y_model_kernel<K, MAXT>, a);
 }
 
@@ -252,11 +255,6 @@ cudaError_t launch_y_model(const ModelYArgs& a, int K, cudaStream_t st) {
   const int threads = 1 << (a.log2W + a.log2tcol);
   ADI_MODEL_DISPATCH(launch_ym_t, threads)
   return cudaErrorInvalidValue;
-}
-
-cudaError_t launch_advance_level(GridDev* gd, cudaStream_t st) {
-  advance_level_kernel<<<1, 1, 0, st>>>(gd);
-  return cudaGetLastError();
 }
 
 template <typename KernT>

@@ -647,7 +647,7 @@ int adi_wave::run(int steps, const adi_source* src, const int32_t* rec_xy, int n
   // gradient is made of differences of nearly equal FP32 fields (z - w), so
   // its last digits follow the rounding of every forward value.
   const bool one_pass = G.plan.tile != 0 && every == 0;
-  const bool use_graph = (one_pass ? tuning.use_graph > 0 : G.plan.graph) && !profile;
+  const bool use_graph = tuning.use_graph > 0 && !profile;
   const size_t fbytes = sizeof(float) * (size_t)G.ld * G.ny;
   int s = 0;
   while (s < steps) {
@@ -873,8 +873,7 @@ int adi_wave::enqueue_model_step(Grid& G, cudaStream_t st, bool gather) {
   ya.err = d_err;
   CK(launch_x_model(xa, P.kx, st), "model x pass");
   CK(launch_y_model(ya, P.ky, st), "model y pass");
-  CK(launch_advance_level(G.gd, st), "advance level");
-  launches += 3;
+  launches += 2;
   if (gather) {
     CK(launch_gather(G.gd, A, G.ld, G.hgd.n_rec, st), "gather launch");
     launches += 1;

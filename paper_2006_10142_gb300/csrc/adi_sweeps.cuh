@@ -17,18 +17,21 @@
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
+#include "adi_chain.cuh"
 #include "adi_device.cuh"
 
 namespace adi {
 
 namespace cgx = cooperative_groups;
 
+// (coherent loads: the field may have been written by the kernel before,
+// which this one may have overlapped up to its chain_wait())
 template <int K>
-__device__ __forceinline__ void load_vec(float (&v)[K], const float* __restrict__ p) {
+__device__ __forceinline__ void load_vec(float (&v)[K], const float* p) {
   const float4* p4 = reinterpret_cast<const float4*>(p);
 #pragma unroll
   for (int q = 0; q < K / 4; ++q) {
-    float4 t = __ldg(p4 + q);
+    float4 t = __ldca(p4 + q);
     v[4 * q + 0] = t.x; v[4 * q + 1] = t.y; v[4 * q + 2] = t.z; v[4 * q + 3] = t.w;
   }
 }
