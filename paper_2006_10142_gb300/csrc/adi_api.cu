@@ -61,7 +61,11 @@ int plan_grid(Grid& G, const adi_wave_tuning& t, std::string& why) {
   P.fp64x = G.fp64mode == ADI_FP64_ALWAYS || (G.fp64mode == ADI_FP64_AUTO && weak_x);
   P.fp64y = G.fp64mode == ADI_FP64_ALWAYS || (G.fp64mode == ADI_FP64_AUTO && weak_y);
   if (t.solver < ADI_SOLVER_AUTO || t.solver > ADI_SOLVER_CR_SMEM) { why = "unknown solver"; return ADI_EINVAL; }
-  P.tree = t.solver != ADI_SOLVER_CR_SMEM;
+  // FP64 in both directions is bound by the FP64 pipe (1/64 of the FP32
+  // rate), where the tree's merges, done by all lanes of a warp at every
+  // level, are work: cyclic reduction in shared memory then (ms at 4096^2, x
+  // and y: tree 1.21 and 1.30, CR 1.00 and 0.71).
+  P.tree = t.solver != ADI_SOLVER_CR_SMEM && !(t.solver == ADI_SOLVER_AUTO && P.fp64x && P.fp64y);
   int pcr = t.pcr_size ? t.pcr_size : 32;
   if (pcr != 2 && pcr != 4 && pcr != 8 && pcr != 16 && pcr != 32) { why = "pcr_size must be 2..32, a power of two"; return ADI_EINVAL; }
   P.pcr = pcr;
@@ -183,6 +187,27 @@ x_done:
       return C <= maxC && (!P.tree || groups <= 32);
     };
     int K = t.chunk_y;
+    const bool y64_auto = P.fp64y && !P.tree && t.solver == ADI_SOLVER_AUTO && cty == 0 && t.chunk_y == 0 &&
+                          t.cols_per_cta == 0;
+    if (y64_auto) {
+      // strips of 8 columns, 16 (32) rows per thread, CTAs of 256 threads (ms
+      // at 2048 x 1500 and 4096^2: 0.202 and 0.76 with 16 rows, 0.71 with 32
+      // at 4096^2; 16 columns and 512 threads 0.44 and 1.30); shorter columns
+      // 8 rows, 128 threads (700^2: 0.045 against 0.102).  The reverse step
+      // solves with the tree, so its top system has to fit as well.
+      W = 8;
+      K = G.ny >= 4096 ? 32 : G.ny >= 1024 ? 16 : 8;
+      auto fits_tree = [&] {
+        int tcol, C;
+        geom(K, tcol, C);
+        return C <= maxC && C * std::max(1, tcol / 32) <= 32;
+      };
+      ymaxT = G.ny >= 1024 ? 256 : 128;
+      while (!fits_tree() && (K < 32 || ymaxT < 512)) {
+        if (K < 32) K *= 2;
+        else ymaxT *= 2;
+      }
+    }
     if (K == 0) {
       K = P.fp64y ? 8 : (G.ny >= 64 ? 8 : 4);
       // prefer portable clusters (<= 8 CTAs) and a top system that fits a warp

@@ -37,10 +37,20 @@ __device__ __forceinline__ float rcp_t(float x) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
-__device__ __forceinline__ double rcp_t(double x) { return 1.0 / x; }
+// 1/x for the eliminations' denominators (finite, 1 and above): the hardware's
+// gross approximation and two Newton steps, r <- r + r (1 - x r), which square
+// its error twice, past the last place of a double.  FP64 runs at 1/64 of the
+// FP32 rate, so the four instructions count: a general division takes twice
+// as many and a branch for the special cases that cannot occur here.
+__device__ __forceinline__ double rcp_t(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  r = fma(fma(-x, r, 1.0), r, r);
+  return fma(fma(-x, r, 1.0), r, r);
+}
 
 __device__ __forceinline__ float div_t(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ double div_t(double a, double b) { return a / b; }
+__device__ __forceinline__ double div_t(double a, double b) { return a * rcp_t(b); }
 
 // One equation a x_{i-1} + b x_i + c x_{i+1} = d of a (reduced) system.
 template <typename T> struct alignas(4 * sizeof(T)) Eq {
