@@ -293,8 +293,13 @@ __global__ void __launch_bounds__(MAXT, adj_min_ctas(MAXT)) x_adj_staged_kernel(
 }
 
 // lam^k += 2 lam^{k+1} + tau^2 Lap(m . rbar) (+ the previous step's receiver
-// residuals);  lam^{k-1} -= lam^{k+1};  lam^{k+1} = 0.  Four nodes of a row
-// per thread (16-byte accesses; nodes past nx keep their values).
+// residuals), over the array that holds it.  That array came in holding the
+// step before's lam^{k+2}: lam^k is minus that until now, and lam^{k-1} is
+// minus this step's lam^{k+1}, which stays where it is for the next step to
+// negate.  So a reverse step reads two lambda fields and writes one (20 B per
+// point; adding into a third field and clearing the first took 32).  Four
+// nodes of a row per thread (16-byte accesses; nodes past nx keep their
+// values).
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ void st4(float* p, const float (&v)[4]) {
   *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
@@ -327,20 +332,16 @@ __global__ void __launch_bounds__(256) lam_update_kernel(LamArgs a) {
     if (i0 + k >= a.nx) mr[k] = 0.f;
   const float mL = i0 > 0 ? __ldg(a.m + c - 1) * __ldca(a.rbar + c - 1) : 0.f;
   const float mR = i0 + 4 < a.nx ? __ldg(a.m + c + 4) * __ldca(a.rbar + c + 4) : 0.f;
-  const float4 z0 = ld4(a.L0 + c), l1 = ld4(a.L1 + c), l2 = ld4(a.L2 + c);
+  const float4 z0 = ld4(a.L0 + c), l1 = ld4(a.L1 + c);
   const float zb[4] = {z0.x, z0.y, z0.z, z0.w};
   float v1[4] = {l1.x, l1.y, l1.z, l1.w};
-  float v2[4] = {l2.x, l2.y, l2.z, l2.w};
-  float v0[4] = {z0.x, z0.y, z0.z, z0.w};
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     if (i0 + k >= a.nx) continue;
     const float l = k > 0 ? mr[k - 1] : mL;
     const float r = k < 3 ? mr[k + 1] : mR;
     const float lap = a.cx * (l + r - 2.f * mr[k]) + a.cy * (dn[k] + up[k] - 2.f * mr[k]);
-    v1[k] += 2.f * zb[k] + lap;
-    v2[k] -= zb[k];
-    v0[k] = 0.f;
+    v1[k] = -v1[k] + (2.f * zb[k] + lap);
   }
   for (int q = q0; q < q1; ++q) {
     const int d = __ldg(a.rix + q) - i0;
@@ -352,8 +353,6 @@ __global__ void __launch_bounds__(256) lam_update_kernel(LamArgs a) {
     }
   }
   st4(a.L1 + c, v1);
-  st4(a.L2 + c, v2);
-  st4(a.L0 + c, v0);
 }
 
 // lam[rec r] += resid[s][r] (receivers may share a node, hence the atomics).

@@ -42,9 +42,8 @@ struct LamArgs {
   int nx, ny, ld;
   const float* m;
   const float* rbar;
-  float* L0;  // lam^{k+1}, read then cleared
-  float* L1;  // lam^k
-  float* L2;  // lam^{k-1}
+  const float* L0;  // lam^{k+1}
+  float* L1;        // in: lam^{k+2} (minus lam^k so far); out: lam^k
   float cx, cy;  // tau^2 / h1^2, tau^2 / h2^2
   // receiver residuals of the previous step (u^k's misfit), added to lam^k
   // at the receiver nodes, or null: the receivers of row j are

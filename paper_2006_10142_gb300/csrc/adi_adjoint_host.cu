@@ -8,8 +8,12 @@
 // the segment backward (adi_adjoint.cu, and y_pipe_kernel's adjoint mode in
 // adi_forward.cu for the column solves).  dJ/dm is summed in FP64 over all
 // reverse steps (a pitched [ny][ld] FP64 field) and copied to the caller's
-// array at the end.  Memory: 2 fields per checkpoint + 2 fields per step of
-// one segment + 7 FP32 work fields + the FP64 sum.
+// array at the end.  The next segment is recomputed on a second stream while
+// the reverse steps of the current one run: the two share nothing but m, and
+// at moderate sizes neither fills the GPU.  Memory: 2 fields per checkpoint
+// + 2 fields per step of two segments (one on large grids
+// or where memory is short) + 6 FP32
+// work fields + the FP64 sum.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -33,7 +37,7 @@ void adi_wave::free_adj_work() {
   cudaFree(aw.wb);
   cudaFree(aw.rb);
   cudaFree(aw.g64);
-  for (int q = 0; q < 3; ++q) cudaFree(aw.L[q]);
+  for (int q = 0; q < 2; ++q) cudaFree(aw.L[q]);
   cudaFree(aw.A);
   cudaFree(aw.B);
   cudaFree(aw.gd);
@@ -41,19 +45,27 @@ void adi_wave::free_adj_work() {
   aw = AdjWork{};
 }
 
-int adi_wave::ensure_adj_work(Grid& G, int E, int n_rec) {
+int adi_wave::ensure_adj_work(Grid& G, int E, int n_rec, int bufs) {
   const size_t fbytes = sizeof(float) * (size_t)G.ld * G.ny;
-  if (aw.fbytes != fbytes || aw.E < E) {
-    free_adj_work();
-    cudaError_t e = cudaMalloc(&aw.wseg, fbytes * E);
-    if (e == cudaSuccess) e = cudaMalloc(&aw.zseg, fbytes * E);
-    if (e == cudaSuccess) e = cudaMalloc(&aw.wb, fbytes);
-    if (e == cudaSuccess) e = cudaMalloc(&aw.rb, fbytes);
-    if (e == cudaSuccess) e = cudaMalloc(&aw.g64, 2 * fbytes);
-    for (int q = 0; q < 3 && e == cudaSuccess; ++q) e = cudaMalloc(&aw.L[q], fbytes);
-    if (e == cudaSuccess) e = cudaMalloc(&aw.A, fbytes);
-    if (e == cudaSuccess) e = cudaMalloc(&aw.B, fbytes);
-    if (e == cudaSuccess) e = cudaMalloc(&aw.gd, sizeof(GridDev));
+  if (aw.fbytes != fbytes || aw.E < E || (aw.bufs < bufs && !aw.one_buf)) {
+    cudaError_t e = cudaSuccess;
+    bool one_buf = false;
+    for (;;) {
+      free_adj_work();
+      e = cudaMalloc(&aw.wseg, fbytes * E * bufs);
+      if (e == cudaSuccess) e = cudaMalloc(&aw.zseg, fbytes * E * bufs);
+      if (e == cudaSuccess) e = cudaMalloc(&aw.wb, fbytes);
+      if (e == cudaSuccess) e = cudaMalloc(&aw.rb, fbytes);
+      if (e == cudaSuccess) e = cudaMalloc(&aw.g64, 2 * fbytes);
+      for (int q = 0; q < 2 && e == cudaSuccess; ++q) e = cudaMalloc(&aw.L[q], fbytes);
+      if (e == cudaSuccess) e = cudaMalloc(&aw.A, fbytes);
+      if (e == cudaSuccess) e = cudaMalloc(&aw.B, fbytes);
+      if (e == cudaSuccess) e = cudaMalloc(&aw.gd, sizeof(GridDev));
+      if (e == cudaSuccess || bufs == 1) break;
+      cudaGetLastError();
+      bufs = 1;  // room for one segment, perhaps
+      one_buf = true;
+    }
     if (e != cudaSuccess) {
       cudaGetLastError();
       free_adj_work();
@@ -61,6 +73,8 @@ int adi_wave::ensure_adj_work(Grid& G, int E, int n_rec) {
     }
     aw.fbytes = fbytes;
     aw.E = E;
+    aw.bufs = bufs;
+    aw.one_buf = one_buf;
   }
   // receivers [n_rec][2], then row offsets [ny + 1], columns [n_rec], indexes [n_rec]
   const int rec_ints = 4 * n_rec + G.ny + 1;
@@ -92,16 +106,24 @@ int adi_wave::adjoint(const float* resid, double* grad_m, float* grad_wavelet, i
   if (!grad_m || (n_rec > 0 && !resid)) return fail(this, ADI_EINVAL, "null gradient or residual");
   Grid& G = g[0];
   const int S = rr.steps, E = rr.every;
-  int rc = ensure_adj_work(G, E, n_rec);
-  if (rc != ADI_OK) return rc;
-  const size_t fbytes = aw.fbytes;
+  const int nck = (S + E - 1) / E;
   const size_t ffl = (size_t)G.ld * G.ny;  // floats per field
+  // Two segment buffers let the next segment be recomputed beside the current
+  // one's reverse steps: up to 2 million points, beyond which a step fills
+  // the GPU by itself.  (There the columns are also short enough for the
+  // cluster form of the y sweep; the other form's segment scratch, y_stage 4,
+  // is one per grid and must not serve both directions at once.)
+  const bool beside = nck > 1 && ffl <= ((size_t)1 << 21) && G.plan.y_stage != ADI_STAGE_COOP;
+  int rc = ensure_adj_work(G, E, n_rec, beside ? 2 : 1);
+  if (rc != ADI_OK) return rc;
+  const int bufs = beside ? aw.bufs : 1;
+  const size_t fbytes = aw.fbytes;
 
   const bool src_on = rr.src.ix >= 0 && rr.src.wavelet != nullptr && rr.src.n_wavelet > 0;
   if (grad_wavelet && rr.src.n_wavelet > 0)
     CKA(cudaMemsetAsync(grad_wavelet, 0, sizeof(float) * (size_t)rr.src.n_wavelet, st),
         "clear grad_wavelet");
-  for (int q = 0; q < 3; ++q) CKA(cudaMemsetAsync(aw.L[q], 0, fbytes, st), "clear lambda");
+  for (int q = 0; q < 2; ++q) CKA(cudaMemsetAsync(aw.L[q], 0, fbytes, st), "clear lambda");
   CKA(cudaMemsetAsync(aw.g64, 0, 2 * fbytes, st), "clear gradient sum");
   // Receivers grouped by row: the residual of step s - 1 is added to lam at
   // the end of reverse step s (lam_update_kernel), that of the last step by
@@ -138,37 +160,70 @@ int adi_wave::adjoint(const float* resid, double* grad_m, float* grad_wavelet, i
 
   const GridPlan& P = G.plan;
   // the column solves of the reverse step take the forward TMA pipeline
-  // when the forward y sweep does (strip maps of m and the three lam fields)
+  // when the forward y sweep does (strip maps of m and the two lam fields)
   const bool ypipe = (P.y_stage == 3 || P.y_stage == 4) && !P.fp64y;
-  CUtensorMap tl_m, tl_L[3];
+  CUtensorMap tl_m, tl_L[2];
   if (ypipe) {
     const int BH = y_pipe_box_rows(1 << P.log2tcol, P.ky);
     const int BW = 1 << P.log2W;
     CKA(encode_strip_map(&tl_m, G.m, G.ld, G.ny, BW, BH), "strip map m");
-    for (int q = 0; q < 3; ++q) CKA(encode_strip_map(&tl_L[q], aw.L[q], G.ld, G.ny, BW, BH), "strip map lambda");
+    for (int q = 0; q < 2; ++q) CKA(encode_strip_map(&tl_L[q], aw.L[q], G.ld, G.ny, BW, BH), "strip map lambda");
   }
   // the row solves of the reverse step stage their rows through shared
   // memory unless the forward x sweep is set to direct loads
   const bool x_adj_staged = P.x_stage != 2;
   float* L0 = aw.L[0];
   float* L1 = aw.L[1];
-  float* L2 = aw.L[2];
-  const int nck = (S + E - 1) / E;
-  for (int c = nck - 1; c >= 0; --c) {
+  cudaStream_t rst = st;
+  if (bufs > 1) {
+    if (!rec_st) {
+      CKA(cudaStreamCreateWithFlags(&rec_st, cudaStreamNonBlocking), "create recomputation stream");
+      CKA(cudaEventCreateWithFlags(&fork_adj, cudaEventDisableTiming), "create event");
+      for (int b = 0; b < 2; ++b) {
+        CKA(cudaEventCreateWithFlags(&rev_ev[b], cudaEventDisableTiming), "create event");
+        CKA(cudaEventCreateWithFlags(&seg_ev[b], cudaEventDisableTiming), "create event");
+      }
+    }
+    rst = rec_st;
+    CKA(cudaEventRecord(fork_adj, st), "fork");
+    CKA(cudaStreamWaitEvent(rst, fork_adj, 0), "fork");
+  }
+  // restore segment c's checkpoint and recompute it forward on rst
+  auto recompute = [&](int c) -> int {
     const int s0 = c * E;
     const int len = std::min(E, S - s0);
-    // restore the checkpoint and recompute the segment forward
-    CKA(cudaMemcpyAsync(aw.A, rr.ckpt[c], fbytes, cudaMemcpyDeviceToDevice, st), "restore");
-    CKA(cudaMemcpyAsync(aw.B, rr.ckpt[c] + ffl, fbytes, cudaMemcpyDeviceToDevice, st), "restore");
+    const size_t off = ffl * E * (size_t)(c % bufs);
+    // the buffer's last user was segment c + bufs
+    if (bufs > 1 && c + bufs < nck) CKA(cudaStreamWaitEvent(rst, rev_ev[c % bufs], 0), "segment buffer");
+    CKA(cudaMemcpyAsync(aw.A, rr.ckpt[c], fbytes, cudaMemcpyDeviceToDevice, rst), "restore");
+    CKA(cudaMemcpyAsync(aw.B, rr.ckpt[c] + ffl, fbytes, cudaMemcpyDeviceToDevice, rst), "restore");
     hg.k = rr.k0 + s0;
     hg.k0 = hg.k;
-    CKA(cudaMemcpyAsync(aw.gd, &hg, sizeof(GridDev), cudaMemcpyHostToDevice, st), "adjoint state");
+    CKA(launch_put_gd(&aw.gd, &hg, 1, rst), "adjoint state");
     float* cur = aw.B;
     float* prev = aw.A;
     for (int i = 0; i < len; ++i) {
-      rc = launch_fwd(G, cur, prev, aw.wseg + ffl * i, aw.zseg + ffl * i, aw.gd, false, st);
-      if (rc != ADI_OK) return rc;
+      const int rc2 = launch_fwd(G, cur, prev, aw.wseg + off + ffl * i, aw.zseg + off + ffl * i, aw.gd, false, rst);
+      if (rc2 != ADI_OK) return rc2;
       std::swap(cur, prev);
+    }
+    if (bufs > 1) CKA(cudaEventRecord(seg_ev[c % bufs], rst), "segment recomputed");
+    return ADI_OK;
+  };
+  if (nck > 0) {
+    rc = recompute(nck - 1);
+    if (rc != ADI_OK) return rc;
+  }
+  for (int c = nck - 1; c >= 0; --c) {
+    const int s0 = c * E;
+    const int len = std::min(E, S - s0);
+    const size_t off = ffl * E * (size_t)(c % bufs);
+    if (bufs > 1) {
+      CKA(cudaStreamWaitEvent(st, seg_ev[c % bufs], 0), "segment");
+      if (c > 0) {
+        rc = recompute(c - 1);
+        if (rc != ADI_OK) return rc;
+      }
     }
     // reverse steps of the segment
     for (int i = len - 1; i >= 0; --i) {
@@ -183,7 +238,7 @@ int adi_wave::adjoint(const float* resid, double* grad_m, float* grad_wavelet, i
         ya.err = d_err;
         ya.stage_mode = 3;
         ya.persist = 1;
-        const int q = L0 == aw.L[0] ? 0 : L0 == aw.L[1] ? 1 : 2;
+        const int q = L0 == aw.L[0] ? 0 : 1;
         if (P.y_stage == 4) CKA(launch_y_coop_adj(ya, P.ky, G.yc, tl_L[q], tl_m, st), "adjoint y sweep");
         else CKA(launch_y_pipe_adj(ya, P.ky, tl_L[q], tl_m, st), "adjoint y sweep");
       } else {
@@ -197,7 +252,7 @@ int adi_wave::adjoint(const float* resid, double* grad_m, float* grad_wavelet, i
       XAdjArgs xa;
       xa.nx = G.nx; xa.ny = G.ny; xa.ld = G.ld;
       xa.log2tsys = P.log2tsys; xa.spc = P.spc; xa.pcr = P.pcr;
-      xa.m = G.m; xa.wbar = aw.wb; xa.w = aw.wseg + ffl * i; xa.z = aw.zseg + ffl * i;
+      xa.m = G.m; xa.wbar = aw.wb; xa.w = aw.wseg + off + ffl * i; xa.z = aw.zseg + off + ffl * i;
       xa.rbar = aw.rb; xa.g64 = aw.g64; xa.gw = grad_wavelet; xa.level = k;
       xa.sc = G.dt * G.dt / (2.0 * G.hx * G.hx);
       xa.src_scale = G.dt * G.dt / (G.hx * G.hy);
@@ -207,7 +262,7 @@ int adi_wave::adjoint(const float* resid, double* grad_m, float* grad_wavelet, i
       CKA(launch_x_adj(xa, P.kx, P.fp64x, st), "adjoint x sweep");
       LamArgs la;
       la.nx = G.nx; la.ny = G.ny; la.ld = G.ld;
-      la.m = G.m; la.rbar = aw.rb; la.L0 = L0; la.L1 = L1; la.L2 = L2;
+      la.m = G.m; la.rbar = aw.rb; la.L0 = L0; la.L1 = L1;
       la.cx = (float)(G.dt * G.dt / (G.hx * G.hx));
       la.cy = (float)(G.dt * G.dt / (G.hy * G.hy));
       la.resid = (n_rec > 0 && s > 0) ? resid + (size_t)(s - 1) * n_rec : nullptr;
@@ -216,10 +271,13 @@ int adi_wave::adjoint(const float* resid, double* grad_m, float* grad_wavelet, i
       la.rid = d_rid;
       CKA(launch_lam_update(la, st), "adjoint lambda update");
       launches += 3;
-      float* t = L0;
-      L0 = L1;
-      L1 = L2;
-      L2 = t;
+      std::swap(L0, L1);
+    }
+    if (bufs > 1) {
+      CKA(cudaEventRecord(rev_ev[c % bufs], st), "segment reversed");
+    } else if (c > 0) {
+      rc = recompute(c - 1);
+      if (rc != ADI_OK) return rc;
     }
   }
   // the FP64 sum (pitched rows) into the caller's [ny][nx] array

@@ -798,6 +798,12 @@ adi_wave::~adi_wave() {
     if (join_ev[b]) cudaEventDestroy(join_ev[b]);
   }
   if (fork_ev) cudaEventDestroy(fork_ev);
+  if (fork_adj) cudaEventDestroy(fork_adj);
+  for (int b = 0; b < 2; ++b) {
+    if (rev_ev[b]) cudaEventDestroy(rev_ev[b]);
+    if (seg_ev[b]) cudaEventDestroy(seg_ev[b]);
+  }
+  if (rec_st) cudaStreamDestroy(rec_st);
   if (cap) cudaStreamDestroy(cap);
 }
 

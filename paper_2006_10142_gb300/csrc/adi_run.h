@@ -100,12 +100,14 @@ struct ProfRec {
 struct AdjWork {
   size_t fbytes = 0;  // bytes of one pitched field
   int E = 0;          // segment length it was sized for
-  float* wseg = nullptr;  // [E] forward x-sweep results of a segment
-  float* zseg = nullptr;  // [E] forward y-sweep results of a segment
+  bool one_buf = false;  // there was no room for two segments
+  int bufs = 0;       // segments wseg and zseg hold (2: one recomputed while the other is reversed)
+  float* wseg = nullptr;  // [bufs][E] forward x-sweep results of a segment
+  float* zseg = nullptr;  // [bufs][E] forward y-sweep results of a segment
   float* wb = nullptr;    // wbar
   float* rb = nullptr;    // rbar
   double* g64 = nullptr;  // [ny][ld] FP64 sum of the dJ/dm increments
-  float* L[3] = {nullptr, nullptr, nullptr};  // lam^{k+1}, lam^k, lam^{k-1}
+  float* L[2] = {nullptr, nullptr};  // lam^{k+1}, lam^k in turn (see lam_update_kernel)
   float* A = nullptr;     // recompute state
   float* B = nullptr;
   GridDev* gd = nullptr;
@@ -134,6 +136,10 @@ struct adi_wave {
   adi::RunRecord rr;
   adi::Model model;
   adi::AdjWork aw;
+  cudaStream_t rec_st = nullptr;              // the adjoint's recomputation, beside the reverse steps
+  cudaEvent_t fork_adj = nullptr;
+  cudaEvent_t rev_ev[2] = {};                 // per segment buffer: reversed
+  cudaEvent_t seg_ev[2] = {};                 // per segment buffer: recomputed
   bool profile = false;
   std::vector<adi::ProfRec> prof;
   std::vector<cudaEvent_t> ev_pool;
@@ -195,7 +201,7 @@ struct adi_wave {
                  adi::GridDev* gd, bool gather, cudaStream_t st);
   int launch_fwd_tile(adi::Grid& G, const float* u_cur, float* u_prev, adi::GridDev* gd, int par, bool gather,
                       cudaStream_t st);
-  int ensure_adj_work(adi::Grid& G, int E, int n_rec);
+  int ensure_adj_work(adi::Grid& G, int E, int n_rec, int bufs);
   void free_adj_work();
   int launch_pair_graph(adi::Grid& G, cudaStream_t st, bool gather, bool one_pass);
   void drop_graphs();
