@@ -311,12 +311,13 @@ y_done:
   // separate sweeps is set: wherever the couplings of both directions decay
   // below 2^-30 within its halo, the elimination is FP32 and a row fills a
   // TMA box (32 columns).  us per step, sweeps and one pass: 128^2 7.3 and
-  // 6.1, 1024^2 15.5 and 7.5, 2048^2 36.1 and 25.9, 4096^2 137 and 58,
+  // 3.4, 1024^2 15.5 and 7.5, 2048^2 36.1 and 25.9, 4096^2 137 and 58,
   // 16384^2 2063 and 768.  Its steps are launched one by one: consecutive
   // launches overlap, which those on either side of a graph's end do not
   // (1024^2: 7.5 against 9.3 from graphs of two steps).
   P.tile = 0;
   P.tile_rows = 0;
+  P.small_patch = false;
   const bool sweeps_set = t.chunk_x || t.chunk_y || t.rows_per_cta || t.cols_per_cta || t.pcr_size || t.solver ||
                           t.cta_threads || t.cta_threads_y || t.y_stage || t.persist || t.x_stage || t.x_cluster;
   if (!sweeps_set && !P.fp64x && !P.fp64y && G.nx >= 32) {
@@ -326,7 +327,8 @@ y_done:
       if (cudaGetDevice(&dev) != cudaSuccess ||
           cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         nsm = 152;
-      P.tile_rows = tile_band_rows(G.nx, G.ny, P.tile, nsm);
+      P.small_patch = small_patch_strips(G.nx) * ((G.ny + patch_rows(P.tile) - 1) / patch_rows(P.tile)) <= 2 * nsm;
+      P.tile_rows = P.small_patch ? 0 : tile_band_rows(G.nx, G.ny, P.tile, nsm);
     }
   }
   G.plan = P;

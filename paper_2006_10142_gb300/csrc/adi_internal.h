@@ -152,6 +152,7 @@ struct TileArgs {
   int nx, ny, ld;
   int strips;          // set by the launcher
   int band_rows;       // rows of a band, a multiple of 16
+  int small;           // patches of 32 columns instead of 96
   int par;             // which of gd->kf holds the level
   float cx, cy;        // tau^2 / h1^2, tau^2 / h2^2
   float scx, scy;      // tau^2 / (2 h1^2), tau^2 / (2 h2^2)
@@ -177,6 +178,7 @@ cudaError_t configure_tile_kernels();
 // The same step patch by patch (adi_patch.cu).
 int patch_rows(int H);
 int patch_strips(int nx);
+int small_patch_strips(int nx);
 cudaError_t encode_patch_map(CUtensorMap* out, const float* base, int nx, int ld, int ny, bool u);
 cudaError_t launch_patch(const TileArgs& a, int H, const CUtensorMap& u, const CUtensorMap& m, cudaStream_t st);
 cudaError_t configure_patch_kernels();

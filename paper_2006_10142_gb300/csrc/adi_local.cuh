@@ -105,6 +105,38 @@ __device__ __forceinline__ f2 updated(int i, f2 q, f2 X) {
 }
 
 
+// The same elimination of one system in scalar arithmetic, operation for
+// operation: x_k = G x_{k+1} + D.
+struct Elim1 {
+  float p, a, N;
+  __device__ __forceinline__ void begin(float a0, float n0) {
+    p = 1.f;
+    a = a0;
+    N = n0;
+  }
+  __device__ __forceinline__ void add(float s, float d) {
+    const float t = fmaf(2.f, p, -a);
+    a = s * p;
+    N = fmaf(s, N, d * p);
+    p = fmaf(s, t, p);
+  }
+  template <int H>
+  __device__ __forceinline__ void tail(const float (&S)[16], const float (&D)[16]) {
+#pragma unroll
+    for (int k = 16 - H; k < 16; ++k) add(S[k], D[k]);
+  }
+  __device__ __forceinline__ void chunk(float (&S)[16], float (&D)[16]) {
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      add(S[k], D[k]);
+      float r = rcp_t(p);
+      r = fmaf(fmaf(-p, r, 1.f), r, r);
+      S[k] = a * r;
+      D[k] = N * r;
+    }
+  }
+};
+
 // Receiver sampling inside the step: traces[s][r] = u^{k+1}(rec r), s = k -
 // k0, of the receivers in columns [x0, x1), rows [y0, y1).  find() looks up
 // the thread's first receiver early, so that only the sample itself is left

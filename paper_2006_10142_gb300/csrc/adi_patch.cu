@@ -316,10 +316,245 @@ __global__ void __launch_bounds__(kPN, 2)
 }
 
 // ---------------------------------------------------------------------------
+// Small patches: 64 x 64 staged points, 32 columns of its own, one row or
+// column per thread in scalar arithmetic.  On a grid of few patches the time
+// of a step is that of one patch (its two phases, about 3.6 us above, where
+// two warps per scheduler share the issue slots), and here each thread has
+// half the work and an SM half the points: 128^2 3.4 against 6.1 us per step,
+// 512^2 4.5 against 6.1.  The operations on an unknown and the chunks are
+// the same, so with H = 12 the results are too, bit for bit (H = 16 reaches
+// the stage's outermost column, which the two kinds cut elsewhere).  Taken
+// while two per SM hold the grid: 640 x 600 (300 patches) 4.6 against 6.3,
+// 700^2 (396) 7.9 against 7.0.
+// ---------------------------------------------------------------------------
+namespace {
+
+constexpr int kSX = 32;                 // columns of a small patch
+constexpr int kSChunks = (kSX + 2 * kPH) / 16;
+// shared memory: u | m | w | XT[5][64] 8 B | X0[5][64] 4 B | YT[5][32] 8 B | Y0[5][32] 4 B | mbarrier
+constexpr int kSOffM = 2 * kUPanel;
+constexpr int kSOffW = kSOffM + 2 * kMPanel;
+constexpr int kSOffXT = kSOffW + kMPanel;
+constexpr int kSOffX0 = kSOffXT + (kSChunks + 1) * kPR * 8;
+constexpr int kSOffYT = kSOffX0 + (kSChunks + 1) * kPR * 4;
+constexpr int kSOffY0 = kSOffYT + 5 * kSX * 8;
+constexpr int kSOffBar = kSOffY0 + 5 * kSX * 4;
+constexpr int kSmallSmem = kSOffBar + 8 + 1016;  // the base is aligned to 1024
+
+__device__ __forceinline__ float4 lds4f(uint32_t a) {
+  return *reinterpret_cast<const float4*>(__cvta_shared_to_generic(a));
+}
+
+}  // namespace
+
+template <int H>
+__global__ void __launch_bounds__(kPN, 2)
+    small_patch_kernel(const TileArgs a, const __grid_constant__ CUtensorMap tm_u,
+                       const __grid_constant__ CUtensorMap tm_m) {
+  constexpr int PY = kPR - 2 * H;
+  extern __shared__ unsigned char smem_raw[];
+  const uint32_t sa0 = (uint32_t)__cvta_generic_to_shared(smem_raw);
+  const uint32_t sa = (sa0 + 1023u) & ~1023u;
+  unsigned char* smem = smem_raw + (sa - sa0);
+  float2* XT = reinterpret_cast<float2*>(smem + kSOffXT);
+  float* X0 = reinterpret_cast<float*>(smem + kSOffX0);
+  float2* YT = reinterpret_cast<float2*>(smem + kSOffYT);
+  float* Y0 = reinterpret_cast<float*>(smem + kSOffY0);
+  const uint32_t bar = sa + kSOffBar;
+  const int tid = threadIdx.x;
+  const int lane = tid & 31;
+  const int strip = blockIdx.x % a.strips;
+  const int band = blockIdx.x / a.strips;
+  const int r0 = band * PY - H;
+  const int c0 = strip * kSX - kPH;
+
+  if (tid == 0) {
+    mbar_init(bar, 1);
+    mbar_fence_init();
+  }
+  if (tid < kPR) {
+    XT[tid] = make_float2(0.f, 0.f);
+    X0[kSChunks * kPR + tid] = 0.f;
+  } else if (tid < kPR + kSX) {
+    YT[tid - kPR] = make_float2(0.f, 0.f);
+    Y0[4 * kSX + tid - kPR] = 0.f;
+  }
+  __syncthreads();
+  if (tid < 32) {
+    if (lane == 0) mbar_arrive_expect_tx(bar, (uint32_t)(2 * (66 + kPR) * 128));
+    __syncwarp();
+    if (lane < 2) tma_load_2d(sa + kSOffM + (uint32_t)(lane * kMPanel), &tm_m, c0 + 32 * lane, r0, bar);
+    chain_wait();
+    if (lane < 2) tma_load_2d(sa + (uint32_t)(lane * kUPanel), &tm_u, c0 + 32 * lane, r0 - 1, bar);
+  } else {
+    chain_wait();
+  }
+  chain_release();
+
+  // x phase: row xr of the patch, chunk ch
+  const int xr = (tid >> 6) * 16 + (tid & 15);
+  const int ch = (tid >> 4) & 3;
+  auto unit0 = [](int panel, int r, int c) {
+    return (uint32_t)((c >> 1) * panel + r * 128 + (((c & 1) * 64) ^ ((r & 7) << 4)));
+  };
+  const uint32_t pu = sa + unit0(kUPanel, xr, ch), pc = sa + unit0(kUPanel, xr + 1, ch),
+                 pd = sa + unit0(kUPanel, xr + 2, ch), pm = sa + kSOffM + unit0(kMPanel, xr, ch);
+  const uint32_t pL = ch > 0 ? sa + (unit0(kUPanel, xr + 1, ch - 1) ^ 48u) + 12u : sa;
+  const uint32_t pR = ch < kSChunks - 1 ? sa + unit0(kUPanel, xr + 1, ch + 1) : sa;
+  const uint32_t ow = sa + kSOffW + unit0(kMPanel, xr, ch - 1);
+  const int gx0 = c0 + 16 * ch;
+  const float cx = a.cx, cy = a.cy, scx = a.scx, scy = a.scy;
+  int sx = -1, sy = -1;
+  float fsrc = 0.f;
+  const GridDev* gd = a.gd;
+  const long long lev = gd->kf[a.par];
+  if (gd->src_ix >= 0 && gd->wavelet != nullptr && lev >= 0 && lev < gd->n_wavelet) {
+    sx = gd->src_ix;
+    sy = gd->src_iy;
+    fsrc = a.src_scale * gd->wavelet[lev];
+  }
+  if (blockIdx.x == 0 && tid == 0) a.gd->kf[a.par ^ 1] = lev + 1;
+  Sampler rec;
+  if (a.gather) rec.find(gd, lev, c0 + kPH, c0 + kPH + kSX, r0 + H, r0 + H + PY);
+
+  // y phase: chunk yc (a warp) of column `lane`; its rows that are the patch's
+  const int yc = tid >> 5;
+  const bool ythread = tid < 4 * kSX;
+  const int yi = strip * kSX + lane;
+  const bool ok = ythread && yi < a.nx;
+  const int ylo = max(0, H - 16 * yc), yhi = min(16, min(kPR - H - 16 * yc, a.ny - r0 - 16 * yc));
+  const size_t ld = (size_t)a.ld;
+  float* const orow = a.u_prev + ((ptrdiff_t)(r0 + 16 * yc) * (ptrdiff_t)ld + yi);
+
+  bool timed_out = false;
+  if (!mbar_wait_bounded(bar, 0u, 1000000000ull)) timed_out = true;
+  // ---------------- x phase ----------------
+  {
+    float D[16], S[16], c[16];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float4 v = lds4f(pc ^ (16u * q));
+      c[4 * q] = v.x; c[4 * q + 1] = v.y; c[4 * q + 2] = v.z; c[4 * q + 3] = v.w;
+    }
+    const float uL = lds(pL), uR = lds(pR);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float4 t4 = lds4f(pu ^ (16u * q)), b4 = lds4f(pd ^ (16u * q)), m4 = lds4f(pm ^ (16u * q));
+      const float vs[4] = {t4.x + b4.x, t4.y + b4.y, t4.z + b4.z, t4.w + b4.w};
+      const float mv[4] = {m4.x, m4.y, m4.z, m4.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int k = 4 * q + e;
+        const float l = k > 0 ? c[k > 0 ? k - 1 : 0] : uL;
+        const float r = k < 15 ? c[k < 15 ? k + 1 : 15] : uR;
+        const float t1 = fmaf(-2.f, c[k], l + r), t2 = fmaf(-2.f, c[k], vs[e]);
+        D[k] = mv[e] * fmaf(cy, t2, cx * t1);
+        S[k] = scx * mv[e];
+      }
+    }
+    if (r0 + xr == sy && sx >= gx0 && sx < gx0 + 16) {
+#pragma unroll
+      for (int k = 0; k < 16; ++k)
+        if (gx0 + k == sx) D[k] += fsrc;
+    }
+    // the stage's outermost columns lack a neighbour: zero there, as beyond
+    if (ch == 0) { D[0] = 0.f; S[0] = 0.f; }
+    if (ch == kSChunks - 1) { D[15] = 0.f; S[15] = 0.f; }
+    Elim1 e;
+    e.begin(0.f, 0.f);
+    e.tail<H>(S, D);
+    {
+      const float r = rcp_t(e.p);
+      XT[(ch + 1) * kPR + xr] = make_float2(e.a * r, e.N * r);
+    }
+    __syncthreads();
+    {
+      const float2 t = XT[ch * kPR + xr];
+      e.begin(t.x, t.y);
+    }
+    e.chunk(S, D);
+    float x = 0.f;
+#pragma unroll
+    for (int k = H - 1; k >= 0; --k) x = fmaf(S[k], x, D[k]);
+    X0[ch * kPR + xr] = x;
+    __syncthreads();
+    x = X0[(ch + 1) * kPR + xr];
+#pragma unroll
+    for (int k = 15; k >= 0; --k) {
+      x = fmaf(S[k], x, D[k]);
+      D[k] = x;
+    }
+    if (ch >= 1 && ch <= kSChunks - 2) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        *reinterpret_cast<float4*>(__cvta_shared_to_generic(ow ^ (16u * q))) =
+            make_float4(D[4 * q], D[4 * q + 1], D[4 * q + 2], D[4 * q + 3]);
+    }
+  }
+  __syncthreads();
+  // ---------------- y phase ----------------
+  float up[16], D[16], S[16];
+  Elim1 e;
+  if (ythread) {
+    const uint32_t row = (uint32_t)(16 * yc * 128);
+    const uint32_t ym = sa + kSOffM + row + (uint32_t)(((lane + kPH) >> 5) * kMPanel + (((lane + kPH) & 31) << 2));
+    const uint32_t yw = sa + kSOffW + row + (uint32_t)(lane << 2);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) up[i] = ok && i >= ylo && i < yhi ? __ldcg(orow + i * ld) : 0.f;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const uint32_t key = (uint32_t)((i & 7) << 4);
+      S[i] = scy * lds((ym ^ key) + i * 128);
+      D[i] = lds((yw ^ key) + i * 128);
+    }
+    e.begin(0.f, 0.f);
+    e.tail<H>(S, D);
+    const float r = rcp_t(e.p);
+    YT[(yc + 1) * kSX + lane] = make_float2(e.a * r, e.N * r);
+  }
+  __syncthreads();
+  if (ythread) {
+    const float2 t = YT[yc * kSX + lane];
+    e.begin(t.x, t.y);
+    e.chunk(S, D);
+    float x = 0.f;
+#pragma unroll
+    for (int k = H - 1; k >= 0; --k) x = fmaf(S[k], x, D[k]);
+    Y0[yc * kSX + lane] = x;
+    const uint32_t yu = sa + (uint32_t)(16 * yc * 128) +
+                        (uint32_t)(((lane + kPH) >> 5) * kUPanel + (((lane + kPH) & 31) << 2));
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      up[i] = fmaf(2.f, lds((yu ^ (uint32_t)(((i + 1) & 7) << 4)) + (i + 1) * 128), -up[i]);
+  }
+  __syncthreads();
+  float chk = 0.f;
+  if (ythread) {
+    float x = Y0[(yc + 1) * kSX + lane];
+#pragma unroll
+    for (int i = 15; i >= 0; --i) {
+      x = fmaf(S[i], x, D[i]);
+      if (ok && i >= ylo && i < yhi) {
+        const float un = up[i] + x;
+        orow[i * ld] = un;
+        chk = fmaf(un, 0.f, chk);
+      }
+    }
+  }
+  if (__any_sync(0xffffffffu, chk != 0.f) && lane == 0 && a.err) atomicOr(a.err, ERR_NUMERIC);
+  if (timed_out && lane == 0 && a.err) atomicOr(a.err, ERR_TIMEOUT);
+  if (a.gather) {
+    __syncthreads();  // the patch's u^{k+1} is written
+    rec.take(gd, lev, a.u_prev, a.ld, c0 + kPH, c0 + kPH + kSX, r0 + H, r0 + H + PY);
+  }
+}
+
+// ---------------------------------------------------------------------------
 // host
 // ---------------------------------------------------------------------------
 int patch_rows(int H) { return kPR - 2 * H; }
 int patch_strips(int nx) { return (nx + kPX - 1) / kPX; }
+int small_patch_strips(int nx) { return (nx + kSX - 1) / kSX; }
 
 cudaError_t encode_patch_map(CUtensorMap* out, const float* base, int nx, int ld, int ny, bool u) {
   return encode_box_map(out, base, nx, ld, ny, 32, u ? kPR + 2 : kPR, true);
@@ -327,9 +562,14 @@ cudaError_t encode_patch_map(CUtensorMap* out, const float* base, int nx, int ld
 
 cudaError_t launch_patch(const TileArgs& a_in, int H, const CUtensorMap& u, const CUtensorMap& m, cudaStream_t st) {
   TileArgs a = a_in;
-  a.strips = patch_strips(a.nx);
   if (H != 12 && H != 16) return cudaErrorInvalidValue;
   const int bands = (a.ny + patch_rows(H) - 1) / patch_rows(H);
+  if (a.small) {
+    a.strips = small_patch_strips(a.nx);
+    return launch_chained(H == 12 ? small_patch_kernel<12> : small_patch_kernel<16>, a.strips * bands, kPN, kSmallSmem,
+                          st, a, u, m);
+  }
+  a.strips = patch_strips(a.nx);
   return launch_chained(H == 12 ? patch_step_kernel<12> : patch_step_kernel<16>, a.strips * bands, kPN, kPatchSmem, st,
                         a, u, m);
 }
@@ -349,6 +589,10 @@ cudaError_t configure_patch_kernels() {
   ADI_PATCH_CFG(patch_batch_kernel<12>)
   ADI_PATCH_CFG(patch_batch_kernel<16>)
 #undef ADI_PATCH_CFG
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(small_patch_kernel<12>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(small_patch_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmem);
   return e;
 }
 

@@ -59,6 +59,7 @@ TileArgs adi::tile_args(const Grid& G) {
   a.ny = G.ny;
   a.ld = G.ld;
   a.band_rows = G.plan.tile_rows;
+  a.small = G.plan.small_patch ? 1 : 0;
   a.cx = (float)(G.dt * G.dt / (G.hx * G.hx));
   a.cy = (float)(G.dt * G.dt / (G.hy * G.hy));
   a.scx = (float)(G.dt * G.dt / (2.0 * G.hx * G.hx));

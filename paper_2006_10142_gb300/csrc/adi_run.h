@@ -31,6 +31,7 @@ struct GridPlan {
   int x_stage = 2;   // 1: rows staged through shared memory, 2: direct, 3: TMA pipeline
   int xc = 1;        // TMA pipeline: CTAs per row (1 or 2)
   int tile = 0;      // halo of the one-pass step (adi_tile.cu), 0 = separate sweeps
+  bool small_patch = false;  // patches of 32 columns (few patches)
   int tile_rows = 0; // rows per band of the one-pass step, 0 = by patches (adi_patch.cu)
 
   bool operator==(const GridPlan& o) const {
@@ -39,7 +40,7 @@ struct GridPlan {
            C == o.C && fp64y == o.fp64y && graph == o.graph && tree == o.tree &&
            cta_threads == o.cta_threads && cta_threads_y == o.cta_threads_y &&
            y_stage == o.y_stage && persist == o.persist && x_stage == o.x_stage && xc == o.xc &&
-           tile == o.tile && tile_rows == o.tile_rows;
+           tile == o.tile && tile_rows == o.tile_rows && small_patch == o.small_patch;
   }
 };
 

@@ -446,7 +446,7 @@ int tile_halo(double s_max) {
 
 int tile_strips(int nx) { return (nx + kTX - 1) / kTX; }
 
-// Bands or patches, and the rows of a band.  Times in us as measured on 152
+// Bands or patches (of 96 columns), and the rows of a band.  Times in us as measured on 152
 // SMs: a block of a band takes 2.2 alone on its SM and 3.05 beside a second
 // CTA (4096^2 to 16384^2), a wave of two patches per SM 6.3 (7.5 for one
 // wave at 1024^2, 14.1 for two at 1500^2, 25.9 for four at 2048^2, where

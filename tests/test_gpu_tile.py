@@ -28,11 +28,14 @@ def _problem(nx, ny, cfl, seed):
     return m, smooth_state(nx, ny, seed, 1e-2), tau, wav
 
 
-# strips of 224 columns, blocks of 16 rows, bands, the halo of 12 (cfl 0.5)
-# and of 16 (cfl 1); sources at the corners of strips, chunks and blocks
-@pytest.mark.parametrize("nx,ny,src", [(224, 293, (0, 0)), (225, 304, (224, 303)), (448, 160, (223, 16)),
-                                       (449, 161, (224, 15)), (1000, 700, (15, 31)), (671, 1025, (447, 1024)),
-                                       (4096, 17, (239, 8)), (257, 4099, (16, 32))])
+# small patches (32 x 40 points), patches (96 x 40), bands (strips of 224
+# columns, blocks of 16 rows); the halo of 12 (cfl 0.5) and of 16 (cfl 1, 32
+# rows to a patch); sources at the corners of patches, chunks and blocks
+@pytest.mark.parametrize("nx,ny,src", [(32, 40, (31, 39)), (33, 41, (32, 40)), (95, 7, (0, 0)), (224, 293, (0, 0)),
+                                       (225, 304, (32, 40)), (449, 161, (224, 15)),
+                                       (1000, 700, (96, 40)), (671, 1025, (479, 1024)), (2049, 200, (95, 39)),
+                                       (257, 4099, (16, 32)),
+                                       (2305, 2321, (224, 16)), (9000, 1000, (447, 999))])
 @pytest.mark.parametrize("cfl", [0.5, 1.0])
 def test_one_pass_step_matches_sweeps_and_oracle(nx, ny, src, cfl):
     m, phi, tau, wav = _problem(nx, ny, cfl, nx + ny)
@@ -48,9 +51,9 @@ def test_one_pass_step_matches_sweeps_and_oracle(nx, ny, src, cfl):
 def test_one_pass_step_reports_non_finite_values():
     import torch
     from paper_2006_10142_gb300 import api
-    nx, ny = 600, 500
+    nx, ny = 603, 500
     dev = torch.device("cuda:0")
-    h = api.AdiWave(torch.ones(ny, nx, device=dev), torch.zeros(ny, nx, device=dev), 0.5 / 601)
+    h = api.AdiWave(torch.ones(ny, nx, device=dev), torch.zeros(ny, nx, device=dev), 0.5 / 604)
     for j, i in ((0, 0), (ny - 1, nx - 1), (250, 223), (255, 224)):
         bad = torch.zeros(ny, nx, device=dev)
         bad[j, i] = float("inf")
