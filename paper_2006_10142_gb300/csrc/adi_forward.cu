@@ -894,12 +894,12 @@ __global__ void __launch_bounds__(MAXT, min_ctas(MAXT))
 // ---------------------------------------------------------------------------
 
 // Receiver sampling after a step: traces[s][r] = u^{k}(rec r), s = k - k0 - 1.
-__global__ void gather_kernel(const GridDev* gd, const float* u_new, int ld) {
+__global__ void gather_kernel(const GridDev* gd, const float* u_new, int ld, long long lev) {
   chain_wait();
   chain_release();
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= gd->n_rec) return;
-  const long long s = gd->k - gd->k0 - 1;
+  const long long s = (lev < 0 ? gd->k : lev) - gd->k0 - 1;
   if (s < 0 || s >= gd->steps || gd->traces == nullptr) return;
   const int ix = gd->rec[2 * r], iy = gd->rec[2 * r + 1];
   gd->traces[s * gd->n_rec + r] = u_new[(size_t)iy * ld + ix];
@@ -1414,11 +1414,11 @@ cudaError_t configure_kernels() {
   return e;
 }
 
-cudaError_t launch_gather(const GridDev* gd, const float* u_new, int ld, int n_rec,
+cudaError_t launch_gather(const GridDev* gd, const float* u_new, int ld, int n_rec, long long lev,
                           cudaStream_t st) {
   if (n_rec <= 0) return cudaSuccess;
   const int threads = 128;
-  return launch_chained(gather_kernel, (n_rec + threads - 1) / threads, threads, 0, st, gd, u_new, ld);
+  return launch_chained(gather_kernel, (n_rec + threads - 1) / threads, threads, 0, st, gd, u_new, ld, lev);
 }
 
 __global__ void scan_init_kernel(unsigned int* out3) {

@@ -71,7 +71,8 @@ struct YArgs {
 // Launchers (adi_forward.cu).
 cudaError_t launch_x(const XArgs& a, int K, bool fp64, bool tree, cudaStream_t st);
 cudaError_t launch_y(const YArgs& a, int K, bool fp64, bool tree, cudaStream_t st);
-cudaError_t launch_gather(const GridDev* gd, const float* u_new, int ld, int n_rec, cudaStream_t st);
+// lev: the level of u_new, or -1: gd->k
+cudaError_t launch_gather(const GridDev* gd, const float* u_new, int ld, int n_rec, long long lev, cudaStream_t st);
 // Fields between the caller's contiguous rows and the handle's pitched ones
 // (adi_copy.cu): dst0 <- src0 and, if src1 is given, dst1 <- src1; without
 // src1 a given dst1 gets src0 too.  Both launches also write the grid record
@@ -158,7 +159,9 @@ struct TileArgs {
   float scx, scy;      // tau^2 / (2 h1^2), tau^2 / (2 h2^2)
   float src_scale;     // tau^2 / (h1 h2)
   float* u_prev;       // in: u^{k-1}; out: u^{k+1}
-  int gather;          // sample the receivers of gd
+  const float* u_cur;  // u^k, for the receivers
+  const int* rec;      // [n_rec][2] receivers to sample u^k at
+  int n_rec;           // 0 = none
   GridDev* gd;
   int* err;
 };

@@ -50,10 +50,10 @@ constexpr int kPatchSmem = kPOffBar + 8 + 1016;  // the base is aligned to 1024
 
 }  // namespace
 
-// Patch `blk` of one grid.
-template <int H>
+// Patch `blk` of one grid (REC: with receivers).
+template <int H, bool REC>
 __device__ __forceinline__ void patch_body(const TileArgs& a, const CUtensorMap* tm_u, const CUtensorMap* tm_m,
-                                           int blk) {
+                                           int blk, int par, float* u_prev) {
   constexpr int PY = kPR - 2 * H;  // rows of a patch
   extern __shared__ unsigned char smem_raw[];
   const uint32_t sa0 = (uint32_t)__cvta_generic_to_shared(smem_raw);
@@ -84,6 +84,8 @@ __device__ __forceinline__ void patch_body(const TileArgs& a, const CUtensorMap*
     Y0[4 * kPairs + tid - 64] = 0ull;
   }
   __syncthreads();
+  Sampler rec;
+  if (REC && a.n_rec > 0) rec.look(a, c0 + kPH, c0 + kPH + kPX, r0 + H, r0 + H + PY);
   if (tid < 32) {
     if (lane == 0) mbar_arrive_expect_tx(bar, (uint32_t)((kPCols / 32) * (66 + kPR) * 128));
     __syncwarp();
@@ -115,15 +117,14 @@ __device__ __forceinline__ void patch_body(const TileArgs& a, const CUtensorMap*
   int sx = -1, sy = -1;
   float fsrc = 0.f;
   const GridDev* gd = a.gd;
-  const long long lev = gd->kf[a.par];
+  const long long lev = gd->kf[par];
+  if (REC && a.n_rec > 0) rec.sample(a, gd, lev, c0 + kPH, c0 + kPH + kPX, r0 + H, r0 + H + PY);
   if (gd->src_ix >= 0 && gd->wavelet != nullptr && lev >= 0 && lev < gd->n_wavelet) {
     sx = gd->src_ix;
     sy = gd->src_iy;
     fsrc = sg * (a.src_scale * gd->wavelet[lev]);
   }
-  if (blk == 0 && tid == 0) a.gd->kf[a.par ^ 1] = lev + 1;
-  Sampler rec;
-  if (a.gather) rec.find(gd, lev, c0 + kPH, c0 + kPH + kPX, r0 + H, r0 + H + PY);
+  if (blk == 0 && tid == 0) a.gd->kf[par ^ 1] = lev + 1;
 
   // y phase: chunk yc of columns 2 cp, 2 cp + 1; its rows that are the patch's
   const bool ythread = tid < 4 * kPairs;
@@ -132,7 +133,7 @@ __device__ __forceinline__ void patch_body(const TileArgs& a, const CUtensorMap*
   const bool ok0 = ythread && yi < a.nx, ok1 = ythread && yi + 1 < a.nx;
   const int ylo = max(0, H - 16 * yc), yhi = min(16, min(kPR - H - 16 * yc, a.ny - r0 - 16 * yc));
   const size_t ld = (size_t)a.ld;
-  float* const orow = a.u_prev + ((ptrdiff_t)(r0 + 16 * yc) * (ptrdiff_t)ld + yi);
+  float* const orow = u_prev + ((ptrdiff_t)(r0 + 16 * yc) * (ptrdiff_t)ld + yi);
 
   bool timed_out = false;
   if (!mbar_wait_bounded(bar, 0u, 1000000000ull)) timed_out = true;
@@ -290,17 +291,13 @@ __device__ __forceinline__ void patch_body(const TileArgs& a, const CUtensorMap*
     if (__any_sync(0xffffffffu, bad) && lane == 0 && a.err) atomicOr(a.err, ERR_NUMERIC);
     if (timed_out && lane == 0 && a.err) atomicOr(a.err, ERR_TIMEOUT);
   }
-  if (a.gather) {
-    __syncthreads();  // the patch's u^{k+1} is written
-    rec.take(gd, lev, a.u_prev, a.ld, c0 + kPH, c0 + kPH + kPX, r0 + H, r0 + H + PY);
-  }
 }
 
 template <int H>
 __global__ void __launch_bounds__(kPN, 2)
     patch_step_kernel(const TileArgs a, const __grid_constant__ CUtensorMap tm_u,
                       const __grid_constant__ CUtensorMap tm_m) {
-  patch_body<H>(a, &tm_u, &tm_m, blockIdx.x);
+  patch_body<H, true>(a, &tm_u, &tm_m, blockIdx.x, a.par, a.u_prev);
 }
 
 // A step of many grids: items[b] = (grid, patch) of CTA b.
@@ -309,10 +306,8 @@ __global__ void __launch_bounds__(kPN, 2)
     patch_batch_kernel(const BatchTile* __restrict__ tiles, const int2* __restrict__ items, int par) {
   const int2 it = __ldg(items + blockIdx.x);
   const BatchTile& t = tiles[it.x];
-  TileArgs a = t.a;
-  a.par = par;
-  a.u_prev = t.buf[par ^ 1];
-  patch_body<H>(a, &t.u[par], &t.m, it.y);
+  const TileArgs a = t.a;
+  patch_body<H, false>(a, &t.u[par], &t.m, it.y, par, t.buf[par ^ 1]);
 }
 
 // ---------------------------------------------------------------------------
@@ -380,6 +375,8 @@ __global__ void __launch_bounds__(kPN, 2)
     Y0[4 * kSX + tid - kPR] = 0.f;
   }
   __syncthreads();
+  Sampler rec;
+  if (a.n_rec > 0) rec.look(a, c0 + kPH, c0 + kPH + kSX, r0 + H, r0 + H + PY);
   if (tid < 32) {
     if (lane == 0) mbar_arrive_expect_tx(bar, (uint32_t)(2 * (66 + kPR) * 128));
     __syncwarp();
@@ -408,14 +405,13 @@ __global__ void __launch_bounds__(kPN, 2)
   float fsrc = 0.f;
   const GridDev* gd = a.gd;
   const long long lev = gd->kf[a.par];
+  if (a.n_rec > 0) rec.sample(a, gd, lev, c0 + kPH, c0 + kPH + kSX, r0 + H, r0 + H + PY);
   if (gd->src_ix >= 0 && gd->wavelet != nullptr && lev >= 0 && lev < gd->n_wavelet) {
     sx = gd->src_ix;
     sy = gd->src_iy;
     fsrc = a.src_scale * gd->wavelet[lev];
   }
   if (blockIdx.x == 0 && tid == 0) a.gd->kf[a.par ^ 1] = lev + 1;
-  Sampler rec;
-  if (a.gather) rec.find(gd, lev, c0 + kPH, c0 + kPH + kSX, r0 + H, r0 + H + PY);
 
   // y phase: chunk yc (a warp) of column `lane`; its rows that are the patch's
   const int yc = tid >> 5;
@@ -543,10 +539,6 @@ __global__ void __launch_bounds__(kPN, 2)
   }
   if (__any_sync(0xffffffffu, chk != 0.f) && lane == 0 && a.err) atomicOr(a.err, ERR_NUMERIC);
   if (timed_out && lane == 0 && a.err) atomicOr(a.err, ERR_TIMEOUT);
-  if (a.gather) {
-    __syncthreads();  // the patch's u^{k+1} is written
-    rec.take(gd, lev, a.u_prev, a.ld, c0 + kPH, c0 + kPH + kSX, r0 + H, r0 + H + PY);
-  }
 }
 
 // ---------------------------------------------------------------------------

@@ -376,7 +376,8 @@ int adi_wave::enqueue_step(Grid& G, cudaStream_t st, bool gather, bool one_pass)
 }
 
 // The same step as one launch (adi_tile.cu, adi_patch.cu).  par: which level
-// word of gd it reads (it leaves the next level in the other one).
+// word of gd it reads (it leaves the next level in the other one).  gather:
+// sample u_cur at the run's receivers.
 int adi_wave::launch_fwd_tile(Grid& G, const float* u_cur, float* u_prev, GridDev* gd, int par, bool gather,
                               cudaStream_t st) {
   const bool patch = G.plan.tile_rows == 0;
@@ -407,7 +408,9 @@ int adi_wave::launch_fwd_tile(Grid& G, const float* u_cur, float* u_prev, GridDe
   TileArgs a = tile_args(G);
   a.par = par;
   a.u_prev = u_prev;
-  a.gather = gather ? 1 : 0;
+  a.u_cur = u_cur;
+  a.rec = gather ? d_rec : nullptr;
+  a.n_rec = gather ? G.hgd.n_rec : 0;
   a.gd = gd;
   a.err = d_err;
   cudaEvent_t ev = nullptr;
@@ -522,7 +525,7 @@ int adi_wave::launch_fwd(Grid& G, const float* u_cur, float* u_prev, float* w, f
   if (profile && prof_end(st, a, ADI_KERNEL_Y) != ADI_OK) return ADI_ECUDA;
   launches += 2;
   if (gather) {
-    CK(launch_gather(gd, u_prev, G.ld, G.hgd.n_rec, st), "gather launch");
+    CK(launch_gather(gd, u_prev, G.ld, G.hgd.n_rec, -1, st), "gather launch");
     launches += 1;
   }
   return ADI_OK;
@@ -643,6 +646,11 @@ int adi_wave::run(int steps, const adi_source* src, const int32_t* rec_xy, int n
   }
 
   const bool gather = n_rec > 0;
+  if (gather && (n_rec != graph_rec || d_rec != graph_rec_at)) {  // captured steps hold both
+    drop_graphs();
+    graph_rec = n_rec;
+    graph_rec_at = d_rec;
+  }
   // A run that keeps checkpoints is one to be differentiated: its steps are
   // the separate sweeps, whose w and z the reverse sweep recomputes.  The
   // gradient is made of differences of nearly equal FP32 fields (z - w), so
@@ -683,6 +691,10 @@ int adi_wave::run(int steps, const adi_source* src, const int32_t* rec_xy, int n
       t += 1;
     }
     s += seg;
+  }
+  if (one_pass && gather) {  // the steps have sampled the levels before the last
+    CK(launch_gather(G.gd, G.buf[G.cur], G.ld, n_rec, G.k, st), "gather launch");
+    launches += 1;
   }
   G.hgd.k = G.k;
   return ADI_OK;
@@ -882,7 +894,7 @@ int adi_wave::enqueue_model_step(Grid& G, cudaStream_t st, bool gather) {
   CK(launch_y_model(ya, P.ky, st), "model y pass");
   launches += 2;
   if (gather) {
-    CK(launch_gather(G.gd, A, G.ld, G.hgd.n_rec, st), "gather launch");
+    CK(launch_gather(G.gd, A, G.ld, G.hgd.n_rec, -1, st), "gather launch");
     launches += 1;
   }
   if (mode == ADI_SCHEME_FACTORED) {

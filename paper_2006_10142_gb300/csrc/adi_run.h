@@ -133,6 +133,8 @@ struct adi_wave {
   cudaStream_t cap = nullptr;  // private stream used only for graph capture
   cudaGraphExec_t pair[2][4] = {};  // [orientation][gather + 2 one_pass]
   adi_wave_tuning tuning = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+  int graph_rec = 0;                // receivers the captured steps sample ...
+  const int* graph_rec_at = nullptr;  // ... and their list
   int ckpt_every = 0;
   adi::RunRecord rr;
   adi::Model model;

@@ -81,10 +81,10 @@ struct Col {
 
 }  // namespace
 
-// CTA `blk` of one grid.
-template <int H>
+// CTA `blk` of one grid (REC: with receivers).
+template <int H, bool REC>
 __device__ __forceinline__ void tile_body(const TileArgs& a, const CUtensorMap* tm_u, const CUtensorMap* tm_m,
-                                          const CUtensorMap* tm_p, const CUtensorMap* tm_o, int blk) {
+                                          const CUtensorMap* tm_p, const CUtensorMap* tm_o, int blk, int par, float* u_prev) {
   extern __shared__ unsigned char smem_raw[];
   const uint32_t sa0 = (uint32_t)__cvta_generic_to_shared(smem_raw);
   const uint32_t sa = (sa0 + 1023u) & ~1023u;
@@ -137,6 +137,8 @@ __device__ __forceinline__ void tile_body(const TileArgs& a, const CUtensorMap* 
     mbar_arrive_expect_tx(bar + 16u, (uint32_t)kOut);
     tma_load_2d(sa + (uint32_t)kOffP, tm_p, strip * kTX, rs + kTB * b, bar + 16u);
   };
+  Sampler rec;
+  if (REC && a.n_rec > 0) rec.look(a, strip * kTX, strip * kTX + kTX, y0, y1);
   chain_wait();
   chain_release();
   if (tid < 32) {
@@ -168,15 +170,17 @@ __device__ __forceinline__ void tile_body(const TileArgs& a, const CUtensorMap* 
   int sx = -1, sy = -1;
   float fsrc = 0.f;
   const GridDev* gd = a.gd;
-  const long long lev = gd->kf[a.par];
+  const long long lev = gd->kf[par];
+  if (REC && a.n_rec > 0) rec.sample(a, gd, lev, strip * kTX, strip * kTX + kTX, y0, y1);
   {
     if (gd->src_ix >= 0 && gd->wavelet != nullptr && lev >= 0 && lev < gd->n_wavelet) {
       sx = gd->src_ix;
       sy = gd->src_iy;
       fsrc = sg * (a.src_scale * gd->wavelet[lev]);
     }
-    if (blk == 0 && tid == 0) a.gd->kf[a.par ^ 1] = lev + 1;
+    if (blk == 0 && tid == 0) a.gd->kf[par ^ 1] = lev + 1;
   }
+
 
   // y phase: columns 2 tid, 2 tid + 1 of the strip, 16 columns into the stage
   const bool ywarp = tid < kTX / 2;
@@ -196,7 +200,7 @@ __device__ __forceinline__ void tile_body(const TileArgs& a, const CUtensorMap* 
   auto store_row = [&](int i, int j, f2 q, f2 X) {
     if (j < y0 || j >= y1) return;
     const f2 un = updated(i, q, X);
-    float* o = a.u_prev + (size_t)j * ld + yi;
+    float* o = u_prev + (size_t)j * ld + yi;
     if (ok0) o[0] = lo2(un);
     if (ok1) o[1] = hi2(un);
     if (ok0) chk = fma2(un, 0ull, chk);
@@ -396,16 +400,7 @@ __device__ __forceinline__ void tile_body(const TileArgs& a, const CUtensorMap* 
   } else if (n > 0) {
     flush(n - 1, A);
   }
-  if (tid < 32) {
-    bulk_wait_all();
-    fence_proxy_async();
-  }
-  if (a.gather) {
-    __syncthreads();  // the strip's u^{k+1} is written
-    Sampler rec;
-    rec.find(gd, lev, strip * kTX, strip * kTX + kTX, y0, y1);
-    rec.take(gd, lev, a.u_prev, a.ld, strip * kTX, strip * kTX + kTX, y0, y1);
-  }
+  if (tid < 32) bulk_wait_all();
   const bool bad = lo2(chk) != 0.f || hi2(chk) != 0.f;
   if (__any_sync(0xffffffffu, bad) && lane == 0 && a.err) atomicOr(a.err, ERR_NUMERIC);
   if (timed_out && lane == 0 && a.err) atomicOr(a.err, ERR_TIMEOUT);
@@ -416,7 +411,7 @@ __global__ void __launch_bounds__(kTN, 2)
     tile_step_kernel(const TileArgs a, const __grid_constant__ CUtensorMap tm_u,
                      const __grid_constant__ CUtensorMap tm_m, const __grid_constant__ CUtensorMap tm_p,
                      const __grid_constant__ CUtensorMap tm_o) {
-  tile_body<H>(a, &tm_u, &tm_m, &tm_p, &tm_o, blockIdx.x);
+  tile_body<H, true>(a, &tm_u, &tm_m, &tm_p, &tm_o, blockIdx.x, a.par, a.u_prev);
 }
 
 // A step of many grids: items[b] = (grid, CTA of that grid) of CTA b.
@@ -425,10 +420,8 @@ __global__ void __launch_bounds__(kTN, 2)
     tile_batch_kernel(const BatchTile* __restrict__ tiles, const int2* __restrict__ items, int par) {
   const int2 it = __ldg(items + blockIdx.x);
   const BatchTile& t = tiles[it.x];
-  TileArgs a = t.a;
-  a.par = par;
-  a.u_prev = t.buf[par ^ 1];
-  tile_body<H>(a, &t.u[par], &t.m, &t.p[par ^ 1], &t.u[par ^ 1], it.y);
+  const TileArgs a = t.a;
+  tile_body<H, false>(a, &t.u[par], &t.m, &t.p[par ^ 1], &t.u[par ^ 1], it.y, par, t.buf[par ^ 1]);
 }
 
 // ---------------------------------------------------------------------------

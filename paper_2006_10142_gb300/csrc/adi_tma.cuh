@@ -66,9 +66,6 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
-// The same for every state space.
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async;" ::: "memory"); }
-
 // Tiled 3D tensor load into this CTA's shared memory at `dst` (1024-byte
 // aligned for the 128-byte swizzle); completes `box bytes` on `bar`.
 // Coordinates are in elements, innermost first; c0 * 4 bytes must be a
