@@ -112,7 +112,7 @@ int adi_wave::setup_batch(cudaStream_t st) {
 
 // One step of one shot by the single-grid kernels, buf[cur] = u^k.
 int adi_wave::launch_batch_fwd(Grid& G, int cur, cudaStream_t st) {
-  return G.plan.tile ? launch_fwd_tile(G, G.buf[cur], G.buf[1 - cur], G.gd, cur, false, st)
+  return G.plan.tile ? launch_fwd_tile(G, G.buf[cur], G.buf[1 - cur], G.gd, cur, false, false, st)
                      : launch_fwd(G, G.buf[cur], G.buf[1 - cur], G.w, nullptr, G.gd, false, st);
 }
 

@@ -15,25 +15,30 @@ __device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.l
 
 // Launch attribute of a kernel that may overlap the end of the one before it
 // in the stream.  Every such kernel begins with chain_wait().
-inline cudaLaunchAttribute chain_attribute() {
+inline cudaLaunchAttribute chain_attribute(bool overlap = true) {
   cudaLaunchAttribute at = {};
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
+  at.val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
   return at;
 }
 
 template <typename... P, typename... A>
-cudaError_t launch_chained(void (*kern)(P...), dim3 blocks, dim3 threads, size_t smem, cudaStream_t st,
-                           const A&... args) {
+cudaError_t launch_after(bool overlap, void (*kern)(P...), dim3 blocks, dim3 threads, size_t smem, cudaStream_t st,
+                         const A&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = blocks;
   cfg.blockDim = threads;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1] = {chain_attribute()};
+  cudaLaunchAttribute attr[1] = {chain_attribute(overlap)};
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*kern)(P...), dim3 blocks, dim3 threads, size_t smem, cudaStream_t st,
+                           const A&... args) {
+  return launch_after(true, kern, blocks, threads, smem, st, args...);
 }
 
 }  // namespace adi

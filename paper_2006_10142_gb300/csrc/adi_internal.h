@@ -159,6 +159,15 @@ struct TileArgs {
   float scx, scy;      // tau^2 / (2 h1^2), tau^2 / (2 h2^2)
   float src_scale;     // tau^2 / (h1 h2)
   float* u_prev;       // in: u^{k-1}; out: u^{k+1}
+  // The step's level and source: by value (level >= 0), so that the wavelet's
+  // sample is fetched before the step before is done, or from gd (level < 0:
+  // captured steps and batches, whose arguments outlive a run).  The first
+  // step of a run waits for all that is before it (alone): the wavelet may be
+  // the work of the caller's last kernel.
+  int alone;
+  long long level;
+  const float* wavelet;
+  int n_wavelet, src_ix, src_iy;
   const float* u_cur;  // u^k, for the receivers
   const int* rec;      // [n_rec][2] receivers to sample u^k at
   int n_rec;           // 0 = none

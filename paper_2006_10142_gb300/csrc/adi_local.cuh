@@ -137,6 +137,31 @@ struct Elim1 {
   }
 };
 
+// tau^2 f^k of a step's point source, f^k = w(t_k) / (h1 h2) at one node, and
+// the level.  early() before chain_wait(), late() behind it.
+struct Source {
+  int sx, sy;
+  float f;
+  long long lev;
+  __device__ __forceinline__ void set(const float* wavelet, int n, int ix, int iy, float scale) {
+    const bool on = ix >= 0 && wavelet != nullptr && lev >= 0 && lev < n;
+    sx = on ? ix : -1;
+    sy = on ? iy : -1;
+    f = on ? scale * wavelet[lev] : 0.f;
+  }
+  __device__ __forceinline__ void early(const TileArgs& a) {
+    lev = a.level;
+    if (a.level >= 0) set(a.wavelet, a.n_wavelet, a.src_ix, a.src_iy, a.src_scale);
+  }
+  // advance: this thread leaves the next level in the record's other word
+  __device__ __forceinline__ void late(const TileArgs& a, int par, bool advance) {
+    if (a.level >= 0) return;
+    lev = a.gd->kf[par];
+    set(a.gd->wavelet, a.gd->n_wavelet, a.gd->src_ix, a.gd->src_iy, a.src_scale);
+    if (advance) a.gd->kf[par ^ 1] = lev + 1;
+  }
+};
+
 // Receiver sampling inside the step that starts from u^k: traces[k - k0 - 1][r]
 // = u^k(rec r) of the receivers in columns [x0, x1), rows [y0, y1).  (The last
 // level of a run is sampled by a launch of its own.)  Sampling the field a

@@ -84,6 +84,8 @@ __device__ __forceinline__ void patch_body(const TileArgs& a, const CUtensorMap*
     Y0[4 * kPairs + tid - 64] = 0ull;
   }
   __syncthreads();
+  Source src;
+  src.early(a);
   Sampler rec;
   if (REC && a.n_rec > 0) rec.look(a, c0 + kPH, c0 + kPH + kPX, r0 + H, r0 + H + PY);
   if (tid < 32) {
@@ -114,17 +116,11 @@ __device__ __forceinline__ void patch_body(const TileArgs& a, const CUtensorMap*
   const float sg = ((xr & 3) == 1 || (xr & 3) == 2) ? -1.f : 1.f;
   const f2 cx2 = dup2(sg * a.cx), cy2 = dup2(sg * a.cy);
   const float scx = a.scx;
-  int sx = -1, sy = -1;
-  float fsrc = 0.f;
+  src.late(a, par, blk == 0 && tid == 0);
   const GridDev* gd = a.gd;
-  const long long lev = gd->kf[par];
-  if (REC && a.n_rec > 0) rec.sample(a, gd, lev, c0 + kPH, c0 + kPH + kPX, r0 + H, r0 + H + PY);
-  if (gd->src_ix >= 0 && gd->wavelet != nullptr && lev >= 0 && lev < gd->n_wavelet) {
-    sx = gd->src_ix;
-    sy = gd->src_iy;
-    fsrc = sg * (a.src_scale * gd->wavelet[lev]);
-  }
-  if (blk == 0 && tid == 0) a.gd->kf[par ^ 1] = lev + 1;
+  const int sx = src.sx, sy = src.sy;
+  const float fsrc = sg * src.f;
+  if (REC && a.n_rec > 0) rec.sample(a, gd, src.lev, c0 + kPH, c0 + kPH + kPX, r0 + H, r0 + H + PY);
 
   // y phase: chunk yc of columns 2 cp, 2 cp + 1; its rows that are the patch's
   const bool ythread = tid < 4 * kPairs;
@@ -375,6 +371,8 @@ __global__ void __launch_bounds__(kPN, 2)
     Y0[4 * kSX + tid - kPR] = 0.f;
   }
   __syncthreads();
+  Source src;
+  src.early(a);
   Sampler rec;
   if (a.n_rec > 0) rec.look(a, c0 + kPH, c0 + kPH + kSX, r0 + H, r0 + H + PY);
   if (tid < 32) {
@@ -401,17 +399,11 @@ __global__ void __launch_bounds__(kPN, 2)
   const uint32_t ow = sa + kSOffW + unit0(kMPanel, xr, ch - 1);
   const int gx0 = c0 + 16 * ch;
   const float cx = a.cx, cy = a.cy, scx = a.scx, scy = a.scy;
-  int sx = -1, sy = -1;
-  float fsrc = 0.f;
+  src.late(a, a.par, blockIdx.x == 0 && tid == 0);
   const GridDev* gd = a.gd;
-  const long long lev = gd->kf[a.par];
-  if (a.n_rec > 0) rec.sample(a, gd, lev, c0 + kPH, c0 + kPH + kSX, r0 + H, r0 + H + PY);
-  if (gd->src_ix >= 0 && gd->wavelet != nullptr && lev >= 0 && lev < gd->n_wavelet) {
-    sx = gd->src_ix;
-    sy = gd->src_iy;
-    fsrc = a.src_scale * gd->wavelet[lev];
-  }
-  if (blockIdx.x == 0 && tid == 0) a.gd->kf[a.par ^ 1] = lev + 1;
+  const int sx = src.sx, sy = src.sy;
+  const float fsrc = src.f;
+  if (a.n_rec > 0) rec.sample(a, gd, src.lev, c0 + kPH, c0 + kPH + kSX, r0 + H, r0 + H + PY);
 
   // y phase: chunk yc (a warp) of column `lane`; its rows that are the patch's
   const int yc = tid >> 5;
@@ -558,11 +550,11 @@ cudaError_t launch_patch(const TileArgs& a_in, int H, const CUtensorMap& u, cons
   const int bands = (a.ny + patch_rows(H) - 1) / patch_rows(H);
   if (a.small) {
     a.strips = small_patch_strips(a.nx);
-    return launch_chained(H == 12 ? small_patch_kernel<12> : small_patch_kernel<16>, a.strips * bands, kPN, kSmallSmem,
+    return launch_after(!a.alone, H == 12 ? small_patch_kernel<12> : small_patch_kernel<16>, a.strips * bands, kPN, kSmallSmem,
                           st, a, u, m);
   }
   a.strips = patch_strips(a.nx);
-  return launch_chained(H == 12 ? patch_step_kernel<12> : patch_step_kernel<16>, a.strips * bands, kPN, kPatchSmem, st,
+  return launch_after(!a.alone, H == 12 ? patch_step_kernel<12> : patch_step_kernel<16>, a.strips * bands, kPN, kPatchSmem, st,
                         a, u, m);
 }
 

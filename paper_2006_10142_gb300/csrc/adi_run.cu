@@ -65,6 +65,7 @@ TileArgs adi::tile_args(const Grid& G) {
   a.scx = (float)(G.dt * G.dt / (2.0 * G.hx * G.hx));
   a.scy = (float)(G.dt * G.dt / (2.0 * G.hy * G.hy));
   a.src_scale = (float)(G.dt * G.dt / (G.hx * G.hy));
+  a.level = -1;
   return a;
 }
 
@@ -366,7 +367,7 @@ int adi_wave::prof_end(cudaStream_t st, cudaEvent_t a, int kind) {
 int adi_wave::enqueue_step(Grid& G, cudaStream_t st, bool gather, bool one_pass) {
   float* u_cur = G.buf[G.cur];
   float* u_prev = G.buf[1 - G.cur];
-  int rc = one_pass ? launch_fwd_tile(G, u_cur, u_prev, G.gd, G.cur, gather, st)
+  int rc = one_pass ? launch_fwd_tile(G, u_cur, u_prev, G.gd, G.cur, gather, st != cap, st)
                     : launch_fwd(G, u_cur, u_prev, G.w, nullptr, G.gd, gather, st);
   if (rc != ADI_OK) return rc;
   G.cur = 1 - G.cur;
@@ -378,8 +379,9 @@ int adi_wave::enqueue_step(Grid& G, cudaStream_t st, bool gather, bool one_pass)
 // The same step as one launch (adi_tile.cu, adi_patch.cu).  par: which level
 // word of gd it reads (it leaves the next level in the other one).  gather:
 // sample u_cur at the run's receivers.
+// by_value: the level and the source travel with the launch (it is not captured).
 int adi_wave::launch_fwd_tile(Grid& G, const float* u_cur, float* u_prev, GridDev* gd, int par, bool gather,
-                              cudaStream_t st) {
+                              bool by_value, cudaStream_t st) {
   const bool patch = G.plan.tile_rows == 0;
   auto encode = [&](CUtensorMap* out, const float* p, bool u) {
     return patch ? encode_patch_map(out, p, G.nx, G.ld, G.ny, u) : encode_tile_map(out, p, G.nx, G.ld, G.ny, false);
@@ -408,6 +410,14 @@ int adi_wave::launch_fwd_tile(Grid& G, const float* u_cur, float* u_prev, GridDe
   TileArgs a = tile_args(G);
   a.par = par;
   a.u_prev = u_prev;
+  if (by_value) {
+    a.level = G.k;
+    a.alone = G.k == G.hgd.k0;
+    a.wavelet = G.hgd.wavelet;
+    a.n_wavelet = G.hgd.n_wavelet;
+    a.src_ix = G.hgd.src_ix;
+    a.src_iy = G.hgd.src_iy;
+  }
   a.u_cur = u_cur;
   a.rec = gather ? d_rec : nullptr;
   a.n_rec = gather ? G.hgd.n_rec : 0;
@@ -614,9 +624,18 @@ int adi_wave::run(int steps, const adi_source* src, const int32_t* rec_xy, int n
   G.hgd.n_rec = n_rec;
   G.hgd.rec = d_rec;
   G.hgd.traces = traces;
-  if (upload_gd(G, st) != ADI_OK) return ADI_ECUDA;
-
   const int every = record ? ckpt_every : 0;
+  // A run that keeps checkpoints is one to be differentiated: its steps are
+  // the separate sweeps, whose w and z the reverse sweep recomputes.  The
+  // gradient is made of differences of nearly equal FP32 fields (z - w), so
+  // its last digits follow the rounding of every forward value.
+  const bool one_pass = G.plan.tile != 0 && every == 0 && !model.active;
+  const bool use_graph = tuning.use_graph > 0 && !profile;
+  // chained one-pass steps carry level and source by value: without receivers
+  // nothing reads the grid record
+  if (!one_pass || use_graph || n_rec > 0)
+    if (upload_gd(G, st) != ADI_OK) return ADI_ECUDA;
+
   if (record) {
     rr.valid = true;
     rr.k0 = G.k;
@@ -651,12 +670,6 @@ int adi_wave::run(int steps, const adi_source* src, const int32_t* rec_xy, int n
     graph_rec = n_rec;
     graph_rec_at = d_rec;
   }
-  // A run that keeps checkpoints is one to be differentiated: its steps are
-  // the separate sweeps, whose w and z the reverse sweep recomputes.  The
-  // gradient is made of differences of nearly equal FP32 fields (z - w), so
-  // its last digits follow the rounding of every forward value.
-  const bool one_pass = G.plan.tile != 0 && every == 0;
-  const bool use_graph = tuning.use_graph > 0 && !profile;
   const size_t fbytes = sizeof(float) * (size_t)G.ld * G.ny;
   int s = 0;
   while (s < steps) {

@@ -203,7 +203,7 @@ struct adi_wave {
   int launch_fwd(adi::Grid& G, const float* u_cur, float* u_prev, float* w, float* z_out,
                  adi::GridDev* gd, bool gather, cudaStream_t st);
   int launch_fwd_tile(adi::Grid& G, const float* u_cur, float* u_prev, adi::GridDev* gd, int par, bool gather,
-                      cudaStream_t st);
+                      bool by_value, cudaStream_t st);
   int ensure_adj_work(adi::Grid& G, int E, int n_rec, int bufs);
   void free_adj_work();
   int launch_pair_graph(adi::Grid& G, cudaStream_t st, bool gather, bool one_pass);

@@ -137,6 +137,8 @@ __device__ __forceinline__ void tile_body(const TileArgs& a, const CUtensorMap* 
     mbar_arrive_expect_tx(bar + 16u, (uint32_t)kOut);
     tma_load_2d(sa + (uint32_t)kOffP, tm_p, strip * kTX, rs + kTB * b, bar + 16u);
   };
+  Source src;
+  src.early(a);
   Sampler rec;
   if (REC && a.n_rec > 0) rec.look(a, strip * kTX, strip * kTX + kTX, y0, y1);
   chain_wait();
@@ -166,21 +168,10 @@ __device__ __forceinline__ void tile_body(const TileArgs& a, const CUtensorMap* 
   const float sg = ((xr & 3) == 1 || (xr & 3) == 2) ? -1.f : 1.f;
   const f2 cx2 = dup2(sg * a.cx), cy2 = dup2(sg * a.cy);
   const float scx = a.scx;
-  // point source f^k = w(t_k) / (h1 h2) at one node
-  int sx = -1, sy = -1;
-  float fsrc = 0.f;
-  const GridDev* gd = a.gd;
-  const long long lev = gd->kf[par];
-  if (REC && a.n_rec > 0) rec.sample(a, gd, lev, strip * kTX, strip * kTX + kTX, y0, y1);
-  {
-    if (gd->src_ix >= 0 && gd->wavelet != nullptr && lev >= 0 && lev < gd->n_wavelet) {
-      sx = gd->src_ix;
-      sy = gd->src_iy;
-      fsrc = sg * (a.src_scale * gd->wavelet[lev]);
-    }
-    if (blk == 0 && tid == 0) a.gd->kf[par ^ 1] = lev + 1;
-  }
-
+  src.late(a, par, blk == 0 && tid == 0);
+  const int sx = src.sx, sy = src.sy;
+  const float fsrc = sg * src.f;
+  if (REC && a.n_rec > 0) rec.sample(a, a.gd, src.lev, strip * kTX, strip * kTX + kTX, y0, y1);
 
   // y phase: columns 2 tid, 2 tid + 1 of the strip, 16 columns into the stage
   const bool ywarp = tid < kTX / 2;
@@ -479,7 +470,7 @@ cudaError_t launch_tile(const TileArgs& a_in, int H, const TileMaps& mp, cudaStr
   a.strips = tile_strips(a.nx);
   if (a.band_rows < kTB || a.band_rows % kTB != 0 || (H != 12 && H != 16)) return cudaErrorInvalidValue;
   const int bands = (a.ny + a.band_rows - 1) / a.band_rows;
-  return launch_chained(H == 12 ? tile_step_kernel<12> : tile_step_kernel<16>, a.strips * bands, kTN, kTileSmem, st,
+  return launch_after(!a.alone, H == 12 ? tile_step_kernel<12> : tile_step_kernel<16>, a.strips * bands, kTN, kTileSmem, st,
                         a, mp.u, mp.m, mp.p, mp.o);
 }
 
