@@ -132,7 +132,7 @@ class AdiWave:
             import numpy as np
             r = np.ascontiguousarray(np.asarray(rec, dtype=np.int32).reshape(-1, 2))
             n_rec = r.shape[0]
-            rec_arr = (ctypes.c_int32 * (2 * n_rec))(*r.ravel().tolist())
+            rec_arr = r.ctypes.data_as(ctypes.POINTER(ctypes.c_int32))
             traces = torch.zeros((steps, n_rec), dtype=torch.float32, device=self.device)
         self._run_keep = [srcs, getattr(self, "_wav_keep", None), traces]
         rc = self._lib.adi_wave_run(self._h, int(steps), srcs, rec_arr, n_rec, _ptr(traces),
