@@ -33,10 +33,27 @@ namespace adi {
 // holds the CTA, so long chunks (K = 16, 32) keep their registers.
 constexpr int min_ctas(int maxt) { return maxt <= 64 ? 8 : maxt <= 128 ? 4 : maxt <= 256 ? 2 : 1; }
 
+// Receiver samples of the level the step starts from, traces[k - k0 - 1][r] =
+// u^k(rec r) (the run's last level by gather_kernel): the receivers dealt out
+// over the CTAs' last warps, while the first warp starts the row loads.  A
+// launch of its own per step took about 2 us of a step of 1024^2.
+__device__ __forceinline__ void x_sample(const XArgs& a) {
+  const int t = (int)threadIdx.x - ((int)blockDim.x - 32);
+  if (a.n_rec <= 0 || t < 0) return;
+  const GridDev* gd = a.gd;
+  for (int r = blockIdx.x + gridDim.x * t; r < a.n_rec; r += 32 * gridDim.x) {
+    const int2 at = __ldg(reinterpret_cast<const int2*>(a.rec) + r);
+    const long long s = gd->k - gd->k0 - 1;
+    if (s < 0 || s >= gd->steps || gd->traces == nullptr) return;
+    gd->traces[s * a.n_rec + r] = __ldcg(a.u + (size_t)at.y * a.ld + at.x);
+  }
+}
+
 template <int K, typename T, int MAXT, bool TREE>
 __global__ void __launch_bounds__(MAXT, min_ctas(MAXT)) x_sweep_kernel(const XArgs a) {
   chain_wait();
   chain_release();
+  x_sample(a);
   extern __shared__ __align__(16) unsigned char smem[];
   if constexpr (sizeof(T) == 4) {
     if (a.stage_off >= 0) {
@@ -101,6 +118,7 @@ __global__ void __launch_bounds__(MAXT, min_ctas(MAXT))
                   const __grid_constant__ CUtensorMap tm_m, const __grid_constant__ CUtensorMap tm_w) {
   chain_wait();
   chain_release();
+  x_sample(a);
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int NQ = K / 4;
   const int tid = threadIdx.x;
@@ -509,6 +527,7 @@ __global__ void __launch_bounds__(MAXT, min_ctas(MAXT))
                   const __grid_constant__ CUtensorMap tm_m, const __grid_constant__ CUtensorMap tm_w) {
   chain_wait();
   chain_release();
+  x_sample(a);
   static_assert((K == 16 || K == 32) && XC > 1, "band form: K = 16 or 32, rows over a cluster");
   extern __shared__ __align__(16) unsigned char smem[];
   const int tid = threadIdx.x;
@@ -893,7 +912,7 @@ __global__ void __launch_bounds__(MAXT, min_ctas(MAXT))
 // small kernels
 // ---------------------------------------------------------------------------
 
-// Receiver sampling after a step: traces[s][r] = u^{k}(rec r), s = k - k0 - 1.
+// Receiver samples of the last level of a run: traces[s][r] = u^k(rec r), s = k - k0 - 1.
 __global__ void gather_kernel(const GridDev* gd, const float* u_new, int ld, long long lev) {
   chain_wait();
   chain_release();

@@ -46,6 +46,8 @@ struct XArgs {
   int stage_off;    // byte offset of the staging area (set by the launcher), -1: none
   int* err;         // device error word (bounded waits), or null
   int xc;           // TMA pipeline: 2 = each row split over a cluster of two CTAs, else 1
+  const int* rec;   // [n_rec][2] receivers at which u^k is sampled into gd's traces
+  int n_rec;        // 0 = none
 };
 
 // Arguments of the y-sweep + update kernel (Eq. fr2's y operator).

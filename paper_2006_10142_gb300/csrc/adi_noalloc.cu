@@ -185,6 +185,8 @@ extern "C" int adi_wave_step_noalloc(const adi_wave_desc* desc, int32_t ld, doub
   xa.stage_off = -1;
   xa.err = nullptr;
   xa.xc = P.xc;
+  xa.rec = nullptr;
+  xa.n_rec = 0;
   YArgs ya;
   ya.nx = d.nx;
   ya.ny = d.ny;

@@ -433,7 +433,7 @@ int adi_wave::launch_fwd_tile(Grid& G, const float* u_cur, float* u_prev, GridDe
 
 // One forward step on explicit buffers: x sweep into w, y sweep + update
 // writing u^{k+1} over u_prev (and z into z_out when given).  gather: sample
-// the receivers of gd.
+// u_cur at the run's receivers.
 int adi_wave::launch_fwd(Grid& G, const float* u_cur, float* u_prev, float* w, float* z_out,
                          GridDev* gd, bool gather, cudaStream_t st) {
   const GridPlan& P = G.plan;
@@ -457,6 +457,8 @@ int adi_wave::launch_fwd(Grid& G, const float* u_cur, float* u_prev, float* w, f
   xa.stage_off = -1;
   xa.err = d_err;
   xa.xc = P.xc;
+  xa.rec = gather ? d_rec : nullptr;
+  xa.n_rec = gather ? G.hgd.n_rec : 0;
   YArgs ya;
   ya.nx = G.nx;
   ya.ny = G.ny;
@@ -534,10 +536,6 @@ int adi_wave::launch_fwd(Grid& G, const float* u_cur, float* u_prev, float* w, f
   }
   if (profile && prof_end(st, a, ADI_KERNEL_Y) != ADI_OK) return ADI_ECUDA;
   launches += 2;
-  if (gather) {
-    CK(launch_gather(gd, u_prev, G.ld, G.hgd.n_rec, -1, st), "gather launch");
-    launches += 1;
-  }
   return ADI_OK;
 }
 
@@ -577,7 +575,7 @@ int adi_wave::launch_pair_graph(Grid& G, cudaStream_t st, bool gather, bool one_
     }
   }
   CK(cudaGraphLaunch(ex, st), "graph launch");
-  launches += one_pass ? 2 : gather ? 6 : 4;
+  launches += one_pass ? 2 : 4;
   G.k += 2;
   return ADI_OK;
 }
@@ -705,7 +703,7 @@ int adi_wave::run(int steps, const adi_source* src, const int32_t* rec_xy, int n
     }
     s += seg;
   }
-  if (one_pass && gather) {  // the steps have sampled the levels before the last
+  if (gather && !model.active) {  // the steps have sampled the levels before the last
     CK(launch_gather(G.gd, G.buf[G.cur], G.ld, n_rec, G.k, st), "gather launch");
     launches += 1;
   }
