@@ -206,20 +206,29 @@ int adi_wave::ensure_batch_tiles() {
   }
   double best = 1.2 + 6.3 * std::max(1.0, std::ceil(patches / slots));
   int best_b = 0;
-  // bands of b blocks: the time of the slot that ends last when the CTAs,
+  // bands of b blocks with their halo: the time of the slot that ends last when the CTAs,
   // longest first, each go to the slot that is free first (even shares alone
   // would choose bands of which a few are left over for a second round: 32
   // shots of 256^2 to 2048^2 174 us per step instead of 130)
-  for (int b = 4; wide && b < 2 * max_blocks; b += std::max(1, b / 6)) {
+  auto band_len = [&](int ny, int rows, int q, int bands) {
+    const int own = std::min(rows, ny - q * rows);
+    return (own + (q > 0 ? bt_h : 0) + (q + 1 < bands ? bt_h : 0) + 15) / 16;
+  };
+  for (int b = 4; wide && b < std::min(2 * max_blocks, 128); ++b) {
+    const int rows = 16 * b - 2 * bt_h;
+    // no schedule ends before the longest CTA or an even share
+    long long total = 0;
+    int longest = 0;
+    for (int s : shots) {
+      const int bands = (g[s].ny + rows - 1) / rows;
+      longest = std::max(longest, band_len(g[s].ny, rows, bands > 2 ? 1 : 0, bands));
+      total += (long long)tile_strips(g[s].nx) * ((g[s].ny + 2 * (bands - 1) * bt_h + 15) / 16);
+    }
+    if (3.5 + 3.05 * std::max((double)longest, total / slots) >= best) continue;
     std::vector<int> lens;
     for (int s : shots) {
-      const int blocks = (g[s].ny + 15) / 16;
-      const int bands = (blocks + b - 1) / b;
-      for (int q = 0; q < bands; ++q) {
-        const int own = std::min(b, blocks - q * b);
-        const int len = own + (q > 0 ? 1 : 0) + (q + 1 < bands ? 1 : 0);
-        lens.insert(lens.end(), tile_strips(g[s].nx), len);
-      }
+      const int bands = (g[s].ny + rows - 1) / rows;
+      for (int q = 0; q < bands; ++q) lens.insert(lens.end(), tile_strips(g[s].nx), band_len(g[s].ny, rows, q, bands));
     }
     std::sort(lens.begin(), lens.end(), std::greater<int>());
     std::priority_queue<int, std::vector<int>, std::greater<int>> ends;
@@ -263,14 +272,12 @@ int adi_wave::ensure_batch_tiles() {
     t.a = tile_args(G);
     t.a.gd = G.gd;
     t.a.err = d_err;
-    t.a.band_rows = bt_patch ? patch_rows(bt_h) : 16 * best_b;
+    t.a.band_rows = bt_patch ? patch_rows(bt_h) : 16 * best_b - 2 * bt_h;
     t.a.strips = bt_patch ? patch_strips(G.nx) : tile_strips(G.nx);
     const int bands = (G.ny + t.a.band_rows - 1) / t.a.band_rows;
     for (int b = 0; b < bands; ++b)
       for (int c = 0; c < t.a.strips; ++c) {
-        const int rows = std::min(t.a.band_rows, G.ny - b * t.a.band_rows);
-        const int len = (rows + 15) / 16 + (b > 0 ? 1 : 0) + (b + 1 < bands ? 1 : 0);
-        items.push_back(Item{bt_patch ? 0 : -len, make_int2((int)tiles.size(), b * t.a.strips + c)});
+        items.push_back(Item{bt_patch ? 0 : -band_len(G.ny, t.a.band_rows, b, bands), make_int2((int)tiles.size(), b * t.a.strips + c)});
       }
     tiles.push_back(t);
   }
