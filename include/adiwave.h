@@ -145,6 +145,8 @@ int adi_wave_run(adi_wave *h, int32_t steps, const adi_source *src,
                  void *stream);
 
 /* Keep (u^{k-1}, u^k) every `every` steps during adi_wave_run (0 = off).
+ * Runs that keep checkpoints take the separate sweeps, whose results the
+ * reverse sweep recomputes; other runs agree with them to rounding.
  * The memory (2 fields per checkpoint) is allocated by the next run. */
 int adi_wave_set_checkpointing(adi_wave *h, int32_t every);
 
@@ -302,10 +304,10 @@ int adi_wave_profile_read(adi_wave *h, double *ms, int64_t *launches,
  * items of a shot wait, bounded, for that shot's x items);
  * mode 1: the plain single-grid kernels (TMA-pipelined where the shape
  * allows) launched once per shot and step, one after the other;
- * mode 2 (default): the same plain kernels, each shot's steps a chain on one
- * of eight streams that fork from and join into the caller's stream
- * (parallel graph branches when replayed), so shots overlap one another's
- * launches and tails.
+ * mode 2 (default): the shots whose step is one launch (see adi_wave_tuning)
+ * advance together, one launch per step for all of them; the other shots'
+ * steps are chains of the plain kernels on eight streams that fork from and
+ * join into the caller's stream.
  * ADI_EINVAL for other modes or single-grid handles. */
 int adi_wave_set_batch_mode(adi_wave *h, int32_t mode);
 
@@ -378,8 +380,8 @@ int adi_wave_set_model(adi_wave *h, const adi_wave_model *model);
  * own pool, or a time loop that must not meet the device-wide
  * synchronisation cudaFree implies or the latency of cudaMalloc.
  *
- * The x sweep's result w, the one intermediate field of a step, lives in a
- * static device array of 4,194,304 floats (16 MiB) that the library sets
+ * The x sweep's result w, the one intermediate field of a step of two
+ * sweeps (a step of one launch has none), lives in a static device array of 4,194,304 floats (16 MiB) that the library sets
  * aside when its module loads, so grids are limited to ld * ny <= 4194304
  * (for example 2048 x 2048); larger grids get ADI_EINVAL and a message
  * from adi_wave_last_error(NULL).  The array needs no initial value.

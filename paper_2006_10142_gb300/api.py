@@ -227,8 +227,9 @@ class AdiWaveBatch:
 
     ``ms``, ``phis`` (and optional ``psis``): lists of float32 CUDA tensors
     [ny_b, nx_b]; ``dts``: tau per shot (a float applies to all).  Each step of
-    all shots is one persistent kernel launch (``mode=0``) or the plain
-    kernels launched per shot (``mode=1``).
+    all shots is one launch (the default, ``mode=2``), one launch of a
+    persistent kernel with separate sweeps (``mode=0``) or the plain kernels
+    launched per shot (``mode=1``).
     """
 
     def __init__(self, ms: Sequence[torch.Tensor], phis: Sequence[torch.Tensor], dts,

@@ -918,7 +918,7 @@ __global__ void gather_kernel(const GridDev* gd, const float* u_new, int ld, lon
   chain_release();
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= gd->n_rec) return;
-  const long long s = (lev < 0 ? gd->k : lev) - gd->k0 - 1;
+  const long long s = (lev == kRecordLevel ? gd->k : lev) - gd->k0 - 1;
   if (s < 0 || s >= gd->steps || gd->traces == nullptr) return;
   const int ix = gd->rec[2 * r], iy = gd->rec[2 * r + 1];
   gd->traces[s * gd->n_rec + r] = u_new[(size_t)iy * ld + ix];

@@ -73,7 +73,8 @@ struct YArgs {
 // Launchers (adi_forward.cu).
 cudaError_t launch_x(const XArgs& a, int K, bool fp64, bool tree, cudaStream_t st);
 cudaError_t launch_y(const YArgs& a, int K, bool fp64, bool tree, cudaStream_t st);
-// lev: the level of u_new, or -1: gd->k
+// lev: the level of u_new, or kRecordLevel: gd->k
+constexpr long long kRecordLevel = -0x7fffffffffffffffll;
 cudaError_t launch_gather(const GridDev* gd, const float* u_new, int ld, int n_rec, long long lev, cudaStream_t st);
 // Fields between the caller's contiguous rows and the handle's pitched ones
 // (adi_copy.cu): dst0 <- src0 and, if src1 is given, dst1 <- src1; without
@@ -154,19 +155,19 @@ cudaError_t configure_y_coop_kernels();
 struct TileArgs {
   int nx, ny, ld;
   int strips;          // set by the launcher
-  int band_rows;       // rows of a band, a multiple of 16
+  int band_rows;       // rows of a band
   int small;           // patches of 32 columns instead of 96
   int par;             // which of gd->kf holds the level
   float cx, cy;        // tau^2 / h1^2, tau^2 / h2^2
   float scx, scy;      // tau^2 / (2 h1^2), tau^2 / (2 h2^2)
   float src_scale;     // tau^2 / (h1 h2)
   float* u_prev;       // in: u^{k-1}; out: u^{k+1}
-  // The step's level and source: by value (level >= 0), so that the wavelet's
-  // sample is fetched before the step before is done, or from gd (level < 0:
+  // The step's level and source: by value, so that the wavelet's
+  // sample is fetched before the step before is done, or from gd (by_value = 0:
   // captured steps and batches, whose arguments outlive a run).  The first
   // step of a run waits for all that is before it (alone): the wavelet may be
   // the work of the caller's last kernel.
-  int alone;
+  int by_value, alone;
   long long level;
   const float* wavelet;
   int n_wavelet, src_ix, src_iy;
@@ -184,7 +185,7 @@ struct TileMaps {
 // the couplings decay too slowly.
 int tile_halo(double s_max);
 int tile_strips(int nx);
-// rows of a band, a multiple of 16, or 0 = by patches
+// rows of a band, or 0 = by patches
 int tile_band_rows(int nx, int ny, int H, int nsm);
 cudaError_t encode_tile_map(CUtensorMap* out, const float* base, int nx, int ld, int ny, bool strip);
 cudaError_t launch_tile(const TileArgs& a, int H, const TileMaps& mp, cudaStream_t st);

@@ -151,11 +151,11 @@ struct Source {
   }
   __device__ __forceinline__ void early(const TileArgs& a) {
     lev = a.level;
-    if (a.level >= 0) set(a.wavelet, a.n_wavelet, a.src_ix, a.src_iy, a.src_scale);
+    if (a.by_value) set(a.wavelet, a.n_wavelet, a.src_ix, a.src_iy, a.src_scale);
   }
   // advance: this thread leaves the next level in the record's other word
   __device__ __forceinline__ void late(const TileArgs& a, int par, bool advance) {
-    if (a.level >= 0) return;
+    if (a.by_value) return;
     lev = a.gd->kf[par];
     set(a.gd->wavelet, a.gd->n_wavelet, a.gd->src_ix, a.gd->src_iy, a.src_scale);
     if (advance) a.gd->kf[par ^ 1] = lev + 1;

@@ -1,8 +1,8 @@
 // adi_noalloc.cu -- adi_wave_step_noalloc: one forward step of the factored
 // scheme on caller-owned buffers that allocates no device memory.
 //
-// A step has one intermediate field, the x sweep's result w (Eq. fr1), and
-// one small device record (GridDev: time level and source) that the sweep
+// A step of two sweeps has one intermediate field, the x sweep's result w
+// (Eq. fr1; a step of one launch has none), and one small device record (GridDev: time level and source) that the sweep
 // kernels read.  Here both live in static device arrays of this translation
 // unit, sized at build time; their addresses are looked up once per device
 // with cudaGetSymbolAddress and handed to the same x / y sweep kernels the

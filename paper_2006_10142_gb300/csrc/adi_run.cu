@@ -65,7 +65,6 @@ TileArgs adi::tile_args(const Grid& G) {
   a.scx = (float)(G.dt * G.dt / (2.0 * G.hx * G.hx));
   a.scy = (float)(G.dt * G.dt / (2.0 * G.hy * G.hy));
   a.src_scale = (float)(G.dt * G.dt / (G.hx * G.hy));
-  a.level = -1;
   return a;
 }
 
@@ -411,6 +410,7 @@ int adi_wave::launch_fwd_tile(Grid& G, const float* u_cur, float* u_prev, GridDe
   a.par = par;
   a.u_prev = u_prev;
   if (by_value) {
+    a.by_value = 1;
     a.level = G.k;
     a.alone = G.k == G.hgd.k0;
     a.wavelet = G.hgd.wavelet;
@@ -905,7 +905,7 @@ int adi_wave::enqueue_model_step(Grid& G, cudaStream_t st, bool gather) {
   CK(launch_y_model(ya, P.ky, st), "model y pass");
   launches += 2;
   if (gather) {
-    CK(launch_gather(G.gd, A, G.ld, G.hgd.n_rec, -1, st), "gather launch");
+    CK(launch_gather(G.gd, A, G.ld, G.hgd.n_rec, kRecordLevel, st), "gather launch");
     launches += 1;
   }
   if (mode == ADI_SCHEME_FACTORED) {

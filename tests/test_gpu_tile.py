@@ -48,6 +48,84 @@ def test_one_pass_step_matches_sweeps_and_oracle(nx, ny, src, cfl):
         assert rel_l2(a[f], o[f]) < 1e-4, f
 
 
+@pytest.mark.parametrize("shapes", [[(2300, 2000, 0.5), (700, 900, 0.5), (224, 300, 1.0)],   # bands
+                                    [(300, 260, 0.5), (33, 41, 0.5), (449, 64, 1.0)],        # patches
+                                    [(300, 260, 0.5), (300, 200, 2.0), (120, 90, 5.0), (17, 40, 0.5),
+                                     (100, 80, 0.5)]])  # with shots that need the sweeps
+def test_batch_in_one_launch_matches_oracle(shapes):
+    import torch
+    from helpers import f32
+    from paper_2006_10142_gb300 import api
+    t = lambda a: torch.from_numpy(f32(a)).to("cuda:0")
+    probs = [_problem(nx, ny, cfl, nx + ny) for nx, ny, cfl in shapes]
+    srcs = [(nx // 3, ny // 2) for nx, ny, _ in shapes]
+    B = api.AdiWaveBatch([t(p[0]) for p in probs], [t(p[1]) for p in probs], [p[2] for p in probs])
+    for n in (STEPS - 1, 1):  # both orientations of the buffers
+        B.run(n, srcs=srcs, wavelets=[t(p[3]) for p in probs])
+    B.sync_status()
+    for b, (m, phi, tau, wav) in enumerate(probs):
+        up, uc, k = B.state(b)
+        o = oracle_run(m, phi, tau, STEPS, src=srcs[b], wavelet=wav)
+        assert k == STEPS + 1
+        assert rel_l2(uc.double().cpu().numpy(), o["u_cur"]) < BOUND, shapes[b]
+        assert rel_l2(up.double().cpu().numpy(), o["u_prev"]) < BOUND, shapes[b]
+    B.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(300, 1100), (40, 4500), (1100, 700)])
+def test_fp64_elimination_of_long_lines_matches_oracle(nx, ny):
+    """The automatic FP64 geometry: 16 and 32 rows per thread over clusters,
+    short columns."""
+    m, phi, tau, wav = _problem(nx, ny, 6.0, nx + ny)
+    a = gpu_run(m, phi, tau, STEPS, src=(nx // 2, ny - 1), wavelet=wav)
+    o = oracle_run(m, phi, tau, STEPS, src=(nx // 2, ny - 1), wavelet=wav)
+    for f in ("u_cur", "u_prev"):
+        assert rel_l2(a[f], o[f]) < BOUND, f
+
+
+def test_noalloc_step_of_two_sweeps_matches_handle():
+    """tau = 2 h / max c: the couplings reach too far for the one-launch step;
+    bit for bit the handle's step, as with it."""
+    import torch
+    from helpers import f32
+    from paper_2006_10142_gb300 import api
+    nx, ny = 300, 200
+    m, phi, tau, wav = _problem(nx, ny, 2.0, 7)
+    dev = torch.device("cuda:0")
+    pit = lambda a: torch.nn.functional.pad(torch.from_numpy(f32(a)), (0, 320 - nx)).contiguous().to(dev)
+    wav = torch.from_numpy(f32(wav)).to(dev)
+    h = api.AdiWave(torch.from_numpy(f32(m)).to(dev), torch.from_numpy(f32(phi)).to(dev), tau)
+    u0, u1, md = pit(phi), pit(phi), pit(m)
+    for k in (1, 2):
+        h.step(src=(9, 9), wavelet=wav)
+        api.step_noalloc(md, u1, u0, nx, tau, float(f32(m).max()), k, src=(9, 9), wavelet=wav)
+        u0, u1 = u1, u0
+    assert torch.equal(h.state()[1], u1[:, :nx])
+    h.close()
+
+
+@pytest.mark.parametrize("tuning", [dict(), dict(use_graph=1)])
+def test_levels_below_zero_have_no_source(tuning):
+    """Levels -2 .. 2: the wavelet starts at level 0; every level is sampled."""
+    import torch
+    from helpers import f32
+    from paper_2006_10142_gb300 import api
+    nx, ny = 300, 260
+    m, phi, tau, wav = _problem(nx, ny, 0.5, 5)
+    t = lambda a: torch.from_numpy(f32(a)).to("cuda:0")
+    out = []
+    for tun in (tuning, dict(solver=1)):
+        h = api.AdiWave(t(m), t(phi), tau)
+        h.set_tuning(**tun)
+        h.set_state(t(phi), t(phi), -2)
+        tr = h.run(5, src=(31, 39), wavelet=t(1e4 * wav + 1e4), rec=[[31, 39], [32, 40], [299, 0]])
+        out.append((tr, h.state()[1]))
+        h.sync_status()
+        h.close()
+    for a, b in zip(*out):
+        assert rel_l2(a.double().cpu().numpy(), b.double().cpu().numpy()) < BOUND
+
+
 def test_one_pass_step_reports_non_finite_values():
     import torch
     from paper_2006_10142_gb300 import api
