@@ -10,18 +10,17 @@ steps, four FP32 fields of 1 GiB each resident (far larger than L2, so no
 flush is needed between steps).
 
 Prints ONE JSON line (rank 0).  `value` is whole-job grid-point updates per
-second over the timed region (the library's own time loop, step pairs
-replayed from CUDA graphs; CUDA events on the launching stream, max over
-ranks).  A second timed region of the same steps records a CUDA event pair
-around every launch (direct launches): `roofline` reports the dominant
+second over the timed region (the library's own time loop; CUDA events on the
+launching stream, max over ranks).  A second timed region of the same steps records a CUDA event pair
+around every launch: `roofline` reports the dominant
 kernel's algorithmic HBM bytes per launch over its average duration there,
 against the measured copy bandwidth.  `e2e` is the same metric from pinned
 host buffers (H2D of m, phi and the wavelet, D2H of the final field inside
 the timed region).  `cpu_baseline` is the FP64 oracle timed on the host cores
 on a bounded sample of the same workload.  The default line also carries an
 `adjoint` sub-record (adjoint_1024: gradient time per time step) and a
-`batch` sub-record (batch_64_shots: one persistent launch per step against
-the plain kernels launched per shot).
+`batch` sub-record (batch_64_shots: one launch per step against the plain
+kernels launched per shot).
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
                   [--workload ricker_16384|ricker_4096|standing_wave_128|
@@ -65,6 +64,7 @@ UNIT = "grid-point updates/s"
 # algorithmic HBM bytes per grid point per launch (FP32 fields)
 BYTES_X = 12  # read u^k, m; write w
 BYTES_Y = 20  # read w, m, u^k, u^{k-1}; write u^{k+1}
+BYTES_STEP = 16  # the one-launch step: read u^k, u^{k-1}, m; write u^{k+1}
 # dram__bytes_read.sum + dram__bytes_write.sum per 16384^2 launch, measured by
 # ncu on a smaller grid with the same launch shape and scaled by the number of
 # grid points (profiles/).  Only valid for the 16384^2 workload and the
@@ -478,15 +478,21 @@ def run_single(ctx, prob):
     tun = h.tuning()
     # the kernels the plan launches: the TMA-pipelined forms (stage 3) or the
     # one-CTA-per-tile forms
+    one_pass = kcnt[2] > 0  # one launch per step instead of two sweeps
     xname = {3: "x_pipe_kernel", 5: "x_band_kernel"}.get(tun.get("x_stage"), "x_sweep_kernel")
     yname = {3: "y_pipe_kernel", 4: "y_coop_kernel"}.get(tun.get("y_stage"), "y_sweep_kernel")
-    roof = _roofline(kms, kcnt, {0: xname, 1: yname}, {0: BYTES_X * pts, 1: BYTES_Y * pts},
-                     args.workload)
-    roof["step_gbs_32B"] = 32.0 * pts * ts * args.steps / (max_ms / 1e3) / 1e9
+    if one_pass:
+        # bands from about 4 million points up, patches below
+        kinds, nbytes = {2: "tile_step_kernel" if pts > 4e6 else "patch_step_kernel"}, BYTES_STEP
+        roof = _roofline(kms, kcnt, kinds, {2: nbytes * pts}, args.workload)
+    else:
+        nbytes = BYTES_X + BYTES_Y
+        roof = _roofline(kms, kcnt, {0: xname, 1: yname}, {0: BYTES_X * pts, 1: BYTES_Y * pts},
+                         args.workload)
+    roof["step_gbs_%dB" % nbytes] = nbytes * pts * ts * args.steps / (max_ms / 1e3) / 1e9
     roof["timed_region"] = ("second timed region of the same K bench steps, a CUDA event pair "
-                            "around every launch (direct launches, no graphs): %.3f ms per bench "
-                            "step against %.3f ms with graphs" % (prof_ms / args.steps,
-                                                                   max_ms / args.steps))
+                            "around every launch: %.3f ms per bench step against %.3f ms without"
+                            % (prof_ms / args.steps, max_ms / args.steps))
 
     e2e = None
     if not args.no_e2e:
@@ -507,7 +513,8 @@ def run_single(ctx, prob):
                        "l2": ("inputs larger than L2 (4 FP32 fields of %.0f MiB)" % (pts * 4 / 2**20)
                               if pts * 16 > 2 * 129e6 else "inputs smaller than L2: no flush, "
                               "steps of one run reuse L2-resident fields"),
-                       "timed_launches": "adi_wave_run: step pairs replayed from CUDA graphs",
+                       "timed_launches": "adi_wave_run: chained launches, %s per step"
+                                         % ("one" if one_pass else "two"),
                        "e2e_copies": "per bench step: H2D of m, phi, wavelet from pinned host memory "
                                      "(torch copy_ on a copy stream into a second device set) and "
                                      "D2H of u^{S+1}, overlapping the neighbouring steps' compute; "
@@ -588,9 +595,8 @@ def _e2e(ctx, h, prob, m_d, phi_d, wav_d):
 
 def run_batch(ctx, steps=None):
     """64 shots with n from {256, 512, 1024, 2048} in the default batch mode
-    (per-shot chains of the single-grid kernels on parallel graph branches);
-    the one-launch persistent kernel and the serial per-shot launches are timed
-    beside it."""
+    (a step of all shots in one launch); the persistent kernel with sweeps
+    (mode 0) and the serial per-shot launches (mode 1) are timed beside it."""
     import torch
     from paper_2006_10142_gb300 import api, inputs, shard
     args, world, rank, dev = ctx["args"], ctx["world"], ctx["rank"], ctx["dev"]
@@ -618,15 +624,14 @@ def run_batch(ctx, steps=None):
     B.sync_status()
     max_ms, _, launches, clk = _timed(ctx, bench_step, B.launch_count, steps=K)
     B.sync_status()
-    # the shots' kernels run concurrently, so a per-launch duration says
-    # little: the roofline here is the whole batched step's (all shots' x and
-    # y sweeps, 32 algorithmic bytes per point) over the wall time
+    # the roofline of the whole batched step (one launch for all shots, 16
+    # algorithmic bytes per point) over the wall time
     peak, peak_kind = measured_peak_gbs()
-    ach = 32.0 * pts_all * ts * K / (max_ms / 1e3) / 1e9
-    roof = {"bound": "hbm", "kernel": "batched step (every shot's x and y sweeps)",
+    ach = BYTES_STEP * pts_all * ts * K / (max_ms / 1e3) / 1e9
+    roof = {"bound": "hbm", "kernel": "tile_batch_kernel (a step of every shot)",
             "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak,
             "peak_source": peak_kind, "traffic": None,
-            "alg_bytes_per_step": 32 * pts_all, "timed_region": "wall time of the timed region"}
+            "alg_bytes_per_step": BYTES_STEP * pts_all, "timed_region": "wall time of the timed region"}
     # the same work in the other batch modes: the one-launch persistent
     # kernel (mode 0) and the plain kernels launched serially per shot (mode 1)
     other = {}
@@ -648,9 +653,7 @@ def run_batch(ctx, steps=None):
                        "points_per_step": pts_all, "time_steps": ts,
                        "l2": "inputs larger than L2 (%.0f MiB per field over all shots)"
                              % (pts_all * 4 / 2**20),
-                       "timed_launches": "batch mode 2: each shot's steps a chain of the "
-                                         "single-grid kernels on one of eight streams, step "
-                                         "pairs replayed from one CUDA graph per pair",
+                       "timed_launches": "batch mode 2: a step of all shots is one launch",
                        "persistent_kernel_value": other[0],
                        "persistent_over_plain": other[0] / plain,
                        "parallelism": "shot-sharded" if world > 1 else "single GPU",
