@@ -1,7 +1,8 @@
 // adi_adjoint_host.cu -- adi_wave_adjoint: reverse sweep over the recorded
 // run with checkpointing.
 //
-// The run kept (u^{k-1}, u^k) at every `every`-th step.  The reverse sweep
+// The run kept (u^{k-1}, u^k) at every `every`-th step, and on moderate grids
+// w and z of the steps of its last two segments.  The reverse sweep
 // visits the segments last to first; for each it restores the segment's
 // checkpoint, recomputes the segment forward while storing the x-sweep result
 // w and the y-sweep result z of every step, then runs the reverse steps of
@@ -43,6 +44,32 @@ void adi_wave::free_adj_work() {
   cudaFree(aw.gd);
   cudaFree(aw.rec);
   aw = AdjWork{};
+  rr.kept = 0;
+}
+
+// Whether a segment may be recomputed beside the reverse steps of the one
+// after it (two segment buffers), and the run's last two kept: up to 2
+// million points, beyond which a step fills the GPU by itself and a segment
+// is large.  (There the columns are also short enough for the cluster form of
+// the y sweep; the other form's segment scratch, y_stage 4, is one per grid
+// and must not serve both directions at once.)
+bool adi_wave::adj_beside(const Grid& G) const {
+  return (size_t)G.ld * G.ny <= ((size_t)1 << 21) && G.plan.y_stage != ADI_STAGE_COOP;
+}
+
+// Whether the run may take the reverse sweep's workspace early: it has it
+// already, or more than half of the device's memory stays free.  (Shots that
+// are all run before the first is differentiated would otherwise each hold a
+// workspace that only one of them needs at a time.)
+bool adi_wave::adj_room(const Grid& G, int E, int bufs) const {
+  const size_t fbytes = sizeof(float) * (size_t)G.ld * G.ny;
+  if (aw.fbytes == fbytes && aw.E >= E && (aw.bufs >= bufs || aw.one_buf)) return true;
+  size_t room = 0, total = 0;
+  if (cudaMemGetInfo(&room, &total) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return room / 2 > total / 4 + fbytes * ((size_t)E * bufs + 4);
 }
 
 int adi_wave::ensure_adj_work(Grid& G, int E, int n_rec, int bufs) {
@@ -108,12 +135,7 @@ int adi_wave::adjoint(const float* resid, double* grad_m, float* grad_wavelet, i
   const int S = rr.steps, E = rr.every;
   const int nck = (S + E - 1) / E;
   const size_t ffl = (size_t)G.ld * G.ny;  // floats per field
-  // Two segment buffers let the next segment be recomputed beside the current
-  // one's reverse steps: up to 2 million points, beyond which a step fills
-  // the GPU by itself.  (There the columns are also short enough for the
-  // cluster form of the y sweep; the other form's segment scratch, y_stage 4,
-  // is one per grid and must not serve both directions at once.)
-  const bool beside = nck > 1 && ffl <= ((size_t)1 << 21) && G.plan.y_stage != ADI_STAGE_COOP;
+  const bool beside = nck > 1 && adj_beside(G);
   int rc = ensure_adj_work(G, E, n_rec, beside ? 2 : 1);
   if (rc != ADI_OK) return rc;
   const int bufs = beside ? aw.bufs : 1;
@@ -210,17 +232,19 @@ int adi_wave::adjoint(const float* resid, double* grad_m, float* grad_wavelet, i
     if (bufs > 1) CKA(cudaEventRecord(seg_ev[c % bufs], rst), "segment recomputed");
     return ADI_OK;
   };
-  if (nck > 0) {
+  const int kept = rr.kept_bufs == bufs ? rr.kept : 0;  // the run left its last segments in place
+  if (nck > 0 && kept == 0) {
     rc = recompute(nck - 1);
     if (rc != ADI_OK) return rc;
   }
+  rr.kept = nck <= bufs ? kept : 0;  // the other segments go to the same buffers
   for (int c = nck - 1; c >= 0; --c) {
     const int s0 = c * E;
     const int len = std::min(E, S - s0);
     const size_t off = ffl * E * (size_t)(c % bufs);
     if (bufs > 1) {
-      CKA(cudaStreamWaitEvent(st, seg_ev[c % bufs], 0), "segment");
-      if (c > 0) {
+      if (c < nck - kept) CKA(cudaStreamWaitEvent(st, seg_ev[c % bufs], 0), "segment");
+      if (c > 0 && c - 1 < nck - kept) {
         rc = recompute(c - 1);
         if (rc != ADI_OK) return rc;
       }

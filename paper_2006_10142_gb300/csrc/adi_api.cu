@@ -311,8 +311,8 @@ y_done:
   // separate sweeps is set: wherever the couplings of both directions decay
   // below 2^-30 within its halo, the elimination is FP32 and a row fills a
   // TMA box (32 columns).  us per step, sweeps and one pass: 128^2 7.3 and
-  // 3.4, 1024^2 15.5 and 7.5, 2048^2 36.1 and 25.9, 4096^2 137 and 58,
-  // 16384^2 2063 and 768.  Its steps are launched one by one: consecutive
+  // 2.7, 1024^2 15.5 and 7.5, 2048^2 36.1 and 24.2,
+  // 4096^2 137 and 57, 16384^2 2063 and 768.  Its steps are launched one by one: consecutive
   // launches overlap, which those on either side of a graph's end do not
   // (1024^2: 7.5 against 9.3 from graphs of two steps).
   P.tile = 0;

@@ -312,7 +312,8 @@ __global__ void __launch_bounds__(kPN, 2)
 // of a step is that of one patch (its two phases, about 3.6 us above, where
 // two warps per scheduler share the issue slots), and here each thread has
 // half the work and an SM half the points: 128^2 3.4 against 6.1 us per step,
-// 512^2 4.5 against 6.1.  The operations on an unknown and the chunks are
+// 512^2 4.5 against 6.1 (2.7 and 3.7 since the launch carries level and
+// source by value).  The operations on an unknown and the chunks are
 // the same, so with H = 12 the results are too, bit for bit (H = 16 reaches
 // the stage's outermost column, which the two kinds cut elsewhere).  Taken
 // while two per SM hold the grid: 640 x 600 (300 patches) 4.6 against 6.3,

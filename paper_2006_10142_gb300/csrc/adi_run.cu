@@ -634,6 +634,7 @@ int adi_wave::run(int steps, const adi_source* src, const int32_t* rec_xy, int n
   if (!one_pass || use_graph || n_rec > 0)
     if (upload_gd(G, st) != ADI_OK) return ADI_ECUDA;
 
+  rr.kept = 0;
   if (record) {
     rr.valid = true;
     rr.k0 = G.k;
@@ -669,6 +670,28 @@ int adi_wave::run(int steps, const adi_source* src, const int32_t* rec_xy, int n
     graph_rec_at = d_rec;
   }
   const size_t fbytes = sizeof(float) * (size_t)G.ld * G.ny;
+  // w and z of the last segments, as many as it has buffers for (two), go
+  // straight into the workspace of the reverse sweep that is to come, which
+  // then need not recompute them (the gradient at 1024^2, 100 steps in two
+  // segments: 5.89 -> 4.83 ms; 301^2, 60 steps in three, with set-up: 2.99 ->
+  // 2.78).  Where there is no
+  // room the reverse sweep finds that out for itself.  Not while the stream
+  // is being captured (the workspace may have to grow), nor ever after: a
+  // replay writes the checkpoints behind this handle's back.
+  const int nck = every > 0 ? (steps + every - 1) / every : 0;
+  int keep = 0;
+  if (record && every > 0) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(st, &cs), "capture status");
+    if (cs != cudaStreamCaptureStatusNone) rr.captured = true;
+  }
+  if (record && every > 0 && gather && !model.active && !rr.captured && adj_beside(G)) {
+    const std::string err0 = err;
+    const int bufs = nck > 1 ? 2 : 1;
+    if (adj_room(G, every, bufs) && ensure_adj_work(G, every, n_rec, bufs) == ADI_OK)
+      keep = bufs > 1 ? aw.bufs : 1;
+    err = err0;
+  }
   int s = 0;
   while (s < steps) {
     int seg = steps - s;
@@ -682,6 +705,23 @@ int adi_wave::run(int steps, const adi_source* src, const int32_t* rec_xy, int n
       seg = std::min(seg, every - s % every);
     }
     int t = 0;
+    if (keep > 0 && s >= (nck - keep) * every) {
+      const size_t ffl = (size_t)G.ld * G.ny;
+      const size_t off = ffl * every * (size_t)(s / every % keep);
+      for (; t < seg; ++t) {
+        int rc = launch_fwd(G, G.buf[G.cur], G.buf[1 - G.cur], aw.wseg + off + ffl * t, aw.zseg + off + ffl * t, G.gd,
+                            gather, st);
+        if (rc != ADI_OK) {
+          rr.kept = 0;
+          return rc;
+        }
+        G.cur = 1 - G.cur;
+        G.k += 1;
+        G.from_init = false;
+      }
+      rr.kept += 1;
+      rr.kept_bufs = keep;
+    }
     if (model.active) {
       while (t < seg) {
         int rc = enqueue_model_step(G, st, gather);

@@ -77,6 +77,9 @@ struct RunRecord {
   std::vector<int> rec;             // [n_rec][2] host copy
   std::vector<float*> ckpt;         // checkpoint c: 2 fields (u^{k-1}, u^k) at step c*every
   size_t ckpt_bytes = 0;
+  int kept = 0;                     // w and z of this many last segments are in the adjoint workspace ...
+  int kept_bufs = 0;                // ... at the place they have among this many segment buffers
+  bool captured = false;            // some recorded run went into a caller's graph
   bool taylor = false;              // run started at level 1 right after a Taylor start-up
 };
 
@@ -205,6 +208,8 @@ struct adi_wave {
   int launch_fwd_tile(adi::Grid& G, const float* u_cur, float* u_prev, adi::GridDev* gd, int par, bool gather,
                       bool by_value, cudaStream_t st);
   int ensure_adj_work(adi::Grid& G, int E, int n_rec, int bufs);
+  bool adj_beside(const adi::Grid& G) const;
+  bool adj_room(const adi::Grid& G, int E, int bufs) const;
   void free_adj_work();
   int launch_pair_graph(adi::Grid& G, cudaStream_t st, bool gather, bool one_pass);
   void drop_graphs();

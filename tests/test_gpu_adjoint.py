@@ -260,3 +260,44 @@ def test_adjoint_1024_finite_differences():
         errs.append(abs(fd - an) / max(abs(fd), 1e-30))
     assert max(errs) < 1e-2, errs
     h.close()
+
+
+# ------------------------------------------------------------------------
+# last segments kept by the run
+# ------------------------------------------------------------------------
+
+@pytest.mark.parametrize("n,steps", [(33, 12), (301, 24)])
+def test_gradient_is_the_same_from_kept_and_from_recomputed_segments(n, steps):
+    """The run leaves w and z of its last two segments for the reverse sweep.  Runs
+    of one, two, three and `steps` segments (the last one shorter where `steps`
+    does not divide), each differentiated twice: a second call, or one with
+    other buffers, recomputes what the first one found kept.  The recomputation
+    is the same kernels on the same values, so all gradients agree to the bit.
+    """
+    import torch
+    from paper_2006_10142_gb300 import api
+    dev = _dev()
+    prob, _ = inputs.adjoint_problem(n, steps, seed=3, n_rec=9)
+    src = (n // 2, prob.rec[0][1] + 3)  # near the receivers: few steps
+    wav = torch.from_numpy(f32(prob.wavelet)).to(dev)
+    m = torch.from_numpy(f32(prob.m)).to(dev)
+    zero = torch.zeros(n, n, device=dev)
+    gen = np.random.default_rng(5)
+    resid = torch.from_numpy(f32(gen.standard_normal((steps, len(prob.rec))))).to(dev)
+    seen = []
+    for every in (steps, steps - 1, (steps + 1) // 2, steps // 3 - 1, 1):
+        h = api.AdiWave(m, zero, prob.tau, src=src, wavelet=wav)
+        try:
+            h.set_checkpointing(every)
+            for _ in range(2):  # a second run of the handle finds the workspace in place
+                h.reset(zero, src=src, wavelet=wav)
+                h.run(steps, src=src, wavelet=wav, rec=prob.rec)
+                for _ in range(2):
+                    gm, gw = h.adjoint(resid)
+                    seen.append((every, gm.clone(), gw.clone()))
+            h.sync_status()
+        finally:
+            h.close()
+    for every, gm, gw in seen:
+        assert torch.isfinite(gm).all() and gm.abs().max() > 0
+        assert torch.equal(gm, seen[0][1]) and torch.equal(gw, seen[0][2]), every
