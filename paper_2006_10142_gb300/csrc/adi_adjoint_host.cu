@@ -33,15 +33,7 @@ using namespace adi;
   } while (0)
 
 void adi_wave::free_adj_work() {
-  cudaFree(aw.wseg);
-  cudaFree(aw.zseg);
-  cudaFree(aw.wb);
-  cudaFree(aw.rb);
-  cudaFree(aw.g64);
-  for (int q = 0; q < 2; ++q) cudaFree(aw.L[q]);
-  cudaFree(aw.A);
-  cudaFree(aw.B);
-  cudaFree(aw.gd);
+  cudaFree(aw.mem);
   cudaFree(aw.rec);
   aw = AdjWork{};
   rr.kept = 0;
@@ -75,19 +67,18 @@ bool adi_wave::adj_room(const Grid& G, int E, int bufs) const {
 int adi_wave::ensure_adj_work(Grid& G, int E, int n_rec, int bufs) {
   const size_t fbytes = sizeof(float) * (size_t)G.ld * G.ny;
   if (aw.fbytes != fbytes || aw.E < E || (aw.bufs < bufs && !aw.one_buf)) {
+    const size_t field = (fbytes + 255) / 256 * 256;
+    size_t used = 0;
+    auto take = [&](size_t b) {
+      used += b;
+      return aw.mem + (used - b);
+    };
+    auto seg = [&] { return (fbytes * E * bufs + 255) / 256 * 256; };
     cudaError_t e = cudaSuccess;
     bool one_buf = false;
     for (;;) {
       free_adj_work();
-      e = cudaMalloc(&aw.wseg, fbytes * E * bufs);
-      if (e == cudaSuccess) e = cudaMalloc(&aw.zseg, fbytes * E * bufs);
-      if (e == cudaSuccess) e = cudaMalloc(&aw.wb, fbytes);
-      if (e == cudaSuccess) e = cudaMalloc(&aw.rb, fbytes);
-      if (e == cudaSuccess) e = cudaMalloc(&aw.g64, 2 * fbytes);
-      for (int q = 0; q < 2 && e == cudaSuccess; ++q) e = cudaMalloc(&aw.L[q], fbytes);
-      if (e == cudaSuccess) e = cudaMalloc(&aw.A, fbytes);
-      if (e == cudaSuccess) e = cudaMalloc(&aw.B, fbytes);
-      if (e == cudaSuccess) e = cudaMalloc(&aw.gd, sizeof(GridDev));
+      e = cudaMalloc(&aw.mem, 2 * seg() + 8 * field + sizeof(GridDev));
       if (e == cudaSuccess || bufs == 1) break;
       cudaGetLastError();
       bufs = 1;  // room for one segment, perhaps
@@ -98,6 +89,15 @@ int adi_wave::ensure_adj_work(Grid& G, int E, int n_rec, int bufs) {
       free_adj_work();
       return fail(this, ADI_ENOMEM, "allocate adjoint workspace");
     }
+    aw.wseg = reinterpret_cast<float*>(take(seg()));
+    aw.zseg = reinterpret_cast<float*>(take(seg()));
+    aw.wb = reinterpret_cast<float*>(take(field));
+    aw.rb = reinterpret_cast<float*>(take(field));
+    aw.g64 = reinterpret_cast<double*>(take(2 * field));
+    for (int q = 0; q < 2; ++q) aw.L[q] = reinterpret_cast<float*>(take(field));
+    aw.A = reinterpret_cast<float*>(take(field));
+    aw.B = reinterpret_cast<float*>(take(field));
+    aw.gd = reinterpret_cast<GridDev*>(take(sizeof(GridDev)));
     aw.fbytes = fbytes;
     aw.E = E;
     aw.bufs = bufs;

@@ -48,6 +48,7 @@ struct Grid {
   int nx = 0, ny = 0, ld = 0;
   double lx = 1, ly = 1, dt = 0, hx = 0, hy = 0;
   int start = 0, fp64mode = 0;
+  char* mem = nullptr;              // the one allocation behind m, buf, w and gd
   float* m = nullptr;               // [ny][ld]
   float* buf[2] = {nullptr, nullptr};  // buf[cur] = u^k, buf[1-cur] = u^{k-1}
   float* w = nullptr;               // scratch [ny][ld]
@@ -75,6 +76,7 @@ struct RunRecord {
   int every = 0;
   adi_source src = {-1, -1, nullptr, 0};
   std::vector<int> rec;             // [n_rec][2] host copy
+  std::vector<float*> ckpt_mem;     // allocations behind the checkpoints
   std::vector<float*> ckpt;         // checkpoint c: 2 fields (u^{k-1}, u^k) at step c*every
   size_t ckpt_bytes = 0;
   int kept = 0;                     // w and z of this many last segments are in the adjoint workspace ...
@@ -106,6 +108,7 @@ struct AdjWork {
   int E = 0;          // segment length it was sized for
   bool one_buf = false;  // there was no room for two segments
   int bufs = 0;       // segments wseg and zseg hold (2: one recomputed while the other is reversed)
+  char* mem = nullptr;    // the one allocation behind the pointers up to gd
   float* wseg = nullptr;  // [bufs][E] forward x-sweep results of a segment
   float* zseg = nullptr;  // [bufs][E] forward y-sweep results of a segment
   float* wb = nullptr;    // wbar
