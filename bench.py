@@ -70,7 +70,8 @@ BYTES_STEP = 16  # the one-launch step: read u^k, u^{k-1}, m; write u^{k+1}
 # grid points (profiles/).  Only valid for the 16384^2 workload and the
 # kernel builds the captures were taken on; None once a kernel has changed.
 NCU_TRAFFIC = {("ricker_16384", "y_coop_kernel"): 5702261248,
-               ("ricker_16384", "x_band_kernel"): 3124610560}
+               ("ricker_16384", "x_band_kernel"): 3124610560,
+               ("ricker_16384", "tile_step_kernel"): 4255998464}
 
 
 def measured_peak_gbs():

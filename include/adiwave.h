@@ -147,7 +147,12 @@ int adi_wave_run(adi_wave *h, int32_t steps, const adi_source *src,
 /* Keep (u^{k-1}, u^k) every `every` steps during adi_wave_run (0 = off).
  * Runs that keep checkpoints take the separate sweeps, whose results the
  * reverse sweep recomputes; other runs agree with them to rounding.
- * The memory (2 fields per checkpoint) is allocated by the next run. */
+ * The memory (2 fields per checkpoint) is allocated by the next run.  A run
+ * with receivers on a grid of at most 2^21 points also leaves the sweeps'
+ * results of its last two segments in the workspace of adi_wave_adjoint(),
+ * which it then allocates if more than half of the device's memory stays
+ * free (4 fields per step of a segment, and 8); not while its stream is
+ * being captured.  The gradient is the same either way. */
 int adi_wave_set_checkpointing(adi_wave *h, int32_t every);
 
 /* Gradient of J = 1/2 sum_s sum_r (traces[s][r] - d[s][r])^2 for the last
