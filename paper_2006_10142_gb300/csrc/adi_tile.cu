@@ -51,24 +51,18 @@
 #include "adi_internal.h"
 #include "adi_local.cuh"
 #include "adi_sweeps.cuh"
+#include "adi_tile_stage.h"
 #include "adi_tma.cuh"
 
 namespace adi {
 
 namespace {
 
-constexpr int kTX = 224;              // columns a CTA solves
-constexpr int kTH = 16;               // halo columns on either side
-constexpr int kTB = 16;               // rows per block
-constexpr int kTS = kTX + 2 * kTH;    // staged columns
-constexpr int kTN = kTS / 2;          // threads: two rows (x phase) or two columns (y phase) each
-constexpr int kPanel = kTB * 128;     // bytes of a 32-column panel of a block
-constexpr int kSlot = (kTS / 32) * kPanel;  // bytes of one staged block
 constexpr int kOut = (kTX / 32) * kPanel;   // bytes of a block of the strip's own columns
 // shared memory: u slots 0..2 | m slots 0..1 | w, then the block's u^{k+1} |
 // u^{k-1} [16][224] | XT[17][8] float4 | X0[17][8] float2 | 3 mbarriers
-constexpr int kOffM = 3 * kSlot;
-constexpr int kOffW = 5 * kSlot;
+constexpr int kOffM = kUSlots * kSlot;
+constexpr int kOffW = kOffM + 2 * kSlot;
 constexpr int kOffP = kOffW + kOut;
 constexpr int kOffXT = kOffP + kOut;
 constexpr int kOffX0 = kOffXT + 17 * 8 * 16;
@@ -151,20 +145,11 @@ __device__ __forceinline__ void tile_body(const TileArgs& a, const CUtensorMap* 
     if (nblk > 1) issue(1);
   }
 
-  // x phase: rows xr and xr + 8 of the block, chunk ch.  The 16-byte unit q
-  // of a chunk in row r of a panel lies at byte r 128 + ((unit ^ (r & 7)) 16):
-  // the offsets below hold the chunk's first unit, the others follow by XOR
-  // of 16 q, and row r + 8 lies 1024 bytes on.  u^k's blocks are shifted by
-  // one row: rows r - 1, r, r + 1 of the block are at indexes r - 2, r - 1, r,
-  // the negative ones at the end of the block before.
+  // x phase: rows xr and xr + 8 of the block, chunk ch (offsets: adi_tile_stage.h)
   const int xr = tid & 7;
   const int ch = tid >> 3;
-  auto unit0 = [&](int r, int c) { return (uint32_t)((c >> 1) * kPanel + r * 128 + (((c & 1) * 64) ^ ((r & 7) << 4))); };
-  const uint32_t oc = unit0(xr + 7, ch), ou = unit0(xr + 6, ch), od = unit0(xr, ch);
-  // the unknowns beside the chunk: the last of the one before, the first of the next
-  const uint32_t oL = ch > 0 ? (unit0(xr + 7, ch - 1) ^ 48u) + 12u : 0u;
-  const uint32_t oR = ch < 15 ? unit0(xr + 7, ch + 1) : 0u;
-  const uint32_t ow = sa + kOffW + unit0(xr, ch - 1);  // w holds the strip's own columns
+  const TileRow at = tile_row(xr, ch);
+  const uint32_t ow = sa + kOffW + tile_unit(xr, ch - 1);  // w holds the strip's own columns
   const int gx0 = c0 + 16 * ch;                        // column of the chunk's first unknown
   // w is wanted as sigma w by the column solves (rows xr and xr + 8 have the same sigma)
   const float sg = ((xr & 3) == 1 || (xr & 3) == 2) ? -1.f : 1.f;
@@ -211,10 +196,10 @@ __device__ __forceinline__ void tile_body(const TileArgs& a, const CUtensorMap* 
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         // bases of the slots that hold rows r (centre) and r - 1 (above)
-        const uint32_t bc = h == 0 ? (xr >= 1 ? Ucur - 1024u : Uprev + 1024u) : Ucur;
-        const uint32_t bu = h == 0 ? (xr >= 2 ? Ucur - 1024u : Uprev + 1024u) : Ucur;
-        const uint32_t pc = bc + oc, pu = bu + ou;
-        const uint32_t pd = Ucur + od, pm = Mb + od;
+        const uint32_t bc = tile_row_base(Ucur, Uprev, xr, h, 0);
+        const uint32_t bu = tile_row_base(Ucur, Uprev, xr, h, 1);
+        const uint32_t pc = bc + at.centre, pu = bu + at.above;
+        const uint32_t pd = Ucur + at.below, pm = Mb + at.below;
         f2 c2[8];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -222,7 +207,7 @@ __device__ __forceinline__ void tile_body(const TileArgs& a, const CUtensorMap* 
           c2[2 * q] = t.x;
           c2[2 * q + 1] = t.y;
         }
-        const float uL = lds(bc + oL), uR = lds(bc + oR);
+        const float uL = lds(bc + at.left), uR = lds(bc + at.right);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const ulonglong2 t4 = lds4(pu ^ (16u * q));
