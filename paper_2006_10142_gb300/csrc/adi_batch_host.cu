@@ -190,8 +190,11 @@ int adi_wave::ensure_batch_tiles() {
       shots.push_back((int)s);
       bt_h = std::max(bt_h, g[s].plan.tile);
     }
-  bt_plans = plans;
-  if (shots.size() < 2) return ADI_OK;
+  bt_plans.clear();  // until the tables are in place: a failure below is not taken for them
+  if (shots.size() < 2) {
+    bt_plans = plans;
+    return ADI_OK;
+  }
   int dev = 0, nsm = 0;
   CKB(cudaGetDevice(&dev), "get device");
   CKB(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev), "SM count");
@@ -284,15 +287,18 @@ int adi_wave::ensure_batch_tiles() {
   std::stable_sort(items.begin(), items.end(), [](const Item& x, const Item& y) { return x.cost < y.cost; });
   std::vector<int2> list;
   for (const Item& i : items) list.push_back(i.it);
-  bt_plans.clear();  // until the tables are in place
   cudaFree(bt_dev);
   cudaFree(bt_items);
   bt_dev = nullptr;
   bt_items = nullptr;
   CKB(cudaMalloc(&bt_dev, sizeof(BatchTile) * tiles.size()), "alloc batch tables");
   CKB(cudaMalloc(&bt_items, sizeof(int2) * list.size()), "alloc batch tables");
-  CKB(cudaMemcpy(bt_dev, tiles.data(), sizeof(BatchTile) * tiles.size(), cudaMemcpyHostToDevice), "batch tables");
-  CKB(cudaMemcpy(bt_items, list.data(), sizeof(int2) * list.size(), cudaMemcpyHostToDevice), "batch tables");
+  // On the handle's own stream, and waited for: a copy from pageable memory on
+  // the legacy stream may return before it has landed, and a non-blocking
+  // stream of the caller's is not ordered behind it.
+  CKB(cudaMemcpyAsync(bt_dev, tiles.data(), sizeof(BatchTile) * tiles.size(), cudaMemcpyHostToDevice, cap), "batch tables");
+  CKB(cudaMemcpyAsync(bt_items, list.data(), sizeof(int2) * list.size(), cudaMemcpyHostToDevice, cap), "batch tables");
+  CKB(cudaStreamSynchronize(cap), "batch tables");
   bt_n = (int)tiles.size();
   bt_n_items = (int)list.size();
   bt_plans = plans;
