@@ -3,12 +3,13 @@ list): in place for the first run, whatever stream it is on, and rebuilt when
 a reset changes a plan."""
 import pytest
 
-from helpers import f32
+from helpers import f32, rel_l2
 from test_gpu_tile import _problem
 
 pytestmark = pytest.mark.gpu
 
 STEPS = 3
+BOUND = 4 * STEPS ** 2 * 2.0 ** -24  # two forms of a step, as in test_gpu_tile.py
 
 
 def _batch(probs, mode=None):
@@ -26,7 +27,7 @@ def _states(B):
 
 
 def _shot_by_shot(probs, steps):
-    """The same kernels launched per shot: equal to the bit for the halo of 12."""
+    """The same step launched per shot."""
     B, _ = _batch(probs, mode=1)
     B.run(steps)
     out = _states(B)
@@ -35,12 +36,12 @@ def _shot_by_shot(probs, steps):
     return out
 
 
-def _equal(a, b):
-    import torch
-    return all(torch.equal(x[0], y[0]) and torch.equal(x[1], y[1]) for x, y in zip(a, b))
+def _near(a, b):
+    h = lambda t: t.double().cpu().numpy()
+    return all(rel_l2(h(x[q]), h(y[q])) < BOUND for x, y in zip(a, b) for q in (0, 1))
 
 
-# 256 x 240 and above go by bands, 100 columns by patches
+# by bands and, with a shot of 100 columns, by patches
 @pytest.mark.parametrize("shapes", [[(2300, 2000), (700, 900), (224, 300)], [(300, 260), (100, 41)]])
 def test_first_run_on_a_non_blocking_stream(shapes):
     import torch
@@ -52,5 +53,5 @@ def test_first_run_on_a_non_blocking_stream(shapes):
         torch.cuda.synchronize()
         B.run(STEPS, stream=side)
         side.synchronize()
-        assert _equal(_states(B), want)
+        assert _near(_states(B), want)
         B.close()
