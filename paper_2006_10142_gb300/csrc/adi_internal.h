@@ -199,7 +199,7 @@ cudaError_t launch_patch(const TileArgs& a, int H, const CUtensorMap& u, const C
 cudaError_t configure_patch_kernels();
 // One grid of a batch advanced by one launch per step: arguments (par and
 // u_prev from the launch) and tensor maps, in device memory.
-struct BatchTile {
+struct alignas(128) BatchTile {
   CUtensorMap u[2], p[2], m;  // of buf[0], buf[1] (panel and strip boxes) and m
   TileArgs a;
   float* buf[2];

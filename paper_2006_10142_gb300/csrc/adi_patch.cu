@@ -302,6 +302,10 @@ __global__ void __launch_bounds__(kPN, 2)
     patch_batch_kernel(const BatchTile* __restrict__ tiles, const int2* __restrict__ items, int par) {
   const int2 it = __ldg(items + blockIdx.x);
   const BatchTile& t = tiles[it.x];
+  if (threadIdx.x < 32) {  // the warp that issues the tensor copies
+    tensormap_acquire(&t.u[par]);
+    tensormap_acquire(&t.m);
+  }
   const TileArgs a = t.a;
   patch_body<H, false>(a, &t.u[par], &t.m, it.y, par, t.buf[par ^ 1]);
 }

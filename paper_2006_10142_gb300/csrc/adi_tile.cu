@@ -398,6 +398,12 @@ __global__ void __launch_bounds__(kTN, 2)
     tile_batch_kernel(const BatchTile* __restrict__ tiles, const int2* __restrict__ items, int par) {
   const int2 it = __ldg(items + blockIdx.x);
   const BatchTile& t = tiles[it.x];
+  if (threadIdx.x < 32) {  // the warp that issues the tensor copies
+    tensormap_acquire(&t.u[par]);
+    tensormap_acquire(&t.m);
+    tensormap_acquire(&t.p[par ^ 1]);
+    tensormap_acquire(&t.u[par ^ 1]);
+  }
   const TileArgs a = t.a;
   tile_body<H, false>(a, &t.u[par], &t.m, &t.p[par ^ 1], &t.u[par ^ 1], it.y, par, t.buf[par ^ 1]);
 }

@@ -88,6 +88,13 @@ __device__ __forceinline__ void bulk_load_16(uint32_t dst, const void* src, uint
       : "memory");
 }
 
+// Makes a tensor map that a host copy wrote to global memory visible to this
+// thread's tensor copies: a map at the same address may have been used before
+// with other contents.  (Maps passed as kernel parameters need none.)
+__device__ __forceinline__ void tensormap_acquire(const CUtensorMap* tm) {
+  asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(reinterpret_cast<uint64_t>(tm)) : "memory");
+}
+
 // Tiled 2D tensor load (coordinates in elements, innermost first; c0 * 4
 // bytes a multiple of 16; dst 128-byte aligned).
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* tm, int c0, int c1,

@@ -55,3 +55,21 @@ def test_first_run_on_a_non_blocking_stream(shapes):
         side.synchronize()
         assert _near(_states(B), want)
         B.close()
+
+
+def test_tables_follow_a_reset_that_changes_a_plan():
+    """The second shot's medium moves it from the one-launch step to the sweeps
+    and back, then all shots to the halo of 16: the tables are freed and made
+    again, as like as not at the same address, with other shots and boxes."""
+    import torch
+    shapes = [(300, 260), (224, 300), (700, 500)]
+    base = [_problem(nx, ny, 0.5, nx + ny) for nx, ny in shapes]
+    B, t = _batch(base)
+    for scale in ((1, 1, 1), (1, 16, 1), (1, 1, 1), (3.9, 3.9, 3.9), (1, 16, 16), (1, 1, 1)):
+        probs = [(s * p[0],) + p[1:] for s, p in zip(scale, base)]
+        want = _shot_by_shot(probs, STEPS)
+        B.reset([t(p[1]) for p in probs], ms=[t(p[0]) for p in probs])
+        B.run(STEPS)
+        B.sync_status()
+        assert _near(_states(B), want), scale
+    B.close()
