@@ -140,6 +140,16 @@ int adi_wave::adjoint(const float* resid, double* grad_m, float* grad_wavelet, i
   if (rc != ADI_OK) return rc;
   const int bufs = beside ? aw.bufs : 1;
   const size_t fbytes = aw.fbytes;
+  // Segments the run left in place.  A call that is being captured counts on
+  // none: its replays come after other runs and after one another, and each
+  // overwrites the buffers, so that runs may leave none from now on either.
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  CKA(cudaStreamIsCapturing(st, &cs), "capture status");
+  if (cs != cudaStreamCaptureStatusNone) {
+    rr.captured = true;
+    rr.kept = 0;
+  }
+  const int kept = rr.kept_bufs == bufs ? rr.kept : 0;
 
   const bool src_on = rr.src.ix >= 0 && rr.src.wavelet != nullptr && rr.src.n_wavelet > 0;
   if (grad_wavelet && rr.src.n_wavelet > 0)
@@ -197,7 +207,7 @@ int adi_wave::adjoint(const float* resid, double* grad_m, float* grad_wavelet, i
   float* L0 = aw.L[0];
   float* L1 = aw.L[1];
   cudaStream_t rst = st;
-  if (bufs > 1) {
+  if (bufs > 1 && kept < nck) {
     if (!rec_st) {
       CKA(cudaStreamCreateWithFlags(&rec_st, cudaStreamNonBlocking), "create recomputation stream");
       CKA(cudaEventCreateWithFlags(&fork_adj, cudaEventDisableTiming), "create event");
@@ -232,7 +242,6 @@ int adi_wave::adjoint(const float* resid, double* grad_m, float* grad_wavelet, i
     if (bufs > 1) CKA(cudaEventRecord(seg_ev[c % bufs], rst), "segment recomputed");
     return ADI_OK;
   };
-  const int kept = rr.kept_bufs == bufs ? rr.kept : 0;  // the run left its last segments in place
   if (nck > 0 && kept == 0) {
     rc = recompute(nck - 1);
     if (rc != ADI_OK) return rc;
@@ -298,7 +307,7 @@ int adi_wave::adjoint(const float* resid, double* grad_m, float* grad_wavelet, i
       std::swap(L0, L1);
     }
     if (bufs > 1) {
-      CKA(cudaEventRecord(rev_ev[c % bufs], st), "segment reversed");
+      if (kept < nck) CKA(cudaEventRecord(rev_ev[c % bufs], st), "segment reversed");
     } else if (c > 0) {
       rc = recompute(c - 1);
       if (rc != ADI_OK) return rc;

@@ -81,7 +81,7 @@ struct RunRecord {
   size_t ckpt_bytes = 0;
   int kept = 0;                     // w and z of this many last segments are in the adjoint workspace ...
   int kept_bufs = 0;                // ... at the place they have among this many segment buffers
-  bool captured = false;            // some recorded run went into a caller's graph
+  bool captured = false;            // some recorded run or adjoint went into a caller's graph
   bool taylor = false;              // run started at level 1 right after a Taylor start-up
 };
 
