@@ -61,17 +61,21 @@ int plan_grid(Grid& G, const adi_wave_tuning& t, std::string& why) {
   P.fp64x = G.fp64mode == ADI_FP64_ALWAYS || (G.fp64mode == ADI_FP64_AUTO && weak_x);
   P.fp64y = G.fp64mode == ADI_FP64_ALWAYS || (G.fp64mode == ADI_FP64_AUTO && weak_y);
   if (t.solver < ADI_SOLVER_AUTO || t.solver > ADI_SOLVER_CR_SMEM) { why = "unknown solver"; return ADI_EINVAL; }
+  const int ct = t.cta_threads;
+  const int cty = t.cta_threads_y;
   // FP64 in both directions is bound by the FP64 pipe (1/64 of the FP32
   // rate), where the tree's merges, done by all lanes of a warp at every
   // level, are work: cyclic reduction in shared memory then (ms at 4096^2, x
-  // and y: tree 1.21 and 1.30, CR 1.00 and 0.71).
-  P.tree = t.solver != ADI_SOLVER_CR_SMEM && !(t.solver == ADI_SOLVER_AUTO && P.fp64x && P.fp64y);
+  // and y: tree 1.21 and 1.30, CR 1.00 and 0.71).  Only with the column
+  // geometry chosen for it below: a geometry that is given keeps the tree,
+  // whose top system the reverse step needs to fit too.
+  const bool y64_auto = P.fp64x && P.fp64y && t.solver == ADI_SOLVER_AUTO && cty == 0 && t.chunk_y == 0 &&
+                        t.cols_per_cta == 0;
+  P.tree = t.solver != ADI_SOLVER_CR_SMEM && !y64_auto;
   int pcr = t.pcr_size ? t.pcr_size : 32;
   if (pcr != 2 && pcr != 4 && pcr != 8 && pcr != 16 && pcr != 32) { why = "pcr_size must be 2..32, a power of two"; return ADI_EINVAL; }
   P.pcr = pcr;
 
-  const int ct = t.cta_threads;
-  const int cty = t.cta_threads_y;
   if (cty != 0 && cty != 64 && cty != 128 && cty != 256 && cty != 512 && cty != 1024) { why = "cta_threads_y must be 64..1024, a power of two"; return ADI_EINVAL; }
   if (ct != 0 && ct != 64 && ct != 128 && ct != 256 && ct != 512 && ct != 1024) { why = "cta_threads must be 64..1024, a power of two"; return ADI_EINVAL; }
   // ---- x sweep
@@ -187,8 +191,6 @@ x_done:
       return C <= maxC && (!P.tree || groups <= 32);
     };
     int K = t.chunk_y;
-    const bool y64_auto = P.fp64y && !P.tree && t.solver == ADI_SOLVER_AUTO && cty == 0 && t.chunk_y == 0 &&
-                          t.cols_per_cta == 0;
     if (y64_auto) {
       // strips of 8 columns, 16 (32) rows per thread, CTAs of 256 threads (ms
       // at 2048 x 1500 and 4096^2: 0.202 and 0.76 with 16 rows, 0.71 with 32
