@@ -129,6 +129,14 @@ int adi_wave::adjoint(const float* resid, double* grad_m, float* grad_wavelet, i
                 "the run kept no checkpoints: call adi_wave_set_checkpointing before adi_wave_run");
   if (every != 0 && every != rr.every)
     return fail(this, ADI_EINVAL, "ckpt_every must be 0 or the run's checkpoint interval");
+  const GridPlan& P = g[0].plan;
+  // the column solves of the reverse step take the forward TMA pipeline
+  // when the forward y sweep does (strip maps of m and the two lam fields)
+  const bool ypipe = (P.y_stage == 3 || P.y_stage == 4) && !P.fp64y;
+  // else the tree, also where the forward sweeps take cyclic reduction: its
+  // top system holds at most 32 pieces of a column
+  if (!ypipe && P.C * std::max(1, (1 << P.log2tcol) / 32) > 32)
+    return fail(this, ADI_EUNSUPPORTED, "adjoint of a tuning with more than 32 pieces per column");
   const int n_rec = (int)(rr.rec.size() / 2);
   if (!grad_m || (n_rec > 0 && !resid)) return fail(this, ADI_EINVAL, "null gradient or residual");
   Grid& G = g[0];
@@ -190,10 +198,6 @@ int adi_wave::adjoint(const float* resid, double* grad_m, float* grad_wavelet, i
   hg.wavelet = src_on ? rr.src.wavelet : nullptr;
   hg.n_wavelet = src_on ? rr.src.n_wavelet : 0;
 
-  const GridPlan& P = G.plan;
-  // the column solves of the reverse step take the forward TMA pipeline
-  // when the forward y sweep does (strip maps of m and the two lam fields)
-  const bool ypipe = (P.y_stage == 3 || P.y_stage == 4) && !P.fp64y;
   CUtensorMap tl_m, tl_L[2];
   if (ypipe) {
     const int BH = y_pipe_box_rows(1 << P.log2tcol, P.ky);
