@@ -62,7 +62,6 @@ __device__ __noinline__ void add_wavelet_grad(float* gw, long long level, double
 template <int K, typename T, int MAXT>
 __global__ void __launch_bounds__(MAXT, adj_min_ctas(MAXT)) y_adj_kernel(const YAdjArgs a) {
   chain_wait();
-  chain_release();
   extern __shared__ __align__(16) unsigned char smem[];
   const int W = 1 << a.log2W;
   const int tcol = 1 << a.log2tcol;
@@ -112,7 +111,6 @@ __global__ void __launch_bounds__(MAXT, adj_min_ctas(MAXT)) y_adj_kernel(const Y
 template <int K, typename T, int MAXT>
 __global__ void __launch_bounds__(MAXT, adj_min_ctas(MAXT)) x_adj_kernel(const XAdjArgs a) {
   chain_wait();
-  chain_release();
   extern __shared__ __align__(16) unsigned char smem[];
   const int tsys = 1 << a.log2tsys;
   const int tid = threadIdx.x;
@@ -191,7 +189,6 @@ __global__ void __launch_bounds__(MAXT, adj_min_ctas(MAXT)) x_adj_kernel(const X
 template <int K, int MAXT>
 __global__ void __launch_bounds__(MAXT, adj_min_ctas(MAXT)) x_adj_staged_kernel(const XAdjArgs a) {
   chain_wait();
-  chain_release();
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int NQ = K / 4;  // float4 groups per thread
   const int threads = blockDim.x;
@@ -307,7 +304,6 @@ __device__ __forceinline__ void st4(float* p, const float (&v)[4]) {
 
 __global__ void __launch_bounds__(256) lam_update_kernel(LamArgs a) {
   chain_wait();
-  chain_release();
   const int i0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
   const int j = blockIdx.y;
   if (i0 >= a.nx || j >= a.ny) return;

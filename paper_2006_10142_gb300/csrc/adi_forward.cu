@@ -52,7 +52,6 @@ __device__ __forceinline__ void x_sample(const XArgs& a) {
 template <int K, typename T, int MAXT, bool TREE>
 __global__ void __launch_bounds__(MAXT, min_ctas(MAXT)) x_sweep_kernel(const XArgs a) {
   chain_wait();
-  chain_release();
   x_sample(a);
   extern __shared__ __align__(16) unsigned char smem[];
   if constexpr (sizeof(T) == 4) {
@@ -117,7 +116,6 @@ __global__ void __launch_bounds__(MAXT, min_ctas(MAXT))
     x_pipe_kernel(const XArgs a, const __grid_constant__ CUtensorMap tm_u,
                   const __grid_constant__ CUtensorMap tm_m, const __grid_constant__ CUtensorMap tm_w) {
   chain_wait();
-  chain_release();
   x_sample(a);
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int NQ = K / 4;
@@ -526,7 +524,6 @@ __global__ void __launch_bounds__(MAXT, min_ctas(MAXT))
     x_band_kernel(const XArgs a, const __grid_constant__ CUtensorMap tm_u,
                   const __grid_constant__ CUtensorMap tm_m, const __grid_constant__ CUtensorMap tm_w) {
   chain_wait();
-  chain_release();
   x_sample(a);
   static_assert((K == 16 || K == 32) && XC > 1, "band form: K = 16 or 32, rows over a cluster");
   extern __shared__ __align__(16) unsigned char smem[];
@@ -690,7 +687,6 @@ __global__ void __launch_bounds__(MAXT, min_ctas(MAXT))
 template <int K, typename T, int MAXT, bool TREE>
 __global__ void __launch_bounds__(MAXT, min_ctas(MAXT)) y_sweep_kernel(const YArgs a) {
   chain_wait();
-  chain_release();
   extern __shared__ __align__(16) unsigned char smem[];
   const int rank = cluster_rank(a.C);
   if (!a.persist) {
@@ -737,7 +733,6 @@ __global__ void __launch_bounds__(MAXT, min_ctas(MAXT))
                   const __grid_constant__ CUtensorMap tm_m, const __grid_constant__ CUtensorMap tm_uc,
                   const __grid_constant__ CUtensorMap tm_up) {
   chain_wait();
-  chain_release();
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int QG = 32 / W;  // row groups (q) per warp
   const int C = a.C;

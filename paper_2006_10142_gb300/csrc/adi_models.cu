@@ -45,7 +45,6 @@ __device__ __forceinline__ float wavelet_at(const GridDev* gd, long long k) {
 template <int K, int MAXT>
 __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 2 : 1) x_model_kernel(const ModelXArgs a) {
   chain_wait();
-  chain_release();
   extern __shared__ __align__(16) unsigned char smem[];
   const int tsys = 1 << a.log2tsys;
   const int tid = threadIdx.x;
@@ -136,7 +135,6 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 2 : 1) x_model_kernel(cons
 template <int K, int MAXT>
 __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 2 : 1) y_model_kernel(const ModelYArgs a) {
   chain_wait();
-  chain_release();
   extern __shared__ __align__(16) unsigned char smem[];
   const int C = a.C;
   cluster_arrive_early(C);
