@@ -76,8 +76,6 @@ int adi_wave::setup_batch(cudaStream_t st) {
       xa.stage_off = -1;
       xa.err = nullptr;
       xa.xc = 1;
-      xa.rec = nullptr;
-      xa.n_rec = 0;
       YArgs& ya = B.ya[c];
       ya.nx = G.nx; ya.ny = G.ny; ya.ld = G.ld;
       ya.log2W = ilog2(W); ya.log2tcol = ilog2(tcol); ya.C = 1; ya.pcr = 32;

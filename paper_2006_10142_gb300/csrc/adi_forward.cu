@@ -37,22 +37,22 @@ constexpr int min_ctas(int maxt) { return maxt <= 64 ? 8 : maxt <= 128 ? 4 : max
 // u^k(rec r) (the run's last level by gather_kernel): the receivers dealt out
 // over the CTAs' last warps, while the first warp starts the row loads.  A
 // launch of its own per step took about 2 us of a step of 1024^2.
-__device__ __forceinline__ void x_sample(const XArgs& a) {
+__device__ __forceinline__ void x_sample(const XArgs& a, const XRec& q) {
   const int t = (int)threadIdx.x - ((int)blockDim.x - 32);
-  if (a.n_rec <= 0 || t < 0) return;
+  if (q.n_rec <= 0 || t < 0) return;
   const GridDev* gd = a.gd;
-  for (int r = blockIdx.x + gridDim.x * t; r < a.n_rec; r += 32 * gridDim.x) {
-    const int2 at = __ldg(reinterpret_cast<const int2*>(a.rec) + r);
+  for (int r = blockIdx.x + gridDim.x * t; r < q.n_rec; r += 32 * gridDim.x) {
+    const int2 at = __ldg(reinterpret_cast<const int2*>(q.rec) + r);
     const long long s = gd->k - gd->k0 - 1;
     if (s < 0 || s >= gd->steps || gd->traces == nullptr) return;
-    gd->traces[s * a.n_rec + r] = __ldcg(a.u + (size_t)at.y * a.ld + at.x);
+    gd->traces[s * q.n_rec + r] = __ldcg(a.u + (size_t)at.y * a.ld + at.x);
   }
 }
 
 template <int K, typename T, int MAXT, bool TREE>
-__global__ void __launch_bounds__(MAXT, min_ctas(MAXT)) x_sweep_kernel(const XArgs a) {
+__global__ void __launch_bounds__(MAXT, min_ctas(MAXT)) x_sweep_kernel(const XArgs a, const XRec rec) {
   chain_wait();
-  x_sample(a);
+  x_sample(a, rec);
   extern __shared__ __align__(16) unsigned char smem[];
   if constexpr (sizeof(T) == 4) {
     if (a.stage_off >= 0) {
@@ -114,9 +114,9 @@ __device__ __forceinline__ float stage_at(const float* row, int e) {
 template <int K, int MAXT, int XC>
 __global__ void __launch_bounds__(MAXT, min_ctas(MAXT))
     x_pipe_kernel(const XArgs a, const __grid_constant__ CUtensorMap tm_u,
-                  const __grid_constant__ CUtensorMap tm_m, const __grid_constant__ CUtensorMap tm_w) {
+                  const __grid_constant__ CUtensorMap tm_m, const __grid_constant__ CUtensorMap tm_w, const XRec rec) {
   chain_wait();
-  x_sample(a);
+  x_sample(a, rec);
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int NQ = K / 4;
   const int tid = threadIdx.x;
@@ -523,8 +523,6 @@ template <int K, int MAXT, int XC>
 __global__ void __launch_bounds__(MAXT, min_ctas(MAXT))
     x_band_kernel(const XArgs a, const __grid_constant__ CUtensorMap tm_u,
                   const __grid_constant__ CUtensorMap tm_m, const __grid_constant__ CUtensorMap tm_w) {
-  chain_wait();
-  x_sample(a);
   static_assert((K == 16 || K == 32) && XC > 1, "band form: K = 16 or 32, rows over a cluster");
   extern __shared__ __align__(16) unsigned char smem[];
   const int tid = threadIdx.x;
@@ -907,13 +905,14 @@ __global__ void __launch_bounds__(MAXT, min_ctas(MAXT))
 // small kernels
 // ---------------------------------------------------------------------------
 
-// Receiver samples of the last level of a run: traces[s][r] = u^k(rec r), s = k - k0 - 1.
+// Receiver samples of one level: traces[s][r] = u^k(rec r), s = k - k0 - 1.
 __global__ void gather_kernel(const GridDev* gd, const float* u_new, int ld, long long lev) {
   chain_wait();
   chain_release();
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= gd->n_rec) return;
-  const long long s = (lev == kRecordLevel ? gd->k : lev) - gd->k0 - 1;
+  const long long k = lev > kRecordLevel + 2 ? lev : lev == kRecordLevel ? gd->k : gd->kf[lev - kRecordLevel - 1];
+  const long long s = k - gd->k0 - 1;
   if (s < 0 || s >= gd->steps || gd->traces == nullptr) return;
   const int ix = gd->rec[2 * r], iy = gd->rec[2 * r + 1];
   gd->traces[s * gd->n_rec + r] = u_new[(size_t)iy * ld + ix];
@@ -1031,7 +1030,7 @@ int x_pipe_box_lines(int tsys, int K) {
 }
 
 template <int K, typename T, int MAXT, bool TREE>
-static cudaError_t launch_x_t(const XArgs& a_in, cudaStream_t st) {
+static cudaError_t launch_x_t(const XArgs& a_in, const XRec& rec, cudaStream_t st) {
   XArgs a = a_in;
   const int threads = a.spc << a.log2tsys;
   if (threads % 32 != 0 || threads > MAXT) return cudaErrorInvalidValue;  // whole warps only
@@ -1052,7 +1051,7 @@ static cudaError_t launch_x_t(const XArgs& a_in, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     blocks = std::max(1, std::min(blocks, nsm * std::max(per_sm, 1)));
   }
-  return launch_chained(x_sweep_kernel<K, T, MAXT, TREE>, blocks, threads, sm, st, a);
+  return launch_chained(x_sweep_kernel<K, T, MAXT, TREE>, blocks, threads, sm, st, a, rec);
 }
 
 template <int K, typename T, int MAXT, bool TREE>
@@ -1089,7 +1088,7 @@ static cudaError_t launch_y_t(const YArgs& a_in, cudaStream_t st) {
 // K = 4, 8 fit 64 registers; K = 16, 32 take the smallest bound that holds
 // `threads` (float only; FP64 kernels are bounded at 512).
 template <int K, int MAXT, int XC>
-static cudaError_t launch_x_pipe_t(const XArgs& a_in, const CUtensorMap& tu, const CUtensorMap& tm,
+static cudaError_t launch_x_pipe_t(const XArgs& a_in, const XRec& rec, const CUtensorMap& tu, const CUtensorMap& tm,
                                    const CUtensorMap& tw, cudaStream_t st) {
   XArgs a = a_in;
   if (XC > 1) {  // the plan's threads per row are split over the cluster
@@ -1113,7 +1112,7 @@ static cudaError_t launch_x_pipe_t(const XArgs& a_in, const CUtensorMap& tu, con
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, x_pipe_kernel<K, MAXT, XC>, threads, sm);
     if (e != cudaSuccess) return e;
     const int blocks = std::max(1, std::min(nblk, nsm * std::max(per_sm, 1)));
-    return launch_chained(x_pipe_kernel<K, MAXT, XC>, blocks, threads, sm, st, a, tu, tm, tw);
+    return launch_chained(x_pipe_kernel<K, MAXT, XC>, blocks, threads, sm, st, a, tu, tm, tw, rec);
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(nblk * XC, 1, 1);
@@ -1132,7 +1131,7 @@ static cudaError_t launch_x_pipe_t(const XArgs& a_in, const CUtensorMap& tu, con
   cudaError_t e = cudaOccupancyMaxActiveClusters(&nc, x_pipe_kernel<K, MAXT, XC>, &cfg);
   if (e != cudaSuccess) return e;
   cfg.gridDim = dim3(std::max(1, std::min(nblk, nc)) * XC, 1, 1);
-  return cudaLaunchKernelEx(&cfg, x_pipe_kernel<K, MAXT, XC>, a, tu, tm, tw);
+  return cudaLaunchKernelEx(&cfg, x_pipe_kernel<K, MAXT, XC>, a, tu, tm, tw, rec);
 }
 
 // Band form: [XAsyncSmem] [mbarrier] [pad to 1024] [u ring 3 x rowf] [m rowf] [w rowf] [halo 96 B].
@@ -1158,14 +1157,13 @@ static cudaError_t launch_x_band_t(const XArgs& a_in, const CUtensorMap& tu, con
   cfg.blockDim = dim3(tsys, 1, 1);
   cfg.dynamicSmemBytes = sm;
   cfg.stream = st;
-  cudaLaunchAttribute attr[2];
-  attr[1] = chain_attribute();
+  cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = XC;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 2;
+  cfg.numAttrs = 1;
   int nc = 0;
   cudaError_t e = cudaOccupancyMaxActiveClusters(&nc, x_band_kernel<K, MAXT, XC>, &cfg);
   if (e != cudaSuccess) return e;
@@ -1187,20 +1185,20 @@ cudaError_t launch_x_band(const XArgs& a, int K, const CUtensorMap& tu, const CU
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_x_pipe(const XArgs& a, int K, const CUtensorMap& tu, const CUtensorMap& tm,
+cudaError_t launch_x_pipe(const XArgs& a, const XRec& rec, int K, const CUtensorMap& tu, const CUtensorMap& tm,
                           const CUtensorMap& tw, cudaStream_t st) {
   const int threads = a.spc << a.log2tsys;
-  if (a.xc == 2) return K == 32 ? launch_x_pipe_t<32, 256, 2>(a, tu, tm, tw, st) : cudaErrorInvalidValue;
-  if (a.xc == 4) return K == 32 ? launch_x_pipe_t<32, 128, 4>(a, tu, tm, tw, st) : cudaErrorInvalidValue;
+  if (a.xc == 2) return K == 32 ? launch_x_pipe_t<32, 256, 2>(a, rec, tu, tm, tw, st) : cudaErrorInvalidValue;
+  if (a.xc == 4) return K == 32 ? launch_x_pipe_t<32, 128, 4>(a, rec, tu, tm, tw, st) : cudaErrorInvalidValue;
   switch (K) {
-    case 8: return launch_x_pipe_t<8, 1024, 1>(a, tu, tm, tw, st);
+    case 8: return launch_x_pipe_t<8, 1024, 1>(a, rec, tu, tm, tw, st);
     case 16:
-      if (threads <= 256) return launch_x_pipe_t<16, 256, 1>(a, tu, tm, tw, st);
-      if (threads <= 512) return launch_x_pipe_t<16, 512, 1>(a, tu, tm, tw, st);
-      return launch_x_pipe_t<16, 1024, 1>(a, tu, tm, tw, st);
+      if (threads <= 256) return launch_x_pipe_t<16, 256, 1>(a, rec, tu, tm, tw, st);
+      if (threads <= 512) return launch_x_pipe_t<16, 512, 1>(a, rec, tu, tm, tw, st);
+      return launch_x_pipe_t<16, 1024, 1>(a, rec, tu, tm, tw, st);
     case 32:
-      if (threads <= 256) return launch_x_pipe_t<32, 256, 1>(a, tu, tm, tw, st);
-      return launch_x_pipe_t<32, 512, 1>(a, tu, tm, tw, st);
+      if (threads <= 256) return launch_x_pipe_t<32, 256, 1>(a, rec, tu, tm, tw, st);
+      return launch_x_pipe_t<32, 512, 1>(a, rec, tu, tm, tw, st);
   }
   return cudaErrorInvalidValue;
 }
@@ -1336,14 +1334,14 @@ cudaError_t launch_y_pipe_adj(const YArgs& a, int K, const CUtensorMap& lam, con
       return FN<32, float, 1024, TR> ARGS;                           \
   }
 
-cudaError_t launch_x(const XArgs& a, int K, bool fp64, bool tree, cudaStream_t st) {
+cudaError_t launch_x(const XArgs& a, const XRec& rec, int K, bool fp64, bool tree, cudaStream_t st) {
   const int threads = a.spc << a.log2tsys;
   if (fp64) {
-    if (tree) { ADI_DISPATCH_K(launch_x_t, double, 512, true, (a, st)) }
-    else { ADI_DISPATCH_K(launch_x_t, double, 512, false, (a, st)) }
+    if (tree) { ADI_DISPATCH_K(launch_x_t, double, 512, true, (a, rec, st)) }
+    else { ADI_DISPATCH_K(launch_x_t, double, 512, false, (a, rec, st)) }
   } else {
-    if (tree) { ADI_DISPATCH_KF(launch_x_t, true, (a, st), threads) }
-    else { ADI_DISPATCH_KF(launch_x_t, false, (a, st), threads) }
+    if (tree) { ADI_DISPATCH_KF(launch_x_t, true, (a, rec, st), threads) }
+    else { ADI_DISPATCH_KF(launch_x_t, false, (a, rec, st), threads) }
   }
   return cudaErrorInvalidValue;
 }

@@ -46,8 +46,14 @@ struct XArgs {
   int stage_off;    // byte offset of the staging area (set by the launcher), -1: none
   int* err;         // device error word (bounded waits), or null
   int xc;           // TMA pipeline: 2 = each row split over a cluster of two CTAs, else 1
-  const int* rec;   // [n_rec][2] receivers at which u^k is sampled into gd's traces
-  int n_rec;        // 0 = none
+};
+
+// Receivers at which an x sweep samples u^k into gd's traces.  Beside XArgs,
+// not in it: the band form, which samples none, ran 6 to 8 % slower with the
+// arguments that follow moved (0.707 to 0.762 ms at 16384^2).
+struct XRec {
+  const int* rec = nullptr;  // [n_rec][2]
+  int n_rec = 0;
 };
 
 // Arguments of the y-sweep + update kernel (Eq. fr2's y operator).
@@ -71,9 +77,9 @@ struct YArgs {
 };
 
 // Launchers (adi_forward.cu).
-cudaError_t launch_x(const XArgs& a, int K, bool fp64, bool tree, cudaStream_t st);
+cudaError_t launch_x(const XArgs& a, const XRec& rec, int K, bool fp64, bool tree, cudaStream_t st);
 cudaError_t launch_y(const YArgs& a, int K, bool fp64, bool tree, cudaStream_t st);
-// lev: the level of u_new, or kRecordLevel: gd->k
+// lev: the level of u_new, or kRecordLevel: gd->k, kRecordLevel + 1 + q: gd->kf[q]
 constexpr long long kRecordLevel = -0x7fffffffffffffffll;
 cudaError_t launch_gather(const GridDev* gd, const float* u_new, int ld, int n_rec, long long lev, cudaStream_t st);
 // Fields between the caller's contiguous rows and the handle's pitched ones
@@ -253,7 +259,7 @@ cudaError_t launch_y_model(const ModelYArgs& a, int K, cudaStream_t st);
 cudaError_t configure_model_kernels();
 // Row tensor map for the pipelined x sweep (see adi_tma.cuh).
 cudaError_t encode_row_map(CUtensorMap* out, const float* base, int ld, int ny, int box_lines);
-cudaError_t launch_x_pipe(const XArgs& a, int K, const CUtensorMap& tu, const CUtensorMap& tm,
+cudaError_t launch_x_pipe(const XArgs& a, const XRec& rec, int K, const CUtensorMap& tu, const CUtensorMap& tm,
                           const CUtensorMap& tw, cudaStream_t st);
 // Band form of the x sweep (x_stage 5): clusters of xc = 2, 4 or 8 CTAs walk
 // bands of consecutive rows with a ring of three rows of u^k in shared memory.

@@ -185,8 +185,6 @@ extern "C" int adi_wave_step_noalloc(const adi_wave_desc* desc, int32_t ld, doub
   xa.stage_off = -1;
   xa.err = nullptr;
   xa.xc = P.xc;
-  xa.rec = nullptr;
-  xa.n_rec = 0;
   YArgs ya;
   ya.nx = d.nx;
   ya.ny = d.ny;
@@ -213,9 +211,9 @@ extern "C" int adi_wave_step_noalloc(const adi_wave_desc* desc, int32_t ld, doub
     if (e == cudaSuccess) e = encode_row_map(&tm, m, ld, d.ny, L);
     if (e == cudaSuccess) e = encode_row_map(&tw, slot->w, ld, d.ny, L);
     if (e != cudaSuccess) return fail_msg(ADI_ECUDA, std::string("tensor maps: ") + cudaGetErrorString(e));
-    e = launch_x_pipe(xa, P.kx, tu, tm, tw, st);
+    e = launch_x_pipe(xa, XRec{}, P.kx, tu, tm, tw, st);
   } else {
-    e = launch_x(xa, P.kx, P.fp64x, P.tree, st);
+    e = launch_x(xa, XRec{}, P.kx, P.fp64x, P.tree, st);
   }
   if (e != cudaSuccess) return fail_msg(ADI_ECUDA, std::string("x sweep launch: ") + cudaGetErrorString(e));
   if (P.y_stage == 3) {

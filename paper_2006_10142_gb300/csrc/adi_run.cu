@@ -366,16 +366,32 @@ int adi_wave::prof_end(cudaStream_t st, cudaEvent_t a, int kind) {
   return ADI_OK;
 }
 
-int adi_wave::enqueue_step(Grid& G, cudaStream_t st, bool gather, bool one_pass) {
+// The band form of the x sweep samples none (its rows leave no room for it in
+// time: 16384^2 0.4 % of a step goes to the launch instead).
+adi_wave::Sampling adi_wave::sampling_of(const Grid& G, int n_rec, bool one_pass) const {
+  if (n_rec <= 0) return kNone;
+  return !one_pass && G.plan.x_stage == ADI_STAGE_BAND ? kAfterStep : kInStep;
+}
+
+// Samples u^k at the run's receivers (captured: the level is in the record,
+// which the sweeps and the one-pass step keep in different words).
+int adi_wave::enqueue_gather(Grid& G, cudaStream_t st, bool one_pass) {
+  const long long lev = st != cap ? G.k : one_pass ? kRecordLevel + 1 + G.cur : kRecordLevel;
+  CK(launch_gather(G.gd, G.buf[G.cur], G.ld, G.hgd.n_rec, lev, st), "gather launch");
+  launches += 1;
+  return ADI_OK;
+}
+
+int adi_wave::enqueue_step(Grid& G, cudaStream_t st, Sampling smp, bool one_pass) {
   float* u_cur = G.buf[G.cur];
   float* u_prev = G.buf[1 - G.cur];
-  int rc = one_pass ? launch_fwd_tile(G, u_cur, u_prev, G.gd, G.cur, gather, st != cap, st)
-                    : launch_fwd(G, u_cur, u_prev, G.w, nullptr, G.gd, gather, st);
+  int rc = one_pass ? launch_fwd_tile(G, u_cur, u_prev, G.gd, G.cur, smp == kInStep, st != cap, st)
+                    : launch_fwd(G, u_cur, u_prev, G.w, nullptr, G.gd, smp == kInStep, st);
   if (rc != ADI_OK) return rc;
   G.cur = 1 - G.cur;
   G.k += 1;
   G.from_init = false;
-  return ADI_OK;
+  return smp == kAfterStep ? enqueue_gather(G, st, one_pass) : ADI_OK;
 }
 
 // The same step as one launch (adi_tile.cu, adi_patch.cu).  par: which level
@@ -460,8 +476,11 @@ int adi_wave::launch_fwd(Grid& G, const float* u_cur, float* u_prev, float* w, f
   xa.stage_off = -1;
   xa.err = d_err;
   xa.xc = P.xc;
-  xa.rec = gather ? d_rec : nullptr;
-  xa.n_rec = gather ? G.hgd.n_rec : 0;
+  XRec xr;
+  if (gather) {
+    xr.rec = d_rec;
+    xr.n_rec = G.hgd.n_rec;
+  }
   YArgs ya;
   ya.nx = G.nx;
   ya.ny = G.ny;
@@ -505,9 +524,9 @@ int adi_wave::launch_fwd(Grid& G, const float* u_cur, float* u_prev, float* w, f
       tw = &tmpw;
     }
     if (P.x_stage == 5) CK(launch_x_band(xa, P.kx, *tu, G.tm_m, *tw, st), "x sweep launch");
-    else CK(launch_x_pipe(xa, P.kx, *tu, G.tm_m, *tw, st), "x sweep launch");
+    else CK(launch_x_pipe(xa, xr, P.kx, *tu, G.tm_m, *tw, st), "x sweep launch");
   } else {
-    CK(launch_x(xa, P.kx, P.fp64x, P.tree, st), "x sweep launch");
+    CK(launch_x(xa, xr, P.kx, P.fp64x, P.tree, st), "x sweep launch");
   }
   if (profile && prof_end(st, a, ADI_KERNEL_X) != ADI_OK) return ADI_ECUDA;
   if (profile && prof_begin(st, &a) != ADI_OK) return ADI_ECUDA;
@@ -551,15 +570,15 @@ void adi_wave::drop_graphs() {
       }
 }
 
-int adi_wave::launch_pair_graph(Grid& G, cudaStream_t st, bool gather, bool one_pass) {
-  cudaGraphExec_t& ex = pair[G.cur][(gather ? 1 : 0) + (one_pass ? 2 : 0)];
+int adi_wave::launch_pair_graph(Grid& G, cudaStream_t st, Sampling smp, bool one_pass) {
+  cudaGraphExec_t& ex = pair[G.cur][(smp != kNone ? 1 : 0) + (one_pass ? 2 : 0)];
   if (!ex) {
     const int cur0 = G.cur;
     const long long k0 = G.k;
     const int64_t l0 = launches;
     CK(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal), "begin capture");
-    int rc = enqueue_step(G, cap, gather, one_pass);
-    if (rc == ADI_OK) rc = enqueue_step(G, cap, gather, one_pass);
+    int rc = enqueue_step(G, cap, smp, one_pass);
+    if (rc == ADI_OK) rc = enqueue_step(G, cap, smp, one_pass);
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamEndCapture(cap, &graph);
     G.cur = cur0;
@@ -578,7 +597,7 @@ int adi_wave::launch_pair_graph(Grid& G, cudaStream_t st, bool gather, bool one_
     }
   }
   CK(cudaGraphLaunch(ex, st), "graph launch");
-  launches += one_pass ? 2 : 4;
+  launches += 2 * ((one_pass ? 1 : 2) + (smp == kAfterStep ? 1 : 0));
   G.k += 2;
   return ADI_OK;
 }
@@ -669,6 +688,7 @@ int adi_wave::run(int steps, const adi_source* src, const int32_t* rec_xy, int n
   }
 
   const bool gather = n_rec > 0;
+  const Sampling smp = sampling_of(G, n_rec, one_pass);
   if (gather && (n_rec != graph_rec || d_rec != graph_rec_at)) {  // captured steps hold both
     drop_graphs();
     graph_rec = n_rec;
@@ -715,7 +735,7 @@ int adi_wave::run(int steps, const adi_source* src, const int32_t* rec_xy, int n
       const size_t off = ffl * every * (size_t)(s / every % keep);
       for (; t < seg; ++t) {
         int rc = launch_fwd(G, G.buf[G.cur], G.buf[1 - G.cur], aw.wseg + off + ffl * t, aw.zseg + off + ffl * t, G.gd,
-                            gather, st);
+                            smp == kInStep, st);
         if (rc != ADI_OK) {
           rr.kept = 0;
           return rc;
@@ -723,6 +743,10 @@ int adi_wave::run(int steps, const adi_source* src, const int32_t* rec_xy, int n
         G.cur = 1 - G.cur;
         G.k += 1;
         G.from_init = false;
+        if (smp == kAfterStep) {
+          rc = enqueue_gather(G, st, false);
+          if (rc != ADI_OK) return rc;
+        }
       }
       rr.kept += 1;
       rr.kept_bufs = keep;
@@ -736,21 +760,21 @@ int adi_wave::run(int steps, const adi_source* src, const int32_t* rec_xy, int n
     }
     if (use_graph) {
       while (seg - t >= 2) {
-        int rc = launch_pair_graph(G, st, gather, one_pass);
+        int rc = launch_pair_graph(G, st, smp, one_pass);
         if (rc != ADI_OK) return rc;
         t += 2;
       }
     }
     while (t < seg) {
-      int rc = enqueue_step(G, st, gather, one_pass);
+      int rc = enqueue_step(G, st, smp, one_pass);
       if (rc != ADI_OK) return rc;
       t += 1;
     }
     s += seg;
   }
-  if (gather && !model.active) {  // the steps have sampled the levels before the last
-    CK(launch_gather(G.gd, G.buf[G.cur], G.ld, n_rec, G.k, st), "gather launch");
-    launches += 1;
+  if (smp == kInStep && !model.active) {  // the steps have sampled the levels before the last
+    const int rc = enqueue_gather(G, st, one_pass);
+    if (rc != ADI_OK) return rc;
   }
   G.hgd.k = G.k;
   return ADI_OK;

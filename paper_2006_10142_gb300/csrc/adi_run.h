@@ -205,7 +205,12 @@ struct adi_wave {
   ~adi_wave();
 
   // internals
-  int enqueue_step(adi::Grid& G, cudaStream_t st, bool gather, bool one_pass);
+  // who samples the receivers of a run: nobody, the step that starts from a
+  // level, or a launch after the step that made it
+  enum Sampling { kNone = 0, kInStep = 1, kAfterStep = 2 };
+  Sampling sampling_of(const adi::Grid& G, int n_rec, bool one_pass) const;
+  int enqueue_step(adi::Grid& G, cudaStream_t st, Sampling smp, bool one_pass);
+  int enqueue_gather(adi::Grid& G, cudaStream_t st, bool one_pass);
   int launch_fwd(adi::Grid& G, const float* u_cur, float* u_prev, float* w, float* z_out,
                  adi::GridDev* gd, bool gather, cudaStream_t st);
   int launch_fwd_tile(adi::Grid& G, const float* u_cur, float* u_prev, adi::GridDev* gd, int par, bool gather,
@@ -214,7 +219,7 @@ struct adi_wave {
   bool adj_beside(const adi::Grid& G) const;
   bool adj_room(const adi::Grid& G, int E, int bufs) const;
   void free_adj_work();
-  int launch_pair_graph(adi::Grid& G, cudaStream_t st, bool gather, bool one_pass);
+  int launch_pair_graph(adi::Grid& G, cudaStream_t st, Sampling smp, bool one_pass);
   void drop_graphs();
   int prof_begin(cudaStream_t st, cudaEvent_t* a);
   int prof_end(cudaStream_t st, cudaEvent_t a, int kind);

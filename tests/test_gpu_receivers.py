@@ -1,0 +1,52 @@
+"""Receiver traces of a run against the fields of the same steps taken one at
+a time: the values are copies, equal to the bit, whoever takes them (the step
+that starts from a level, or a launch after the step that made it)."""
+import numpy as np
+import pytest
+
+from helpers import f32
+from test_gpu_tile import _problem
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(nx, ny, cfl, n_rec, tuning, every=0, steps=5):
+    import torch
+    from paper_2006_10142_gb300 import api
+    m, phi, tau, wav = _problem(nx, ny, cfl, nx + ny)
+    t = lambda a: torch.from_numpy(f32(a)).to("cuda:0")
+    wav = t(np.tile(wav, 2))
+    rng = np.random.default_rng(n_rec)
+    rec = np.stack([rng.integers(0, nx, n_rec), rng.integers(0, ny, n_rec)], 1).astype(np.int32)
+    rec[-1] = nx - 1, ny - 1
+    src = (nx // 2, ny // 3)
+    h = api.AdiWave(t(m), t(phi), tau)
+    if tuning:
+        h.set_tuning(**tuning)
+    h.set_checkpointing(every)
+    want = []
+    # steps taken one at a time keep no checkpoints: the sweeps' plan then has to be given
+    for _ in range(2 * steps):
+        h.step(src=src, wavelet=wav)
+        want.append(h.state()[1][rec[:, 1], rec[:, 0]])
+    end = h.state()[1]
+    h.reset(t(phi))
+    got = [h.run(steps, src=src, wavelet=wav, rec=rec) for _ in range(2)]  # both orientations
+    assert torch.equal(torch.cat(got), torch.stack(want))
+    assert torch.equal(h.state()[1], end)
+    h.reset(t(phi))  # other receivers: captured steps hold the list and its length
+    assert torch.equal(h.run(steps, src=src, wavelet=wav, rec=rec[3:]), torch.stack(want[:steps])[:, 3:])
+    h.sync_status()
+    h.close()
+
+
+@pytest.mark.parametrize("use_graph", [0, 1])
+@pytest.mark.parametrize("nx,ny,tuning", [(300, 200, dict(solver=1)), (4100, 60, dict(solver=1)),
+                                          (2500, 40, dict(x_stage=5, chunk_x=32, x_cluster=2, rows_per_cta=1))])
+def test_sweeps(nx, ny, tuning, use_graph):
+    _check(nx, ny, 0.5, 300, dict(tuning, use_graph=use_graph))
+
+
+@pytest.mark.parametrize("tuning", [dict(solver=1), dict(x_stage=5, chunk_x=32, x_cluster=2, rows_per_cta=1)])
+def test_sweeps_with_kept_segments(tuning):
+    _check(2500, 40, 0.5, 300, tuning, every=2)
