@@ -908,7 +908,6 @@ __global__ void __launch_bounds__(MAXT, min_ctas(MAXT))
 // Receiver samples of one level: traces[s][r] = u^k(rec r), s = k - k0 - 1.
 __global__ void gather_kernel(const GridDev* gd, const float* u_new, int ld, long long lev) {
   chain_wait();
-  chain_release();
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= gd->n_rec) return;
   const long long k = lev > kRecordLevel + 2 ? lev : lev == kRecordLevel ? gd->k : gd->kf[lev - kRecordLevel - 1];

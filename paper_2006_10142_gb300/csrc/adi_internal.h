@@ -191,6 +191,7 @@ struct TileMaps {
 // the couplings decay too slowly.
 int tile_halo(double s_max);
 int tile_strips(int nx);
+int tile_threads();  // per CTA
 // rows of a band, or 0 = by patches
 int tile_band_rows(int nx, int ny, int H, int nsm);
 cudaError_t encode_tile_map(CUtensorMap* out, const float* base, int nx, int ld, int ny, bool strip);
@@ -199,6 +200,7 @@ cudaError_t configure_tile_kernels();
 // The same step patch by patch (adi_patch.cu).
 int patch_rows(int H);
 int patch_strips(int nx);
+int patch_threads();
 int small_patch_strips(int nx);
 cudaError_t encode_patch_map(CUtensorMap* out, const float* base, int nx, int ld, int ny, bool u);
 cudaError_t launch_patch(const TileArgs& a, int H, const CUtensorMap& u, const CUtensorMap& m, cudaStream_t st);

@@ -169,7 +169,8 @@ struct Source {
 // which the next step waits for: look() finds the receivers of the CTA before
 // chain_wait() -- their list is not written during a run -- and sample()
 // copies the values while the stage is on its way.  1000^2 with 64 receivers:
-// 8.0 against 10.1 us per step.
+// 8.0 against 10.1 us per step.  Long lists are left to a launch after the step
+// (adi_wave::sampling_of).
 struct Sampler {
   int at;  // the node of receiver threadIdx.x, -1 = none of this CTA's
   static __device__ __forceinline__ int node(const TileArgs& a, int r, int x0, int x1, int y0, int y1) {

@@ -542,6 +542,7 @@ __global__ void __launch_bounds__(kPN, 2)
 // host
 // ---------------------------------------------------------------------------
 int patch_rows(int H) { return kPR - 2 * H; }
+int patch_threads() { return kPN; }
 int patch_strips(int nx) { return (nx + kPX - 1) / kPX; }
 int small_patch_strips(int nx) { return (nx + kSX - 1) / kSX; }
 

@@ -366,11 +366,19 @@ int adi_wave::prof_end(cudaStream_t st, cudaEvent_t a, int kind) {
   return ADI_OK;
 }
 
-// The band form of the x sweep samples none (its rows leave no room for it in
-// time: 16384^2 0.4 % of a step goes to the launch instead).
+// In the step as long as that costs less than a launch of its own.  Every CTA
+// of the one-pass step goes through the whole list: eight entries per thread
+// at most.  The x sweep's CTAs share it; its band form samples none.  us per
+// step, in the step and by a launch: 128^2 (2.7 without receivers) 2048
+// receivers 4.7, 4096 6.9 and 4.4; 1000^2 (7.5) 2048 9.0, 4096 10.8 and 9.7,
+// 65536 62 and 11; 3001 x 1501 (21) 1024 22.9, 2048 24.6 and 22.9, 10^6 1950
+// and 29; sweeps at 500 x 400 (10.4) 16384 11.9, 65536 14.9 and 11.9.
 adi_wave::Sampling adi_wave::sampling_of(const Grid& G, int n_rec, bool one_pass) const {
   if (n_rec <= 0) return kNone;
-  return !one_pass && G.plan.x_stage == ADI_STAGE_BAND ? kAfterStep : kInStep;
+  const GridPlan& P = G.plan;
+  const int most = one_pass ? 8 * (P.tile_rows > 0 ? tile_threads() : patch_threads())
+                            : P.x_stage == ADI_STAGE_BAND ? 0 : 16384;
+  return n_rec <= most ? kInStep : kAfterStep;
 }
 
 // Samples u^k at the run's receivers (captured: the level is in the record,

@@ -421,6 +421,7 @@ int tile_halo(double s_max) {
   return 0;
 }
 
+int tile_threads() { return kTN; }
 int tile_strips(int nx) { return (nx + kTX - 1) / kTX; }
 
 // Bands or patches (of 96 columns), and the rows of a band.  Times in us as measured on 152

@@ -50,3 +50,33 @@ def test_sweeps(nx, ny, tuning, use_graph):
 @pytest.mark.parametrize("tuning", [dict(solver=1), dict(x_stage=5, chunk_x=32, x_cluster=2, rows_per_cta=1)])
 def test_sweeps_with_kept_segments(tuning):
     _check(2500, 40, 0.5, 300, tuning, every=2)
+
+
+# small patches (256 threads a CTA), patches (256) and bands (128): up to eight
+# receivers per thread in the step, more after it
+@pytest.mark.parametrize("use_graph", [0, 1])
+@pytest.mark.parametrize("nx,ny,n_rec", [(100, 75, 2048), (100, 75, 2049), (1000, 700, 2048), (1000, 700, 9000),
+                                         (2305, 2321, 1024), (2305, 2321, 1025)])
+def test_one_pass_step(nx, ny, n_rec, use_graph):
+    _check(nx, ny, 0.5, n_rec, dict(use_graph=use_graph))
+
+
+@pytest.mark.parametrize("n_rec", [16384, 16385])
+def test_sweeps_with_many(n_rec):
+    _check(300, 200, 0.5, n_rec, dict(solver=1))
+
+
+def test_many_receivers_are_sampled_by_a_launch_of_their_own():
+    """Every CTA of a one-pass step would go through the list otherwise."""
+    import torch
+    from paper_2006_10142_gb300 import api
+    dev = torch.device("cuda:0")
+    n, steps = 300, 4
+    h = api.AdiWave(torch.ones(n, n, device=dev), torch.zeros(n, n, device=dev), 0.5 / (n + 1))
+    count = []
+    for n_rec in (2048, 2049):
+        before = h.launch_count()
+        h.run(steps, rec=np.zeros((n_rec, 2), dtype=np.int32))
+        count.append(h.launch_count() - before)
+    assert count[1] - count[0] == steps - 1  # the last level has one either way
+    h.close()
