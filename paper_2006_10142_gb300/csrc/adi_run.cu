@@ -157,6 +157,49 @@ int adi_wave::create(const adi_wave_desc* desc, int n, const float* const* m,
   return ADI_OK;
 }
 
+// Two steps of every shot (rest: of those the one-launch step leaves) as a
+// graph, from the present orientation.
+int adi_wave::capture_batch_pair(cudaGraphExec_t* ex, bool rest) {
+  std::vector<int> cur0;
+  std::vector<long long> k0;
+  std::vector<char> init0;
+  for (Grid& G : g) {
+    cur0.push_back(G.cur);
+    k0.push_back(G.k);
+    init0.push_back(G.from_init);
+  }
+  const int64_t l0 = launches;
+  CK(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal), "begin capture");
+  int rc = ADI_OK;
+  if (batch_mode == 2) {
+    rc = enqueue_batch_steps_parallel(2, cap, rest);  // per-shot chains of two steps
+  } else {
+    rc = enqueue_batch_step(cap);
+    if (rc == ADI_OK) rc = enqueue_batch_step(cap);
+  }
+  cudaGraph_t graph = nullptr;
+  cudaError_t e = cudaStreamEndCapture(cap, &graph);
+  for (size_t s = 0; s < g.size(); ++s) {
+    g[s].cur = cur0[s];
+    g[s].k = k0[s];
+    g[s].from_init = init0[s];
+  }
+  pair_launches = launches - l0;
+  launches = l0;
+  if (rc != ADI_OK) {
+    if (graph) cudaGraphDestroy(graph);
+    return rc;
+  }
+  if (e != cudaSuccess) return cuda_fail(this, e, "end capture");
+  e = cudaGraphInstantiate(ex, graph, 0);
+  cudaGraphDestroy(graph);
+  if (e != cudaSuccess) {
+    *ex = nullptr;
+    return cuda_fail(this, e, "graph instantiate");
+  }
+  return ADI_OK;
+}
+
 // Batched run: every shot advances `steps` steps; one persistent launch per
 // step (or the plain kernels per shot in batch mode 1), step pairs replayed
 // from a captured graph.
@@ -202,35 +245,8 @@ int adi_wave::run_batch(int steps, const adi_source* src, cudaStream_t st) {
     while (steps - t >= 2) {
       cudaGraphExec_t& ex = pair[g[0].cur][0];
       if (!ex) {
-        std::vector<int> cur0;
-        std::vector<long long> k0;
-        for (Grid& G : g) { cur0.push_back(G.cur); k0.push_back(G.k); }
-        const int64_t l0 = launches;
-        CK(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal), "begin capture");
-        int rc = ADI_OK;
-        if (batch_mode == 2) {
-          rc = enqueue_batch_steps_parallel(2, cap);  // per-shot chains of two steps
-        } else {
-          rc = enqueue_batch_step(cap);
-          if (rc == ADI_OK) rc = enqueue_batch_step(cap);
-        }
-        cudaGraph_t graph = nullptr;
-        cudaError_t e = cudaStreamEndCapture(cap, &graph);
-        for (size_t s = 0; s < g.size(); ++s) { g[s].cur = cur0[s]; g[s].k = k0[s]; }
-        const int64_t per_pair = launches - l0;
-        launches = l0;
-        if (rc != ADI_OK) {
-          if (graph) cudaGraphDestroy(graph);
-          return rc;
-        }
-        if (e != cudaSuccess) return cuda_fail(this, e, "end capture");
-        e = cudaGraphInstantiate(&ex, graph, 0);
-        cudaGraphDestroy(graph);
-        if (e != cudaSuccess) {
-          ex = nullptr;
-          return cuda_fail(this, e, "graph instantiate");
-        }
-        pair_launches = per_pair;
+        const int rc = capture_batch_pair(&ex, false);
+        if (rc != ADI_OK) return rc;
       }
       CK(cudaGraphLaunch(ex, st), "graph launch");
       launches += pair_launches;

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <functional>
 #include <string>
 #include <vector>
 
@@ -166,7 +167,9 @@ struct adi_wave {
   std::vector<int> shot_order;  // batch mode 2: shots by decreasing size
   std::vector<int> shot_branch; // batch mode 2: branch of each shot
   int ensure_branches();
-  int enqueue_batch_steps_parallel(int nsteps, cudaStream_t st, bool rest = false);
+  int enqueue_batch_steps_parallel(int nsteps, cudaStream_t st, bool rest = false,
+                                   const std::function<int(int)>& beside = nullptr);
+  int capture_batch_pair(cudaGraphExec_t* ex, bool rest);
   adi::BatchShot* d_shots = nullptr;
   int2* d_items = nullptr;
   int n_items = 0;
@@ -185,6 +188,7 @@ struct adi_wave {
   bool bt_patch = false;
   std::vector<adi::GridPlan> bt_plans;   // plans the tables were made for
   int ensure_batch_tiles();
+  int launch_batch_tiles(int par, cudaStream_t st);
   int run_batch_tiles(int steps, cudaStream_t st);
   int launch_batch_fwd(adi::Grid& G, int cur, cudaStream_t st);
   int run_batch(int steps, const adi_source* src, cudaStream_t st);
