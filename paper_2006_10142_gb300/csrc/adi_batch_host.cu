@@ -171,8 +171,9 @@ int adi_wave::ensure_branches() {
   return ADI_OK;
 }
 
-// Tables of the one-launch step: built on the first run in batch mode 2 and
-// again when a reset has changed a plan.  All such shots take the same form
+// Tables of the one-launch step: built with the handle and again when a reset
+// or a tuning has changed a plan, so that no run allocates (a caller may be
+// capturing it).  All such shots take the same form
 // and the largest halo any of them needs: patches, or bands of the length
 // that gives the shortest step by the times of tile_band_rows(), the longest
 // CTAs first.
@@ -297,6 +298,10 @@ int adi_wave::ensure_batch_tiles() {
   CKB(cudaMemcpyAsync(bt_dev, tiles.data(), sizeof(BatchTile) * tiles.size(), cudaMemcpyHostToDevice, cap), "batch tables");
   CKB(cudaMemcpyAsync(bt_items, list.data(), sizeof(int2) * list.size(), cudaMemcpyHostToDevice, cap), "batch tables");
   CKB(cudaStreamSynchronize(cap), "batch tables");
+  if (tiles.size() < g.size()) {
+    const int rc = ensure_branches();
+    if (rc != ADI_OK) return rc;
+  }
   bt_n = (int)tiles.size();
   bt_n_items = (int)list.size();
   bt_plans = plans;
@@ -326,8 +331,6 @@ int adi_wave::run_batch_tiles(int steps, cudaStream_t st) {
   const bool rest = bt_n < (int)g.size();
   int t = 0;
   if (rest) {
-    const int rc = ensure_branches();
-    if (rc != ADI_OK) return rc;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     CKB(cudaStreamIsCapturing(st, &cs), "capture status");
     if (g[0].plan.graph && !profile && cs == cudaStreamCaptureStatusNone && steps >= 2) {

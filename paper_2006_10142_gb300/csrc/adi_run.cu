@@ -153,8 +153,9 @@ int adi_wave::create(const adi_wave_desc* desc, int n, const float* const* m,
     int rc = start_grid(s, m[s], phi[s], psi ? psi[s] : nullptr, src ? &src[s] : nullptr, st);
     if (rc != ADI_OK) return rc;
   }
-  if (n > 1) return setup_batch(st);
-  return ADI_OK;
+  if (n == 1) return ADI_OK;
+  const int rc = setup_batch(st);
+  return rc == ADI_OK ? ensure_batch_tiles() : rc;
 }
 
 // Two steps of every shot (rest: of those the one-launch step leaves) as a
@@ -354,7 +355,7 @@ int adi_wave::reset(const float* const* m, const float* const* phi, const float*
                         src ? &src[s] : nullptr, st);
     if (rc != ADI_OK) return rc;
   }
-  return ADI_OK;
+  return g.size() > 1 ? ensure_batch_tiles() : ADI_OK;
 }
 
 int adi_wave::prof_begin(cudaStream_t st, cudaEvent_t* a) {
@@ -859,7 +860,7 @@ int adi_wave::set_tuning(const adi_wave_tuning& t) {
   }
   tuning = t;
   drop_graphs();
-  return ADI_OK;
+  return g.size() > 1 ? ensure_batch_tiles() : ADI_OK;
 }
 
 int adi_wave::profile_read(double* ms, int64_t* counts, int n_kinds) {

@@ -45,3 +45,23 @@ def test_mixed_batch_matches_oracle(way):
         assert rel_l2(got[b][1].double().cpu().numpy(), o["u_cur"]) < bound, SHAPES[b]
         assert rel_l2(got[b][0].double().cpu().numpy(), o["u_prev"]) < bound, SHAPES[b]
     B.close()
+
+
+@pytest.mark.parametrize("shapes", [SHAPES, [s for s in SHAPES if s[2] < 1 and s[0] >= 32]])
+def test_first_run_of_a_handle_may_be_captured(shapes):
+    """Its tables are there, and nothing is allocated."""
+    import torch
+    probs = [_problem(nx, ny, cfl, nx + ny) for nx, ny, cfl in shapes]
+    want, t = _batch(probs)
+    want.run(3)
+    B, _ = _batch(probs)
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        B.run(3)
+    graph.replay()
+    B.sync_status()
+    for a, b in zip(_states(B), _states(want)):
+        assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+    B.close()
+    want.close()
