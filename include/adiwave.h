@@ -290,6 +290,22 @@ typedef struct {
 int adi_wave_get_tuning(const adi_wave *h, adi_wave_tuning *t);
 int adi_wave_set_tuning(adi_wave *h, const adi_wave_tuning *t);
 
+/* The form the steps of a shot take, as planned from its size, tau, bound of
+ * m and tuning.  Runs that keep checkpoints, and models, take the sweeps
+ * whatever the form is. */
+enum { ADI_FORM_SWEEPS = 0,        /* x sweep and y sweep */
+       ADI_FORM_BANDS = 1,         /* one launch per step, by bands of rows */
+       ADI_FORM_PATCHES = 2,       /* one launch, patches of 96 columns */
+       ADI_FORM_SMALL_PATCHES = 3  /* one launch, patches of 32 columns */ };
+typedef struct {
+    int32_t form;
+    int32_t halo;            /* unknowns the one-launch step solves beyond its own, 0 = sweeps */
+    int32_t band_rows;       /* rows of a band (ADI_FORM_BANDS) */
+    int32_t fp64_x, fp64_y;  /* sweeps eliminate in FP64 */
+    double m_max;            /* bound of m the plan was made for */
+} adi_wave_plan;
+int adi_wave_get_plan(const adi_wave *h, int32_t shot, adi_wave_plan *p);
+
 /* ---- measurement --------------------------------------------------------
  * With profiling on, the single-grid forward path records a CUDA event pair
  * around every launch of each kernel kind on the launching stream and runs

@@ -42,7 +42,7 @@ EXPORTS = (
     "adi_wave_destroy", "adi_wave_strerror", "adi_wave_last_error", "adi_wave_get_tuning",
     "adi_wave_set_tuning", "adi_wave_profile", "adi_wave_profile_read", "adi_wave_launch_count",
     "adi_wave_version", "adi_wave_set_batch_mode", "adi_wave_set_wait_hook",
-    "adi_wave_step_noalloc", "adi_wave_set_model",
+    "adi_wave_step_noalloc", "adi_wave_set_model", "adi_wave_get_plan",
 )
 
 
@@ -65,6 +65,11 @@ class Tuning(ctypes.Structure):
                 ("cta_threads_y", ctypes.c_int32), ("y_stage", ctypes.c_int32),
                 ("persist", ctypes.c_int32), ("x_stage", ctypes.c_int32),
                 ("x_cluster", ctypes.c_int32)]
+
+
+class Plan(ctypes.Structure):
+    _fields_ = [("form", ctypes.c_int32), ("halo", ctypes.c_int32), ("band_rows", ctypes.c_int32),
+                ("fp64_x", ctypes.c_int32), ("fp64_y", ctypes.c_int32), ("m_max", ctypes.c_double)]
 
 
 class Model(ctypes.Structure):
@@ -120,6 +125,7 @@ def load(build_if_missing: bool = True):
         lib.adi_wave_last_error.restype = ctypes.c_char_p
         lib.adi_wave_get_tuning.argtypes = [P, ctypes.POINTER(Tuning)]
         lib.adi_wave_set_tuning.argtypes = [P, ctypes.POINTER(Tuning)]
+        lib.adi_wave_get_plan.argtypes = [P, i32, ctypes.POINTER(Plan)]
         lib.adi_wave_profile.argtypes = [P, i32]
         lib.adi_wave_profile_read.argtypes = [P, ctypes.POINTER(ctypes.c_double),
                                               ctypes.POINTER(i64), i32]

@@ -74,6 +74,7 @@ class AdiWave:
         _lib.check(rc, None, "adi_wave_init")
         self._h = h
         self._run_keep = []
+        self.ckpt_every = 0
 
     # -- helpers ---------------------------------------------------------------
     def _sources(self, src, wavelet):
@@ -165,6 +166,7 @@ class AdiWave:
 
     def set_checkpointing(self, every: int):
         _lib.check(self._lib.adi_wave_set_checkpointing(self._h, int(every)), self._h)
+        self.ckpt_every = int(every)
 
     def adjoint(self, resid: torch.Tensor, ckpt_every: int = 0, want_wavelet: bool = True,
                 stream=None):
@@ -208,6 +210,15 @@ class AdiWave:
     def set_tuning(self, **kw):
         t = Tuning(**{f: int(kw.get(f, 0)) for f, _ in Tuning._fields_})
         _lib.check(self._lib.adi_wave_set_tuning(self._h, ctypes.byref(t)), self._h, "set_tuning")
+
+    def plan(self) -> dict:
+        """The form of a step (adi_wave_get_plan): form "sweeps", "bands",
+        "patches" or "small_patches", halo, band_rows, fp64_x, fp64_y, m_max."""
+        p = _lib.Plan()
+        _lib.check(self._lib.adi_wave_get_plan(self._h, 0, ctypes.byref(p)), self._h)
+        out = {f: getattr(p, f) for f, _ in _lib.Plan._fields_}
+        out["form"] = ("sweeps", "bands", "patches", "small_patches")[p.form]
+        return out
 
     def profile(self, enable: bool = True):
         _lib.check(self._lib.adi_wave_profile(self._h, int(bool(enable))), self._h)

@@ -6,15 +6,24 @@ threads per CTA, the interface solver (warp-shuffle block CR + PCR, or
 shared-memory CR handing `pcr_size` equations to warp PCR -- the CR-to-PCR
 switch level) and graph replay.
 
-Each candidate runs a few steps of a c = 1 problem of the requested shape
-(the kernels do the same work for any coefficient) with per-kernel CUDA
-events on the launching stream.  The x-sweep and y-sweep knobs act on
+The knobs are those of the separate sweeps.  A step that is one launch
+(``AdiWave.plan()``: form other than "sweeps") has none, and setting any of them
+would take it off that path: there the answer is the empty tuning, without a
+search, unless the runs keep checkpoints and so take the sweeps.
+
+Each candidate runs a few steps of a problem of the requested shape with
+per-kernel CUDA events on the launching stream, at the handle's own tau and
+bound of m (which decide where the elimination is in FP64; beyond that the
+sweeps do the same work for any coefficient), keeping one checkpoint so that
+the sweeps are what is timed.  The x-sweep and y-sweep knobs act on
 different kernels: for each setting of the shared knobs (solver, CR-to-PCR
 switch) the x candidates are timed with the y sweep on automatic, then the
 y candidates with the best x.  The planner's automatic choice is timed
 first and kept unless a searched tuning is faster (an empty tuning dict
-means "automatic").  Results are cached per (device, nx, ny, precision) in a JSON file
-(``$ADIWAVE_TUNE_CACHE`` or ``~/.cache/adiwave/tuning.json``).
+means "automatic").  Results are cached per (device, nx, ny, precision) and
+form of the step in a JSON file (``$ADIWAVE_TUNE_CACHE`` or
+``~/.cache/adiwave/tuning.json``); entries of other versions of this search,
+which may hold knobs for a step that has become one launch, are left alone.
 """
 from __future__ import annotations
 
@@ -33,8 +42,21 @@ def cache_path() -> str:
                           os.path.join(os.path.expanduser("~"), ".cache", "adiwave", "tuning.json"))
 
 
-def _key(device_name: str, nx: int, ny: int, fp64: str) -> str:
-    return "%s|%dx%d|%s" % (device_name, nx, ny, fp64)
+VERSION = 2
+
+
+def _key(device_name: str, nx: int, ny: int, fp64: str, form: str = "") -> str:
+    """form: what _form() says; without it the key of version 1."""
+    key = "%s|%dx%d|%s" % (device_name, nx, ny, fp64)
+    return "%s|v%d|%s" % (key, VERSION, form) if form else key
+
+
+def _form(plan: Dict, ckpt_every: int) -> str:
+    """What a handle's steps are made of: "one launch", or the sweeps and the
+    precision of their eliminations."""
+    if plan["form"] != "sweeps" and not ckpt_every:
+        return "one launch"
+    return "sweeps fp%d fp%d" % tuple(64 if plan[d] else 32 for d in ("fp64_x", "fp64_y"))
 
 
 def _load_cache() -> Dict:
@@ -110,51 +132,67 @@ def search(measure, shared, xs, ys):
 
 
 def tune(nx: int, ny: int, fp64: str = "auto", steps: int = 3, warmup: int = 1,
-         use_cache: bool = True, verbose: bool = False) -> Dict:
-    """Best tuning for an nx x ny grid: {'tuning': {...}, 'x_ms': .., 'y_ms': ..}."""
+         use_cache: bool = True, verbose: bool = False, sim=None) -> Dict:
+    """Best tuning for an nx x ny grid: {'tuning': {...}, 'x_ms': .., 'y_ms': ..}.
+
+    For the steps of the handle ``sim`` if one is given, else for runs without
+    checkpoints at tau = 0.5 h / max c.  x_ms and y_ms are times of the
+    sweeps; for a step of one launch 'step_ms' is its time and they are those
+    of the sweeps that runs with checkpoints take.
+    """
     import torch
 
     from . import api
 
     dev = torch.device("cuda", torch.cuda.current_device())
     name = torch.cuda.get_device_name(dev)
-    key = _key(name, nx, ny, fp64)
+    h = min(1.0 / (nx + 1), 1.0 / (ny + 1))
+    dt, lx, ly, m_max, ckpt = 0.5 * h, 1.0, 1.0, 1.0, 0
+    if sim is not None:
+        m_max, ckpt = sim.plan()["m_max"], sim.ckpt_every
+        dt, lx, ly = sim.dt, sim.lx, sim.ly
+    m = torch.full((ny, nx), m_max, dtype=torch.float32, device=dev)
+    t = api.AdiWave(m, torch.zeros_like(m), dt, lx=lx, ly=ly, fp64=fp64)
+    form = _form(t.plan(), ckpt)
+    key = _key(name, nx, ny, fp64, form)
     cache = _load_cache() if use_cache else {}
     if key in cache:
+        t.close()
         return cache[key]
 
-    m = torch.ones((ny, nx), dtype=torch.float32, device=dev)
-    h = min(1.0 / (nx + 1), 1.0 / (ny + 1))
-    tau = 0.5 * h
-    sim = api.AdiWave(m, torch.zeros_like(m), tau, fp64=fp64)
-    shared, xs, ys = candidates(nx, ny)
+    def timed():
+        t.run(warmup)
+        t.profile(True)
+        t.profile_read()
+        t.run(steps)
+        ms, cnt = t.profile_read()
+        t.profile(False)
+        return [a / max(c, 1) for a, c in zip(ms, cnt)]
 
     def measure(cfg):
         """(x_ms, y_ms) of one tuning, or None when the shape rejects it."""
         try:
-            sim.set_tuning(**cfg)
+            t.set_tuning(**cfg)
         except api.AdiError:
             return None
-        sim.run(warmup)
-        sim.profile(True)
-        sim.profile_read()
-        sim.run(steps)
-        ms, cnt = sim.profile_read()
-        sim.profile(False)
-        if cnt[0] == 0 and cnt[2] > 0:  # one launch does both sweeps: half of it each
-            r = (0.5 * ms[2] / cnt[2], 0.5 * ms[2] / cnt[2])
-        else:
-            r = (ms[0] / max(cnt[0], 1), ms[1] / max(cnt[1], 1))
+        r = tuple(timed()[:2])
         if verbose:
             print(json.dumps({"cfg": cfg, "x_ms": r[0], "y_ms": r[1]}))
         return r
 
-    best = search(measure, shared, xs, ys)
-    sim.sync_status()
-    sim.close()
+    out = {}
+    if form == "one launch":
+        out["step_ms"] = timed()[2]
+    t.set_checkpointing(max(steps, warmup))  # the sweeps, whatever the plan
+    if form == "one launch":
+        best = (0.0, {}) + measure({})
+    else:
+        best = search(measure, *candidates(nx, ny))
+    t.sync_status()
+    t.close()
     if best is None:
         raise RuntimeError("no tuning candidate is valid for %dx%d" % (nx, ny))
-    out = {"tuning": best[1], "x_ms": best[2], "y_ms": best[3]}
+    out.update(tuning=best[1], x_ms=best[2], y_ms=best[3])
     if use_cache:
         cache = _load_cache()
         cache[key] = out
@@ -163,7 +201,10 @@ def tune(nx: int, ny: int, fp64: str = "auto", steps: int = 3, warmup: int = 1,
 
 
 def apply(sim, fp64: str = "auto", **kw) -> Dict:
-    """Tune for sim's grid shape (cached) and set the result on the handle."""
-    res = tune(sim.nx, sim.ny, fp64=fp64, **kw)
+    """Tune for sim's steps (cached) and set the result on the handle."""
+    sim.set_tuning()  # the plan to look at is the automatic one
+    if _form(sim.plan(), sim.ckpt_every) == "one launch":
+        return {"tuning": {}}
+    res = tune(sim.nx, sim.ny, fp64=fp64, sim=sim, **kw)
     sim.set_tuning(**res["tuning"])
     return res

@@ -487,6 +487,19 @@ extern "C" int adi_wave_set_tuning(adi_wave* h, const adi_wave_tuning* t) {
   return h->set_tuning(*t);
 }
 
+extern "C" int adi_wave_get_plan(const adi_wave* h, int32_t shot, adi_wave_plan* p) {
+  if (!h || !p || shot < 0 || shot >= (int)h->g.size()) return ADI_EINVAL;
+  const Grid& G = h->g[shot];
+  const GridPlan& P = G.plan;
+  p->form = !P.tile ? ADI_FORM_SWEEPS : P.tile_rows ? ADI_FORM_BANDS : P.small_patch ? ADI_FORM_SMALL_PATCHES : ADI_FORM_PATCHES;
+  p->halo = P.tile;
+  p->band_rows = P.tile ? P.tile_rows : 0;
+  p->fp64_x = P.fp64x ? 1 : 0;
+  p->fp64_y = P.fp64y ? 1 : 0;
+  p->m_max = G.mmax;
+  return ADI_OK;
+}
+
 extern "C" int adi_wave_profile(adi_wave* h, int32_t enable) {
   if (!h) return ADI_EINVAL;
   h->profile = enable != 0;
