@@ -46,3 +46,63 @@ def test_adjoint_refuses_more_pieces_of_a_column_than_its_top_system_holds():
     h.sync_status()
     assert torch.equal(gm, torch.zeros_like(gm))  # a field at rest
     h.close()
+
+
+def test_use_graph_reports_what_runs_do():
+    import torch
+    from paper_2006_10142_gb300 import _lib, api
+    h = _handle(300, 200, 0.5)
+    for value, reported in ((0, -1), (1, 1), (-1, -1)):
+        h.set_tuning(use_graph=value)
+        assert h.tuning()["use_graph"] == reported
+        assert h.plan()["form"] == "small_patches"  # no knob of the sweeps
+    h.close()
+    m = torch.ones(40, 40, device="cuda:0")
+    B = api.AdiWaveBatch([m, m], [m, m], 0.01)
+    t = _lib.Tuning()
+    _lib.check(B._lib.adi_wave_get_tuning(B._h, t), B._h)
+    assert t.use_graph == 1
+    B.close()
+
+
+@pytest.mark.parametrize("tuning", [dict(solver=1), dict()])
+def test_captured_steps_follow_resets_receivers_and_checkpoints(tuning):
+    """Step pairs replayed from graphs against chained launches, to the bit:
+    a second run, other receivers, a medium that changes nothing in the plan,
+    one that takes the systems to FP64 and back, and runs with checkpoints
+    (whose steps are the sweeps)."""
+    import torch
+    from helpers import f32
+    from paper_2006_10142_gb300 import api
+    from test_gpu_tile import _problem
+    nx, ny, steps = 300, 260, 7
+    m, phi, tau, wav = _problem(nx, ny, 0.5, 5)
+    t = lambda a: torch.from_numpy(f32(a)).to("cuda:0")
+    wav = t(wav)
+    out = []
+    for graph in (1, -1):
+        h = api.AdiWave(t(m), t(phi), tau)
+        h.set_tuning(use_graph=graph, **tuning)
+        got = []
+
+        def run(rec=None):
+            tr = h.run(steps, src=(31, 39), wavelet=wav, rec=rec)
+            got.extend(([] if tr is None else [tr]) + list(h.state()[:2]))
+
+        run()
+        run()
+        run(rec=[[31, 39], [299, 0]])
+        run(rec=[[5, 6], [7, 8], [31, 39]])
+        for scale in (1.3, 100.0, 1.0):
+            h.reset(t(phi), m=t(scale * m))
+            run(rec=[[5, 6], [7, 8], [31, 39]])
+            run()
+        h.set_checkpointing(3)
+        run(rec=[[5, 6]])
+        run()
+        h.set_checkpointing(0)
+        run()
+        h.sync_status()
+        out.append(got)
+        h.close()
+    assert len(out[0]) == len(out[1]) and all(torch.equal(a, b) for a, b in zip(*out))
