@@ -215,11 +215,11 @@ const char *adi_wave_last_error(const adi_wave *h);
  *                   warp-shuffle parallel cyclic reduction (2, 4, 8, 16 or
  *                   32; the CR-to-PCR switch level);
  * use_graph:        1 = replay pairs of steps from a captured CUDA graph, -1 =
- *                   never, 0 = in batches only: there a graph holds many
- *                   shots' sweeps, while a single grid's steps are chained
- *                   launches that overlap one another, also across what would
- *                   be a graph's ends.  Batched steps of one launch have no
- *                   graph;
+ *                   never, 0 = where that is faster: in batches, whose graphs
+ *                   hold many shots' sweeps, and for sweeps of long rows on
+ *                   small grids; other steps are chained launches that overlap
+ *                   one another, also across what would be a graph's ends.
+ *                   Batched steps of one launch have no graph;
  * solver:           ADI_SOLVER_TREE (cyclic reduction of the interface
  *                   system across warp lanes by register shuffles, PCR of the
  *                   warp summaries) or ADI_SOLVER_CR_SMEM (cyclic reduction

@@ -471,7 +471,8 @@ extern "C" int adi_wave_get_tuning(const adi_wave* h, adi_wave_tuning* t) {
   t->rows_per_cta = P.spc;
   t->cols_per_cta = 1 << P.log2W;
   t->pcr_size = P.pcr;
-  t->use_graph = (h->g.size() > 1 ? P.graph != 0 : h->tuning.use_graph > 0) ? 1 : -1;  // as runs do
+  // as runs without checkpoints do
+  t->use_graph = (h->g.size() > 1 ? P.graph != 0 : h->graph_steps(h->g[0], P.tile != 0)) ? 1 : -1;
   t->solver = P.tree ? ADI_SOLVER_TREE : ADI_SOLVER_CR_SMEM;
   t->cta_threads = P.cta_threads;
   t->cta_threads_y = P.cta_threads_y;

@@ -27,6 +27,15 @@ constexpr int kMaxDevices = 64;
 bool g_configured[kMaxDevices] = {};
 std::mutex g_config_mu;
 
+bool stream_captures(cudaStream_t st) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return cs != cudaStreamCaptureStatusNone;
+}
+
 #define CK(call, what)                                          \
   do {                                                          \
     cudaError_t e_ = (call);                                    \
@@ -383,6 +392,16 @@ int adi_wave::prof_end(cudaStream_t st, cudaEvent_t a, int kind) {
   return ADI_OK;
 }
 
+// Whether the steps are replayed as captured pairs.  Launched one by one they
+// overlap, which those on either side of a graph's end do not.  Where the x
+// sweep is the band form, which does not overlap, the graph's shorter gaps
+// win on small grids (us per step at tau = 2h: 8000 x 64 13.4 and 14.4, 16384
+// x 40 19.5 and 20.6, 8000 x 500 50.7 and 51.6; 8192^2 the same either way).
+bool adi_wave::graph_steps(const Grid& G, bool one_pass) const {
+  if (tuning.use_graph != 0) return tuning.use_graph > 0;
+  return !one_pass && !model.active && G.plan.x_stage == ADI_STAGE_BAND && (size_t)G.nx * G.ny <= ((size_t)1 << 22);
+}
+
 // In the step as long as that costs less than a launch of its own.  Every CTA
 // of the one-pass step goes through the whole list: eight entries per thread
 // at most.  The x sweep's CTAs share it; its band form samples none.  us per
@@ -675,7 +694,8 @@ int adi_wave::run(int steps, const adi_source* src, const int32_t* rec_xy, int n
   // gradient is made of differences of nearly equal FP32 fields (z - w), so
   // its last digits follow the rounding of every forward value.
   const bool one_pass = G.plan.tile != 0 && every == 0 && !model.active;
-  const bool use_graph = tuning.use_graph > 0 && !profile;
+  // (a graph cannot be launched into a stream that is being captured)
+  const bool use_graph = graph_steps(G, one_pass) && !profile && !(tuning.use_graph == 0 && stream_captures(st));
   // chained one-pass steps carry level and source by value: without receivers
   // nothing reads the grid record
   if (!one_pass || use_graph || n_rec > 0)

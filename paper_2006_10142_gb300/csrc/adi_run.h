@@ -212,6 +212,7 @@ struct adi_wave {
   // who samples the receivers of a run: nobody, the step that starts from a
   // level, or a launch after the step that made it
   enum Sampling { kNone = 0, kInStep = 1, kAfterStep = 2 };
+  bool graph_steps(const adi::Grid& G, bool one_pass) const;
   Sampling sampling_of(const adi::Grid& G, int n_rec, bool one_pass) const;
   int enqueue_step(adi::Grid& G, cudaStream_t st, Sampling smp, bool one_pass);
   int enqueue_gather(adi::Grid& G, cudaStream_t st, bool one_pass);

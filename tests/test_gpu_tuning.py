@@ -106,3 +106,25 @@ def test_captured_steps_follow_resets_receivers_and_checkpoints(tuning):
         out.append(got)
         h.close()
     assert len(out[0]) == len(out[1]) and all(torch.equal(a, b) for a, b in zip(*out))
+
+
+def test_sweeps_of_long_rows_are_replayed_and_may_be_captured():
+    """Rows of the band form on a small grid: graphs by default, launches in a
+    caller's graph; the same fields."""
+    import torch
+    h = _handle(5000, 40, 2.0)
+    assert h.tuning()["x_stage"] == 5 and h.tuning()["use_graph"] == 1
+    phi = torch.randn(40, 5000, device="cuda:0")
+    h.reset(phi)
+    h.run(5)
+    want = h.state()
+    h.reset(phi)
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        h.run(5)
+    graph.replay()
+    got = h.state()
+    h.sync_status()
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+    h.close()
