@@ -331,6 +331,14 @@ y_done:
         nsm = 152;
       P.small_patch = small_patch_strips(G.nx) * ((G.ny + patch_rows(P.tile) - 1) / patch_rows(P.tile)) <= 2 * nsm;
       P.tile_rows = P.small_patch ? 0 : tile_band_rows(G.nx, G.ny, P.tile, nsm);
+      // Except where three waves do not hold the patches of a grid that fills
+      // little of them: a third of the columns and, with the halo of 16, half
+      // of the rows (tau = h / max c, us per step, one pass and sweeps: 32 x
+      // 32000 25.1 and 21.1, 33 x 32000 30.0 and 28.0, 33 x 20000 22.1 and
+      // 24.6, 48 x 32000 25.3 and 26.4).
+      if (P.tile == 16 && !P.small_patch && P.tile_rows == 0 && G.nx < 40 &&
+          (G.ny + patch_rows(16) - 1) / patch_rows(16) > 3 * 2 * nsm)
+        P.tile = 0;
     }
   }
   G.plan = P;

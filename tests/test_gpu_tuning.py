@@ -128,3 +128,11 @@ def test_sweeps_of_long_rows_are_replayed_and_may_be_captured():
     h.sync_status()
     assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
     h.close()
+
+
+@pytest.mark.parametrize("nx,ny,cfl,form", [(32, 32000, 1.0, "sweeps"), (32, 32000, 0.5, "patches"),
+                                            (33, 20000, 1.0, "patches"), (48, 32000, 1.0, "patches")])
+def test_narrow_grids_of_many_patches_keep_the_sweeps(nx, ny, cfl, form):
+    h = _handle(nx, ny, cfl)
+    assert h.plan()["form"] == form
+    h.close()
