@@ -666,15 +666,22 @@ int adi_wave::run(int steps, const adi_source* src, const int32_t* rec_xy, int n
   if (steps == 0) return ADI_OK;
 
   // per-run device state: level, source, receivers
+  // (a caller's graph that holds the copy reads both ends at every replay)
+  const int32_t* rec_host = rec_xy;
+  if (n_rec > 0 && stream_captures(st)) {
+    graph_recs.emplace_back(rec_xy, rec_xy + 2 * (size_t)n_rec);
+    rec_host = graph_recs.back().data();
+  }
   if (n_rec > rec_cap) {
-    if (d_rec) cudaFree(d_rec);
+    if (d_rec && !graph_recs.empty()) graph_recs_dev.push_back(d_rec);
+    else if (d_rec) cudaFree(d_rec);
     d_rec = nullptr;
     rec_cap = 0;
     CK(cudaMalloc(&d_rec, sizeof(int) * 2 * (size_t)n_rec), "alloc receivers");
     rec_cap = n_rec;
   }
   if (n_rec > 0)
-    CK(cudaMemcpyAsync(d_rec, rec_xy, sizeof(int) * 2 * (size_t)n_rec, cudaMemcpyHostToDevice, st),
+    CK(cudaMemcpyAsync(d_rec, rec_host, sizeof(int) * 2 * (size_t)n_rec, cudaMemcpyHostToDevice, st),
        "copy receivers");
   const adi_source none = {-1, -1, nullptr, 0};
   const adi_source sr = src ? src[0] : none;
@@ -921,6 +928,7 @@ adi_wave::~adi_wave() {
   if (d_err) cudaFree(d_err);
   if (scan_host) cudaFreeHost(const_cast<unsigned int*>(scan_host));
   if (d_rec) cudaFree(d_rec);
+  for (int* p : graph_recs_dev) cudaFree(p);
   if (d_shots) cudaFree(d_shots);
   if (d_items) cudaFree(d_items);
   if (d_sync) cudaFree(d_sync);

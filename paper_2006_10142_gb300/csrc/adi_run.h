@@ -137,6 +137,8 @@ struct adi_wave {
   volatile unsigned int* scan_host = nullptr;
   unsigned int* scan_host_dev = nullptr;
   int rec_cap = 0;
+  std::vector<std::vector<int32_t>> graph_recs;  // receiver lists of runs in callers' graphs ...
+  std::vector<int*> graph_recs_dev;              // ... and device lists outgrown since
   cudaStream_t cap = nullptr;  // private stream used only for graph capture
   cudaGraphExec_t pair[2][4] = {};  // [orientation][gather + 2 one_pass]
   adi_wave_tuning tuning = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};

@@ -80,3 +80,36 @@ def test_many_receivers_are_sampled_by_a_launch_of_their_own():
         count.append(h.launch_count() - before)
     assert count[1] - count[0] == steps - 1  # the last level has one either way
     h.close()
+
+
+def test_captured_run_keeps_its_receiver_list():
+    """The caller's list is gone when the graph is replayed, and the handle has
+    since sampled a longer one."""
+    import gc
+    import torch
+    from paper_2006_10142_gb300 import api
+    nx, ny, steps = 300, 260, 4
+    m, phi, tau, wav = _problem(nx, ny, 0.5, 3)
+    t = lambda a: torch.from_numpy(f32(a)).to("cuda:0")
+    phi = t(phi)
+    h = api.AdiWave(t(m), phi, tau)
+    rng = np.random.default_rng(1)
+    pick = lambda n: np.stack([rng.integers(0, nx, n), rng.integers(0, ny, n)], 1).astype(np.int32)
+    few, many = pick(50), pick(5000)
+    want = h.run(steps, rec=few)
+    h.reset(phi)
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        got = h.run(steps, rec=few.copy())
+    gc.collect()
+    junk = [np.full((50, 2), -7, dtype=np.int32) for _ in range(64)]
+    h.run(steps, rec=many)
+    for _ in range(2):
+        h.reset(phi)
+        got.zero_()
+        graph.replay()
+        assert torch.equal(got, want)
+    h.sync_status()
+    h.close()
+    del junk
