@@ -483,8 +483,11 @@ def run_single(ctx, prob):
     xname = {3: "x_pipe_kernel", 5: "x_band_kernel"}.get(tun.get("x_stage"), "x_sweep_kernel")
     yname = {3: "y_pipe_kernel", 4: "y_coop_kernel"}.get(tun.get("y_stage"), "y_sweep_kernel")
     if one_pass:
-        # bands from about 4 million points up, patches below
-        kinds, nbytes = {2: "tile_step_kernel" if pts > 4e6 else "patch_step_kernel"}, BYTES_STEP
+        form = h.plan()["form"]
+        kinds = {2: {"bands": "tile_step_kernel", "patches": "patch_step_kernel",
+                     "small_patches": "small_patch_kernel"}[form]}
+        nbytes = BYTES_STEP
+        tun = {"form": form, "use_graph": tun["use_graph"]}  # the sweeps' knobs play no part
         roof = _roofline(kms, kcnt, kinds, {2: nbytes * pts}, args.workload)
     else:
         nbytes = BYTES_X + BYTES_Y
@@ -629,7 +632,7 @@ def run_batch(ctx, steps=None):
     # algorithmic bytes per point) over the wall time
     peak, peak_kind = measured_peak_gbs()
     ach = BYTES_STEP * pts_all * ts * K / (max_ms / 1e3) / 1e9
-    roof = {"bound": "hbm", "kernel": "tile_batch_kernel (a step of every shot)",
+    roof = {"bound": "hbm", "kernel": "tile_batch_kernel or patch_batch_kernel (a step of every shot)",
             "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak,
             "peak_source": peak_kind, "traffic": None,
             "alg_bytes_per_step": BYTES_STEP * pts_all, "timed_region": "wall time of the timed region"}

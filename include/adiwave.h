@@ -94,8 +94,8 @@ typedef struct {
 } adi_source;
 
 /* Create a handle for n_shots independent grids (n_shots == 1: one grid;
- * n_shots > 1: the batched form that advances all grids together, one
- * persistent kernel launch per sweep and step).
+ * n_shots > 1: the batched form that advances all grids together, see
+ * adi_wave_set_batch_mode).
  *   desc[s]      grid of shot s (host array of n_shots).
  *   m[s]         device pointer, [ny][nx] FP32 coefficient m = c^2 > 0.
  *   phi[s]       device pointer, [ny][nx] FP32 initial value u(0).
@@ -331,8 +331,9 @@ int adi_wave_profile_read(adi_wave *h, double *ms, int64_t *launches,
  * allows) launched once per shot and step, one after the other;
  * mode 2 (default): the shots whose step is one launch (see adi_wave_tuning)
  * advance together, one launch per step for all of them; the other shots'
- * steps are chains of the plain kernels on eight streams that fork from and
- * join into the caller's stream.
+ * steps run beside them, chains of the plain kernels on eight streams that
+ * fork from the caller's stream and join it (replayed from a graph unless the
+ * caller is capturing).
  * ADI_EINVAL for other modes or single-grid handles. */
 int adi_wave_set_batch_mode(adi_wave *h, int32_t mode);
 

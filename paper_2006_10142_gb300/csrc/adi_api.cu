@@ -1,13 +1,13 @@
 // adi_api.cu -- the C ABI of libadiwave.so (declared in include/adiwave.h):
-// handle lifetime, validation, launch planning, the time loop with CUDA
-// graph replay, state access, measurement hooks.
+// handle lifetime, validation, launch planning, state access, measurement
+// hooks.
 //
 // Algorithm 1 (Section 3.1) keeps four buffers u, U0, Ux, Uy and swaps them
 // after every step.  Here a grid owns two state buffers -- buf[cur] = u^k,
 // buf[1-cur] = u^{k-1} -- plus one scratch field w; the y sweep writes
 // u^{k+1} over u^{k-1} and `cur` flips, which is the same rotation without
-// copies.  Two consecutive steps restore the orientation, so a captured
-// graph of one step pair is replayed for the whole loop.
+// copies.  Two consecutive steps restore the orientation, so that a captured
+// pair can be replayed for the whole loop.
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <stdio.h>

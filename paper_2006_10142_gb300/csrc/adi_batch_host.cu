@@ -1,7 +1,9 @@
-// adi_batch_host.cu -- host side of the batched form: per-shot geometry for
-// the persistent kernel (every item is one full CTA of K = 16 unknowns per
-// thread, so items of different shots carry the same work), the work list,
-// and one step.
+// adi_batch_host.cu -- host side of the batched form: the one-launch step
+// (tables of tensor maps and CTAs, form and band length) with the shots beside
+// it that need the sweeps; per-shot chains of the plain kernels; and for the
+// persistent kernel the per-shot geometry (every item is one full CTA of K = 16
+// unknowns per thread, so items of different shots carry the same work), the
+// work list, and one step.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -37,7 +37,10 @@ __device__ __forceinline__ float rcp_t(float x) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
-// 1/x for the eliminations' denominators (finite, 1 and above): the hardware's
+// 1/x for the eliminations' denominators (finite, 1 and above: pivots of
+// matrices whose off-diagonals are negative and whose rows sum to 1 or more,
+// which elimination preserves, b >= 1 + |a| + |c|; so also the determinants
+// b b' - c a' >= 1 + |c| + |a'| of merged segments): the hardware's
 // gross approximation and two Newton steps, r <- r + r (1 - x r), which square
 // its error twice, past the last place of a double.  FP64 runs at 1/64 of the
 // FP32 rate, so the four instructions count: a general division takes twice

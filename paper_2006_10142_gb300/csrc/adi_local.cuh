@@ -51,7 +51,8 @@ __device__ __forceinline__ ulonglong2 lds4(uint32_t a) {
 // (every term of p is positive, so nothing cancels): two dependent FMAs per
 // unknown, and the reciprocals of the p_k are independent of one another.  p
 // grows by at most 1 + 2s per unknown, 2^16 over a block at s = 1/2, the
-// largest s the halo of 16 allows; every block starts again from p = 1.
+// largest s the halo of 16 allows; every block starts again from p = 1.  N is
+// p times a solution value, so that fields may be as large as 2^111 (2.6e33).
 //
 // The packed instructions take no negated operands, so signs are carried by
 // the data instead, in a fixed pattern of period 4: s enters as (-1)^k s_k,

@@ -1,6 +1,6 @@
 // adi_run.cu -- handle implementation: creation, the time loop (Algorithm 1)
-// with CUDA-graph replay of step pairs, checkpoints, state access, status,
-// tuning and measurement hooks.
+// as chained launches or replayed step pairs, checkpoints, state access,
+// status, tuning and measurement hooks.
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <string.h>
@@ -210,9 +210,10 @@ int adi_wave::capture_batch_pair(cudaGraphExec_t* ex, bool rest) {
   return ADI_OK;
 }
 
-// Batched run: every shot advances `steps` steps; one persistent launch per
-// step (or the plain kernels per shot in batch mode 1), step pairs replayed
-// from a captured graph.
+// Batched run: every shot advances `steps` steps, by the form of the batch
+// mode (one launch per step for all shots where their plans allow it, the
+// persistent kernel, or the plain kernels per shot); step pairs of the latter
+// two are replayed from a captured graph.
 int adi_wave::run_batch(int steps, const adi_source* src, cudaStream_t st) {
   for (size_t s = 0; s < g.size(); ++s) {
     Grid& G = g[s];

@@ -21,21 +21,24 @@
 // A CTA owns a strip of TX = 224 columns and a band of rows.  It stages 256
 // columns (16 of halo on either side) and marches down the band in blocks of
 // 16 rows:
-//   x phase: 16 rows x 16 chunks of 16 unknowns, one chunk per thread (lanes
-//     along the rows, so that the 128-byte-swizzled stage is read without
-//     bank conflicts).  Each thread eliminates the last H unknowns of its
-//     chunk from zero, hands (gamma, delta) to the next chunk through shared
-//     memory, eliminates its chunk from the exact state it was handed,
-//     back-substitutes the first H unknowns from zero, hands x_0 to the
-//     previous chunk and back-substitutes the chunk.
-//   y phase: one column per thread (7 warps, the strip's own columns): the
-//     elimination of a column runs on from block to block in registers;
+//   x phase: 16 rows x 16 chunks of 16 unknowns over 128 threads, a chunk of
+//     rows r and r + 8 per thread in packed arithmetic (lanes along the rows,
+//     so that the 128-byte-swizzled stage is read without bank conflicts).
+//     Each thread eliminates the last H unknowns of its chunk from zero, hands
+//     (gamma, delta) to the next chunk through shared memory, eliminates its
+//     chunk from the exact state it was handed, back-substitutes the first H
+//     unknowns from zero, hands x_0 to the previous chunk and back-substitutes
+//     the chunk.  The outermost column on either side lacks a neighbour for
+//     its RHS and is set to zero: it lies 16 from the strip's own columns, so
+//     that with H = 16 too no factor above lambda^16 is left out.
+//   y phase: two columns per thread (112 threads, the strip's own columns):
+//     the elimination of a column runs on from block to block in registers;
 //     after each block the back substitution starts from its last row and
-//     yields the 16 rows that lie H behind.  The update and the stores are
-//     coalesced along the row.
+//     yields the 16 rows that lie H behind.  Whole blocks leave by TMA, the
+//     rows of a band's edge one by one.
 // Blocks of u^k (three slots, shifted by one row so that a block carries its
-// lower neighbour row) and m (two) arrive by TMA two blocks ahead; u^{k-1} is
-// prefetched into L2 with them.  Rows and columns outside the grid arrive as
+// lower neighbour row) and m (two) arrive by TMA two blocks ahead, u^{k-1} one
+// block ahead from L2, into which it is prefetched with them.  Rows and columns outside the grid arrive as
 // zeros with s = 0, which is the Dirichlet ring.  Bands start H rows early
 // and end H rows late (the halo of the column solves), and their rows are
 // chosen so that halo and all fill whole blocks (3001 x 1501: 21 bands of 72
