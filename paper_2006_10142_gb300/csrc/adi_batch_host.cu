@@ -9,7 +9,6 @@
 #include <algorithm>
 #include <cmath>
 #include <functional>
-#include <queue>
 #include <string>
 #include <vector>
 
@@ -218,9 +217,11 @@ int adi_wave::ensure_batch_tiles() {
     const int own = std::min(rows, ny - q * rows);
     return (own + (q > 0 ? bt_h : 0) + (q + 1 < bands ? bt_h : 0) + 15) / 16;
   };
+  // no schedule ends before the longest CTA or an even share: lengths by that
+  // bound, until it rules out the rest
+  std::vector<std::pair<double, int>> bound;
   for (int b = 4; wide && b < std::min(2 * max_blocks, 128); ++b) {
     const int rows = 16 * b - 2 * bt_h;
-    // no schedule ends before the longest CTA or an even share
     long long total = 0;
     int longest = 0;
     for (int s : shots) {
@@ -228,26 +229,29 @@ int adi_wave::ensure_batch_tiles() {
       longest = std::max(longest, band_len(g[s].ny, rows, bands > 2 ? 1 : 0, bands));
       total += (long long)tile_strips(g[s].nx) * ((g[s].ny + 2 * (bands - 1) * bt_h + 15) / 16);
     }
-    if (3.5 + 3.05 * std::max((double)longest, total / slots) >= best) continue;
-    std::vector<int> lens;
+    bound.emplace_back(3.5 + 3.05 * std::max((double)longest, total / slots), b);
+  }
+  std::sort(bound.begin(), bound.end());
+  for (const auto& lb : bound) {
+    if (lb.first >= best) break;
+    const int b = lb.second, rows = 16 * b - 2 * bt_h;
+    std::vector<long long> count(b + 1, 0);  // CTAs by blocks
     for (int s : shots) {
       const int bands = (g[s].ny + rows - 1) / rows;
-      for (int q = 0; q < bands; ++q) lens.insert(lens.end(), tile_strips(g[s].nx), band_len(g[s].ny, rows, q, bands));
+      for (int q = 0; q < bands; ++q) count[band_len(g[s].ny, rows, q, bands)] += tile_strips(g[s].nx);
     }
-    std::sort(lens.begin(), lens.end(), std::greater<int>());
-    std::priority_queue<int, std::vector<int>, std::greater<int>> ends;
-    int last = 0;
-    for (size_t i = 0; i < lens.size(); ++i) {
-      int end = lens[i];
-      if (ends.size() >= (size_t)slots) {
-        end += ends.top();
-        ends.pop();
+    std::vector<int> ends(1, (int)slots);  // slots by the time they are free
+    size_t now = 0;                        // the first of them: it never goes back
+    for (int len = b; len > 0; --len)
+      for (long long i = 0; i < count[len]; ++i) {
+        while (ends[now] == 0) ++now;
+        if (ends.size() <= now + len) ends.resize(now + len + 1, 0);
+        ends[now] -= 1;
+        ends[now + len] += 1;
       }
-      ends.push(end);
-      last = std::max(last, end);
-    }
+    const int last = (int)ends.size() - 1;
     const double t = 3.5 + 3.05 * last;
-    if (t < best) {
+    if (t < best || (t == best && b < best_b)) {
       best = t;
       best_b = b;
     }
