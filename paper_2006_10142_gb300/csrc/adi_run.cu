@@ -250,7 +250,12 @@ int adi_wave::run_batch(int steps, const adi_source* src, cudaStream_t st) {
     if (rc != ADI_OK) return rc;
     if (bt_n > 0) return run_batch_tiles(steps, st);
   }
-  const bool use_graph = g[0].plan.graph && !profile;
+  bool use_graph = g[0].plan.graph && !profile;
+  // Sweeps shot after shot fill the GPU one by one: as launches they overlap a
+  // little better than in a graph (us per step at tau = 2h: fifteen shots of 64^2
+  // to 1500 x 200 180 and 190, four of 2048^2 153.6 and 155.3).
+  if (batch_mode == 1 && tuning.use_graph == 0)
+    for (const Grid& G : g) use_graph = use_graph && G.plan.tile != 0;
   int t = 0;
   if (use_graph) {
     while (steps - t >= 2) {
